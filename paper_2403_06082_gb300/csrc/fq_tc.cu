@@ -56,7 +56,8 @@ constexpr int kChunk = 16;                  // accumulator columns per TMEM load
 
 struct PhaseArgs {
   int R, K, M;
-  int RT, TT, KB, tiles;
+  int RT, TT, KB, tiles;     // row tiles (128 rows, or 256 on a CTA pair), token tiles, K blocks
+  int RT1;                   // 128-row tiles
   int KS, kbs, units;        // K splits per tile, K blocks per split, tiles * KS work units
   float* part;               // KS > 1: fp32 partial tiles [tile][split][BN][128]
   uint32_t* cnt;             // KS > 1: arrivals per tile (the last resets it to 0)
@@ -68,6 +69,7 @@ struct PhaseArgs {
   const __half* zero;
   const float* gamma;
   int32_t* status;
+  int clear_status;          // this launch starts a call: clear the status word
   // Rounding of the frame representation of the activations (Appendix F), else all null:
   float* out32;              // analysis: z in fp32 (the bf16 z is then the rounded one)
   uint32_t* amax;            // analysis: running max |z| as float bits; the core resets it
@@ -98,7 +100,7 @@ struct Layout {
   static constexpr int oRedSmall = oMisc + 16;                      // [4][kChunk] + 4 floats
   static constexpr int oZsum = oRedSmall + (4 * kChunk + 4) * 4;    // [2][BN] floats
   static constexpr int kBytes = oZsum + 2 * BN * 4 + 1024;          // + alignment slack
-  static_assert(BN == 128 || BN == 256, "prefill tile widths");
+  static_assert(BN == 128, "tile width of the one-SM kernel");
   static_assert(kBTileBytes % 1024 == 0, "B tiles must keep 1024-byte alignment");
   static_assert(kBytes <= 227 * 1024, "shared memory");
   static_assert(kStages >= 2 && (!kCodes || kStages % 4 == 0), "ring depth");
@@ -249,7 +251,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
         }
       }
       pdl_wait();   // the previous kernel is complete and its writes are visible
-      if (PHASE == kAnalysis && blockIdx.x == 0) *p.status = 0;   // new call: clear status
+      if (p.clear_status && blockIdx.x == 0) *p.status = 0;       // a new call
       // the rounding kernel before this one has read the maximum: ready for the next call
       if (PHASE == kCore && p.amax && blockIdx.x == 0) *p.amax = 0u;
       int stage = 0;
@@ -542,6 +544,478 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Batches of more than 128 tokens: 256 x 256 tiles on CTA pairs
+// ---------------------------------------------------------------------------------------------
+// A 128 x 256 tile on one SM is bound by its shared memory: each 128-cycle MMA step reads 12 KiB
+// of operands and the ring refills 12 KiB, 192 B per cycle against the 128 B an SM moves.  A pair of
+// SMs computing a 256 x 256 tile (tcgen05 cta_group::2) reads 4 KiB of A and its own half of B,
+// 4 KiB, per SM and step, and refills as much: 128 B per cycle, and for the code product less
+// (2-bit codes).  PLACEHOLDER_MEASURED
+//
+// Each CTA of the pair loads and decodes its own 128 rows of A and half of the tokens of B;
+// rank 0 issues the MMAs for both, so the barriers the MMAs wait on live in rank 0:
+//   full[s]    rank 0: one arrival (its producer, with both CTAs' bytes) and the copies of both
+//   aready[s]  rank 0: one arrival per CTA's decoder (code product)
+//   tempty[b]  rank 0: one arrival per epilogue warp of both CTAs
+// and the MMAs' completions are committed to both CTAs (empty[s], tfull[b]).  cfull[s] (code
+// blocks landed) stays local.  Ring stage s is decoded by decoder warp s.  Every producer
+// waits for the last use of each of its stages before it leaves, so no copy is in flight then.
+template <int PHASE>
+struct PairLayout {
+  static constexpr bool kCodes = PHASE == kCore;
+  static constexpr int kBN = 256;                       // tokens per tile
+  static constexpr int kBTile = kBN / 2 * kBK * 2;      // this CTA's half of them: 16 KiB
+  static constexpr int kStages = 6;
+  static constexpr int kEpiWarps = 8;                   // two per TMEM quarter
+  static constexpr int kEpiThreads = 32 * kEpiWarps;
+  static constexpr int kDecWarps = kCodes ? kStages : 0;
+  static constexpr int kThreads = 64 + kEpiThreads + 32 * kDecWarps;
+  static constexpr uint32_t kTmemCols = 512;            // two accumulators of 256 columns
+  static constexpr int oA = 0;
+  static constexpr int oB = oA + kStages * kATileBytes;
+  static constexpr int oCodes = oB + kStages * kBTile;
+  static constexpr int oBar = oCodes + (kCodes ? kStages * kCodeBytes : 0);
+  static constexpr int kNumBars = 4 * kStages + 4;
+  static constexpr int oMisc = oBar + kNumBars * 8;     // TMEM address, abort and last-split flags
+  static constexpr int oRed = oMisc + 16;               // analysis: [4][256] sums of z
+  static constexpr int oZsum = oRed + (PHASE == kAnalysis ? 4 * kBN * 4 : 0);   // core: [256]
+  static constexpr int kBytes = oZsum + (kCodes ? kBN * 4 : 0) + 1024;          // + alignment slack
+  static_assert(kBytes <= 227 * 1024, "shared memory");
+};
+
+// Decode 64 2-bit codes (4 words) into one 128-byte row of a swizzled K-major tile, like
+// decode_row, with fewer operations: a pair of codes at bits 2p (p = 0, 1, 2) of the half-words
+// is ORed into the mantissa of 128.0 where it stands, giving 128 + 4^p q, and one fused
+// multiply-add makes it q (every step exact); two shifts per word bring the other pairs there.
+__device__ __forceinline__ void decode_row_fma(const uint4 w4, uint8_t* tile, int r) {
+  const uint32_t wv[4] = {w4.x, w4.y, w4.z, w4.w};
+  const __nv_bfloat162 one[3] = {__floats2bfloat162_rn(1.f, 1.f),
+                                 __floats2bfloat162_rn(0.25f, 0.25f),
+                                 __floats2bfloat162_rn(0.0625f, 0.0625f)};
+  const __nv_bfloat162 bias[3] = {__floats2bfloat162_rn(-128.f, -128.f),
+                                  __floats2bfloat162_rn(-32.f, -32.f),
+                                  __floats2bfloat162_rn(-8.f, -8.f)};
+  uint8_t* row = tile + r * 128;
+#pragma unroll
+  for (int wi = 0; wi < 4; ++wi) {
+    uint32_t h[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      const uint32_t w = wv[wi] >> (6 * (p / 3));
+      const uint32_t bits = (w & (0x00030003u << (2 * (p % 3)))) | 0x43004300u;
+      const __nv_bfloat162 v =
+          __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&bits), one[p % 3], bias[p % 3]);
+      h[p] = *reinterpret_cast<const uint32_t*>(&v);
+    }
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int c = 2 * wi + half;
+      *reinterpret_cast<uint4*>(row + ((c ^ (r & 7)) << 4)) =
+          make_uint4(h[4 * half], h[4 * half + 1], h[4 * half + 2], h[4 * half + 3]);
+    }
+  }
+}
+
+// Sums over a warp's 32 lanes of 16 values per lane: returned to lane l for value l >> 1 (both
+// lanes of a pair hold it).  Each step adds the lane 16, 8, 4, 2, 1 away and halves the values
+// a lane carries, so the additions are those of a full butterfly in 16 instead of 80 shuffles.
+__device__ __forceinline__ float warp_sums16(const float (&v)[kChunk], int lane) {
+  float a[8], b[4], c[2];
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float send = h16 ? v[i] : v[i + 8], keep = h16 ? v[i + 8] : v[i];
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float send = h8 ? a[i] : a[i + 4], keep = h8 ? a[i + 4] : a[i];
+    b[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float send = h4 ? b[i] : b[i + 2], keep = h4 ? b[i + 2] : b[i];
+    c[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  }
+  const float send = h2 ? c[0] : c[1], keep = h2 ? c[1] : c[0];
+  const float d = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+template <int PHASE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::kThreads, 1)
+    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA,
+                   const __grid_constant__ CUtensorMap tmB, const PhaseArgs p) {
+  using Lo = PairLayout<PHASE>;
+  constexpr int S_ = Lo::kStages;
+  constexpr bool kCodes = Lo::kCodes;
+  constexpr int BN = Lo::kBN;
+  constexpr uint32_t kFullBytes = 2 * ((kCodes ? 0 : kATileBytes) + Lo::kBTile);
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* sA = smem + Lo::oA;
+  uint8_t* sB = smem + Lo::oB;
+  uint8_t* sCodes = smem + Lo::oCodes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Lo::oBar);
+  uint64_t* empty = full + S_;
+  uint64_t* aready = empty + S_;
+  uint64_t* cfull = aready + S_;
+  uint64_t* tfull = cfull + S_;
+  uint64_t* tempty = tfull + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Lo::oMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
+  float* red = reinterpret_cast<float*>(smem + Lo::oRed);
+  float* zsum_s = reinterpret_cast<float*>(smem + Lo::oZsum);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = static_cast<int>(blockIdx.x >> 1), npairs = static_cast<int>(gridDim.x >> 1);
+  // work unit u = split * tiles + tile: K blocks [split * kbs, min(KB, (split + 1) * kbs))
+  auto unit_tile = [&](int u) { return u % p.tiles; };
+  auto unit_k0 = [&](int u) { return (u / p.tiles) * p.kbs; };
+  auto unit_k1 = [&](int u) { return min(p.KB, (u / p.tiles + 1) * p.kbs); };
+  // this CTA's 128-row tile of pair row tile rt; past the last one its operand rows are zeros
+  // (tensor map) or the last tile's codes, and its results are dropped
+  auto row_tile = [&](int rt) { return 2 * rt + static_cast<int>(rank); };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S_; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+      mbar_init(&aready[s], 2);
+      mbar_init(&cfull[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&tfull[b], 1);
+      mbar_init(&tempty[b], 2 * Lo::kEpiWarps);
+    }
+    *abort_flag = 0;
+    fence_barrier_init();
+    if (!kCodes) prefetch_tmap(&tmA);
+    prefetch_tmap(&tmB);
+  }
+  if (warp == 1) tmem_alloc_pair(tmem_slot, Lo::kTmemCols);
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_sync();       // both CTAs' barriers and TMEM exist before either signals the other
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_launch_dependents();
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- TMA producer
+    if (lane == 0) {
+      const uint64_t pol_w = policy_evict_first();
+      const uint64_t pol_x = policy_evict_last();
+      const bool leader = rank == 0;
+      auto load_a = [&](int stage, int rt, int kb) {
+        const int rt1 = row_tile(rt);
+        if (kCodes) {
+          mbar_arrive_expect_tx(&cfull[stage], kCodeBytes);
+          bulk_load(sCodes + stage * kCodeBytes,
+                    p.words + (static_cast<int64_t>(min(rt1, p.RT1 - 1)) * p.KB + kb) * 512,
+                    kCodeBytes, &cfull[stage], pol_w);
+        } else {
+          if (leader) mbar_arrive_expect_tx(&full[stage], kFullBytes);
+          tma_load_2d_pair(sA + stage * kATileBytes, &tmA, mapa(smem_u32(&full[stage]), 0),
+                           kb * kBK, rt1 * kBM, pol_w);
+        }
+      };
+      // weight tiles of the first unit do not depend on the previous kernel: a ring of them is
+      // requested, and the rest warmed in L2, before waiting for it
+      int pre = 0;
+      if (pair < p.units) {
+        const int rt = unit_tile(pair) / p.TT, rt1 = min(row_tile(rt), p.RT1 - 1);
+        const int k0 = unit_k0(pair), k1 = unit_k1(pair);
+        pre = min(S_, k1 - k0);
+        for (int i = 0; i < pre; ++i) load_a(i, rt, k0 + i);
+        for (int kb = k0 + pre; kb < k1; ++kb) {
+          if (kCodes)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                             p.words + (static_cast<int64_t>(rt1) * p.KB + kb) * 512),
+                         "r"(kCodeBytes)
+                         : "memory");
+          else
+            asm volatile(
+                "cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                    reinterpret_cast<uint64_t>(&tmA)),
+                "r"(kb * kBK), "r"(rt1 * kBM)
+                : "memory");
+        }
+      }
+      pdl_wait();   // the previous kernel is complete and its writes are visible
+      if (p.clear_status && blockIdx.x == 0) *p.status = 0;       // a new call
+      // the rounding kernel before this one has read the maximum: ready for the next call
+      if (PHASE == kCore && p.amax && blockIdx.x == 0) *p.amax = 0u;
+      int stage = 0, it = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int unit = pair; unit < p.units && ok && !*abort_flag; unit += npairs) {
+        const int tile = unit_tile(unit), k0 = unit_k0(unit), k1 = unit_k1(unit);
+        const int rt = tile / p.TT, tt = tile % p.TT;
+        for (int kb = k0; kb < k1; ++kb, ++it) {
+          if (it >= pre) {
+            if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) {
+              ok = false;
+              break;
+            }
+            load_a(stage, rt, kb);
+          }
+          if (kCodes && leader) mbar_arrive_expect_tx(&full[stage], kFullBytes);
+          tma_load_2d_pair(sB + stage * Lo::kBTile, &tmB, mapa(smem_u32(&full[stage]), 0),
+                           kb * kBK, tt * BN + static_cast<int>(rank) * (BN / 2), pol_x);
+          if (++stage == S_) stage = 0, phase ^= 1;
+        }
+      }
+      if (!ok) {
+        report(p.status, FQ_ERR_TIMEOUT);
+        *abort_flag = 1;
+      }
+      // The MMAs of each stage's last round are complete (so its copies have landed, and every
+      // commit that signals it was made): the waits of one more round of the ring.
+      const int rounds = min(it, S_);
+      if (it < S_) stage = 0, phase = 1;     // the first ring: stages 0 .. it - 1, phase 0
+      for (int r = 0; r < rounds; ++r) {
+        if (!mbar_wait(&empty[stage], phase ^ 1, nullptr)) {
+          report(p.status, FQ_ERR_TIMEOUT);
+          break;
+        }
+        if (++stage == S_) stage = 0, phase ^= 1;
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer (rank 0)
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = umma_idesc_bf16(2 * kBM, BN);
+      int stage = 0, buf = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
+      for (int unit = pair; unit < p.units && ok && !*abort_flag; unit += npairs) {
+        const int k0 = unit_k0(unit), k1 = unit_k1(unit);
+        ok = mbar_wait_cluster(&tempty[buf], acc_phase ^ 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * BN);
+        for (int kb = k0; kb < k1; ++kb) {
+          ok = mbar_wait_cluster(&full[stage], phase, abort_flag) &&
+               (!kCodes || mbar_wait_cluster(&aready[stage], phase, abort_flag));
+          if (!ok) break;
+          tc_fence_after_sync();
+          const uint64_t adesc = umma_desc_sw128(smem_u32(sA + stage * kATileBytes));
+          const uint64_t bdesc = umma_desc_sw128(smem_u32(sB + stage * Lo::kBTile));
+#pragma unroll
+          for (int k = 0; k < kBK / 16; ++k)
+            umma_bf16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc,
+                           (kb > k0 || k > 0) ? 1u : 0u);
+          umma_commit_pair(&empty[stage]);
+          if (++stage == S_) stage = 0, phase ^= 1;
+        }
+        if (!ok) break;
+        umma_commit_pair(&tfull[buf]);
+        if (++buf == 2) buf = 0, acc_phase ^= 1;
+      }
+      if (!ok) {
+        report(p.status, FQ_ERR_TIMEOUT);
+        *abort_flag = 1;
+      }
+    }
+  } else if (warp < 2 + Lo::kEpiWarps) {
+    // ---------------------------------------------------------------- epilogue (rows)
+    constexpr int kN = Lo::kEpiThreads;
+    const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
+    const int half = (warp - 2) >> 2;             // columns 128 * half .. + 127
+    const int r_in_tile = quarter * 32 + lane;
+    const int et = threadIdx.x - 64;
+    pdl_wait();
+    int buf = 0;
+    uint32_t acc_phase = 0;
+    for (int unit = pair; unit < p.units; unit += npairs) {
+      const int tile = unit_tile(unit), split = unit / p.tiles;
+      const int rt = tile / p.TT, tt = tile % p.TT;
+      const int rt1 = row_tile(rt);
+      const int row = rt1 * kBM + r_in_tile;
+      const int t0 = tt * BN;
+      const bool row_ok = row < p.R;
+      float s_i = 0.f, z_i = 0.f;
+      if (PHASE == kCore && row_ok) {
+        s_i = __half2float(p.scale[row]);
+        z_i = __half2float(p.zero[row]);
+      }
+      if (PHASE == kCore) {
+        // sum_j z[t][j] of the tile's tokens (one per thread), from the analysis' per-tile sums
+        const int t = t0 + et;
+        float s = 0.f;
+        if (t < p.M)
+#pragma unroll 8
+          for (int g = 0; g < p.zsum_tiles; ++g)
+            s += ldcg_f32(p.zsum_part + static_cast<int64_t>(g) * p.M + t);
+        named_barrier_sync(1, kN);                // the previous unit's sums have been read
+        zsum_s[et] = s;
+      }
+      const bool fail = !mbar_wait(&tfull[buf], acc_phase, abort_flag);
+      if (fail) report(p.status, FQ_ERR_TIMEOUT);
+      if (bar_red_or(1, kN, fail || *abort_flag)) {
+        if (et == 0) *abort_flag = 1;
+        break;
+      }
+      tc_fence_after_sync();
+      const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
+                             static_cast<uint32_t>(buf * BN);
+      const float g_i = (PHASE == kCore && row_ok && p.gamma) ? p.gamma[row] : 1.f;
+      // with rounded activations the accumulator is the exact integer sum_j q_ij zbar_j, and
+      // u = Delta gamma (s acc + zero sum_j zbar_j)
+      const float dl = (PHASE == kCore && p.delta) ? ldcg_f32(p.delta) : 1.f;
+      float amax_t = 0.f;
+      // the finished values of columns c .. c + 15 of this thread's row
+      auto emit = [&](int c, float (&v)[kChunk]) {
+        if (PHASE == kAnalysis && p.out32) {
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q) {
+            const int t = t0 + c + q;
+            if (row_ok && t < p.M) {
+              p.out32[static_cast<int64_t>(t) * p.R + row] = v[q];
+              amax_t = fmaxf(amax_t, fabsf(v[q]));
+            }
+          }
+          return;
+        }
+#pragma unroll
+        for (int q = 0; q < kChunk; ++q) {
+          if (PHASE == kCore) v[q] = g_i * fmaf(s_i, v[q], z_i * zsum_s[c + q]) * dl;
+          const __nv_bfloat16 b = __float2bfloat16_rn(v[q]);
+          v[q] = row_ok ? __bfloat162float(b) : 0.f;
+          const int t = t0 + c + q;
+          if (row_ok && t < p.M) p.out[static_cast<int64_t>(t) * p.R + row] = b;
+        }
+        if (PHASE == kAnalysis) {
+          // per-token sum over the warp's 32 rows of the bf16 z actually stored
+          const float s = warp_sums16(v, lane);
+          if ((lane & 1) == 0) red[quarter * BN + c + (lane >> 1)] = s;
+        }
+      };
+      bool finish = true;
+      if (p.KS == 1) {
+#pragma unroll 1
+        for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+          float v[kChunk];
+          tmem_ld16(t_row + c, v);
+          tmem_wait_ld();
+          emit(c, v);
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[buf]), 0));
+      } else {
+        // Split K: this CTA's partial tile to the workspace (column-major, so a warp's 32 rows
+        // are one 128-byte line), the accumulator released, the split counted in.  The last
+        // split of the CTA's 128-row tile to arrive adds the partials in split order.
+        const int64_t t1 = static_cast<int64_t>(rt1) * p.TT + tt;
+        const bool mine_ok = rt1 < p.RT1;
+        float* mine = p.part + (t1 * p.KS + split) * BN * kBM;
+#pragma unroll 1
+        for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+          float v[kChunk];
+          tmem_ld16(t_row + c, v);
+          tmem_wait_ld();
+          if (mine_ok) {
+#pragma unroll
+            for (int q = 0; q < kChunk; ++q) mine[(c + q) * kBM + r_in_tile] = v[q];
+          }
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[buf]), 0));
+        __threadfence();
+        named_barrier_sync(1, kN);
+        if (et == 0) {
+          bool last = false;
+          if (mine_ok) {
+            last = atomicAdd(&p.cnt[t1], 1u) == static_cast<uint32_t>(p.KS - 1);
+            if (last) p.cnt[t1] = 0;                 // ready for the next call
+            __threadfence();
+          }
+          *last_flag = last ? 1 : 0;
+        }
+        named_barrier_sync(1, kN);
+        finish = *last_flag != 0;
+        if (finish) {
+          const float* all = p.part + t1 * p.KS * BN * kBM;
+#pragma unroll 1
+          for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+            float v[kChunk];
+#pragma unroll
+            for (int q = 0; q < kChunk; ++q) v[q] = 0.f;
+            for (int sp = 0; sp < p.KS; ++sp) {
+#pragma unroll
+              for (int q = 0; q < kChunk; ++q)
+                v[q] += ldcg_f32(all + (static_cast<int64_t>(sp) * BN + c + q) * kBM + r_in_tile);
+            }
+            emit(c, v);
+          }
+        }
+        named_barrier_sync(1, kN);                   // the flag is read before it is reused
+      }
+      if (PHASE == kAnalysis && !p.out32 && finish) {
+        // the tile's sum of z per token, quarters added in a fixed order
+        named_barrier_sync(1, kN);
+        if (rt1 < p.RT1 && t0 + et < p.M)
+          p.zsum_part[static_cast<int64_t>(rt1) * p.M + t0 + et] =
+              (red[et] + red[BN + et]) + (red[2 * BN + et] + red[3 * BN + et]);
+        named_barrier_sync(1, kN);                   // read before the next unit's sums
+      }
+      if (PHASE == kAnalysis && p.out32) {
+        // one atomic per warp and tile: the tensor's max |z| (non-negative floats order like
+        // their bit patterns)
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+          amax_t = fmaxf(amax_t, __shfl_xor_sync(0xffffffffu, amax_t, off));
+        if (lane == 0 && amax_t > 0.f) atomicMax(p.amax, __float_as_uint(amax_t));
+      }
+      if (++buf == 2) buf = 0, acc_phase ^= 1;
+    }
+  } else {
+    // ---------------------------------------------------------------- code decoders (core)
+    if (kCodes) {
+      // decoder d expands every code block of ring stage d, four rows per lane
+      const int d = warp - 2 - Lo::kEpiWarps;
+      const uint32_t ready_bar = mapa(smem_u32(&aready[d]), 0);
+      const uint4* codes = reinterpret_cast<const uint4*>(sCodes + d * kCodeBytes);
+      uint8_t* tile_a = sA + d * kATileBytes;
+      int total = 0;                              // this pair's K blocks over all its units
+      for (int unit = pair; unit < p.units; unit += npairs) total += unit_k1(unit) - unit_k0(unit);
+      uint32_t phase = 0;
+      for (int it = d; it < total; it += S_, phase ^= 1) {
+        const bool got = mbar_wait(&cfull[d], phase, abort_flag);
+        if (!__all_sync(0xffffffffu, got)) {
+          if (lane == 0) {
+            report(p.status, FQ_ERR_TIMEOUT);
+            *abort_flag = 1;
+          }
+          break;
+        }
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr)
+          decode_row_fma(codes[lane + 32 * rr], tile_a, lane + 32 * rr);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(ready_bar);
+      }
+    }
+  }
+
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_sync();          // no CTA leaves while the other may still signal it or use its TMEM
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc_pair(tmem_base, Lo::kTmemCols);
+  }
+}
+
 // Rounding of the frame representation of the activations (Appendix F): with the tensor's
 // step Delta = max |z| / L, L = 2^(N-1) - 1, zq = nearest integer to z / Delta (ties to even,
 // clamped to [-L, L]) as bf16 (exact: |zq| <= 127 needs 7 significant bits), and the per-token
@@ -639,13 +1113,13 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-// bf16 matrix rows x cols (row-major), boxes of 64 columns x box_rows rows, 128-byte swizzle.
-bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int box_rows) {
+// bf16 matrix rows x cols (row-major), boxes of 64 columns x 128 rows, 128-byte swizzle.
+bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols) {
   auto enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(box_rows)};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(kBM)};
   cuuint32_t estr[2] = {1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -653,6 +1127,7 @@ bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tokens per tile: one-SM tiles of 128 x 128 up to 128 tokens, CTA pairs with 256 x 256 above.
 int pick_bn(int M) { return M <= 128 ? 128 : 256; }
 
 struct DeviceInfo {
@@ -697,7 +1172,7 @@ int split_for(int tiles, int KB, int sms) {
 
 template <int PHASE, int BN>
 void plan_phase(PhaseArgs& a, const DeviceInfo& d, int& grid) {
-  a.RT = static_cast<int>(ceil_div(a.R, kBM));
+  a.RT1 = a.RT = static_cast<int>(ceil_div(a.R, kBM));
   a.TT = static_cast<int>(ceil_div(a.M, BN));
   a.KB = static_cast<int>(ceil_div(a.K, kBK));
   a.tiles = a.RT * a.TT;
@@ -706,6 +1181,23 @@ void plan_phase(PhaseArgs& a, const DeviceInfo& d, int& grid) {
   a.KS = static_cast<int>(ceil_div(a.KB, a.kbs));     // every split non-empty
   a.units = a.tiles * a.KS;
   grid = std::min(a.units, d.sms);
+}
+
+// The same on CTA pairs: units of 256 x 256 tiles (or K splits of them), one pair per unit and
+// round.  A split's partial tiles are kept per 128-row tile, in the workspace planned for those.
+template <int PHASE>
+void plan_pairs(PhaseArgs& a, int pairs, int& grid) {
+  constexpr int BN = PairLayout<PHASE>::kBN;
+  a.RT1 = static_cast<int>(ceil_div(a.R, kBM));
+  a.RT = static_cast<int>(ceil_div(a.R, 2 * kBM));
+  a.TT = static_cast<int>(ceil_div(a.M, BN));
+  a.KB = static_cast<int>(ceil_div(a.K, kBK));
+  a.tiles = a.RT * a.TT;
+  a.KS = split_for(a.tiles, a.KB, std::min(pairs, kMaxSplitSms / 2));
+  a.kbs = static_cast<int>(ceil_div(a.KB, a.KS));
+  a.KS = static_cast<int>(ceil_div(a.KB, a.kbs));
+  a.units = a.tiles * a.KS;
+  grid = 2 * std::min(a.units, pairs);
 }
 
 struct WsLayout {
@@ -745,20 +1237,67 @@ WsLayout ws_layout(int M, int d_in, int n_in, int n_out, int d_out, int act_bits
   return L;
 }
 
-template <int PHASE, int BN>
-cudaError_t launch_phase(const CUtensorMap& tmA, const CUtensorMap& tmB, const PhaseArgs& a,
-                         int grid, cudaStream_t s) {
+// CTA pairs of this kernel that fit the device at once (0 on an error); sets the kernel's shared
+// memory attribute on the device's first call.
+template <int PHASE>
+int resident_pairs(int dev) {
+  static std::mutex mu;
+  static std::map<int, int> cache;
+  std::lock_guard<std::mutex> g(mu);
+  const auto it = cache.find(dev);
+  if (it != cache.end()) return it->second;
+  using Lo = PairLayout<PHASE>;
+  if (cudaFuncSetAttribute(tc_pair_kernel<PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           Lo::kBytes) != cudaSuccess)
+    return 0;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(grid));
-  cfg.blockDim = dim3(threads_for<PHASE>());
-  cfg.dynamicSmemBytes = Layout<PHASE, BN>::kBytes;
+  cfg.gridDim = dim3(2);
+  cfg.blockDim = dim3(Lo::kThreads);
+  cfg.dynamicSmemBytes = Lo::kBytes;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<PHASE>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cache[dev] = n;
+  return n;
+}
+
+// One phase: plan and launch it on CTA pairs (more than 128 tokens and at least two SMs) or on
+// single SMs, chained to the previous kernel with programmatic dependent launch.
+template <int PHASE>
+cudaError_t run_phase(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs& a,
+                      const DeviceInfo& d, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc_phase_kernel<PHASE, BN>, tmA, tmB, a);
+  int grid = 0;
+  if (a.M > 128 && d.sms >= 2) {
+    const int pairs = std::min(resident_pairs<PHASE>(d.dev), d.sms / 2);
+    if (pairs < 1) return cudaErrorLaunchOutOfResources;
+    plan_pairs<PHASE>(a, pairs, grid);
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(PairLayout<PHASE>::kThreads);
+    cfg.dynamicSmemBytes = PairLayout<PHASE>::kBytes;
+    return cudaLaunchKernelEx(&cfg, tc_pair_kernel<PHASE>, tmA, tmB, a);
+  }
+  if (const cudaError_t e = prepare_kernel<PHASE, 128>(d.dev)) return e;
+  plan_phase<PHASE, 128>(a, d, grid);
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(threads_for<PHASE>());
+  cfg.dynamicSmemBytes = Layout<PHASE, 128>::kBytes;
+  return cudaLaunchKernelEx(&cfg, tc_phase_kernel<PHASE, 128>, tmA, tmB, a);
 }
 
 // maps: {T_in, x, z, T_out^T, u}.  The core phase's A operand is the packed codes, so it gets
@@ -779,34 +1318,24 @@ cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const Devi
                             n_in, L, static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
 }
 
-template <int BN>
 fq_status run_forward(const CUtensorMap* maps, PhaseArgs* a, int max_sms, int act_bits,
                       float* delta, cudaStream_t s) {
   DeviceInfo d = device_info();
   if (max_sms > 0) d.sms = std::min(d.sms, max_sms);
-  if (prepare_kernel<kAnalysis, BN>(d.dev) != cudaSuccess ||
-      prepare_kernel<kCore, BN>(d.dev) != cudaSuccess ||
-      prepare_kernel<kSynthesis, BN>(d.dev) != cudaSuccess)
-    return FQ_ERR_CUDA;
-  int g[3];
-  plan_phase<kAnalysis, BN>(a[0], d, g[0]);
-  plan_phase<kCore, BN>(a[1], d, g[1]);
-  plan_phase<kSynthesis, BN>(a[2], d, g[2]);
-  a[1].zsum_tiles = act_bits > 0 ? 1 : a[0].RT;      // rounded: one exact sum per token
-  if (launch_phase<kAnalysis, BN>(maps[0], maps[1], a[0], g[0], s) != cudaSuccess)
-    return FQ_ERR_CUDA;
+  a[1].zsum_tiles =
+      act_bits > 0 ? 1 : static_cast<int>(ceil_div(a[0].R, kBM));   // rounded: one exact sum
+  if (run_phase<kAnalysis>(maps[0], maps[1], a[0], d, s) != cudaSuccess) return FQ_ERR_CUDA;
   if (act_bits > 0 && launch_round(a[0], a[1].K, act_bits, d, delta, a[0].out, a[0].zsum_part,
                                    s) != cudaSuccess)
     return FQ_ERR_CUDA;
-  if (launch_phase<kCore, BN>(maps[1], maps[2], a[1], g[1], s) != cudaSuccess ||
-      launch_phase<kSynthesis, BN>(maps[3], maps[4], a[2], g[2], s) != cudaSuccess)
+  if (run_phase<kCore>(maps[1], maps[2], a[1], d, s) != cudaSuccess ||
+      run_phase<kSynthesis>(maps[3], maps[4], a[2], d, s) != cudaSuccess)
     return FQ_ERR_CUDA;
   return FQ_OK;
 }
 
-// The dense product of the weight-reconstruction path: one analysis-phase kernel with the
-// reconstructed weight as its A operand (the per-tile sums of the output it also writes go to
-// the workspace and are not used).
+// The dense product of the weight-reconstruction path: one synthesis-phase kernel with the
+// reconstructed weight as its A operand.
 WsLayout dense_ws_layout(int M, int d_out) {
   WsLayout L{};
   size_t off = kWsHeader;
@@ -827,33 +1356,22 @@ WsLayout dense_ws_layout(int M, int d_out) {
   return L;
 }
 
-template <int BN>
-fq_status run_dense(const CUtensorMap& tmW, const CUtensorMap& tmX, PhaseArgs& a,
-                    cudaStream_t s) {
-  const DeviceInfo d = device_info();
-  if (prepare_kernel<kAnalysis, BN>(d.dev) != cudaSuccess) return FQ_ERR_CUDA;
-  int grid = 0;
-  plan_phase<kAnalysis, BN>(a, d, grid);
-  return launch_phase<kAnalysis, BN>(tmW, tmX, a, grid, s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
-}
-
 fq_status launch_tc_dense(const void* x, int M, int d_in, const void* W, int d_out, void* y,
                           char* ws, size_t ws_bytes, cudaStream_t s) {
   const WsLayout L = dense_ws_layout(M, d_out);
   if (ws_bytes < L.total) return FQ_ERR_WORKSPACE;
-  const int BN = pick_bn(M);
   PhaseArgs a{};
   a.R = d_out;
   a.K = d_in;
   a.M = M;
   a.out = reinterpret_cast<__nv_bfloat16*>(y);
-  a.zsum_part = reinterpret_cast<float*>(ws + L.zsum);
+  a.clear_status = 1;
   a.status = reinterpret_cast<int32_t*>(ws);
   a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
   a.part = reinterpret_cast<float*>(ws + L.part);
   CUtensorMap mW, mX;
-  if (!make_tmap(&mW, W, d_out, d_in, kBM) || !make_tmap(&mX, x, M, d_in, BN)) return FQ_ERR_CUDA;
-  return BN == 128 ? run_dense<128>(mW, mX, a, s) : run_dense<256>(mW, mX, a, s);
+  if (!make_tmap(&mW, W, d_out, d_in) || !make_tmap(&mX, x, M, d_in)) return FQ_ERR_CUDA;
+  return run_phase<kSynthesis>(mW, mX, a, device_info(), s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -871,7 +1389,6 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
   const int n_in = Cq.n_in, n_out = Cq.n_out;
   const WsLayout L = ws_layout(M, d_in, n_in, n_out, d_out, act_bits);
   if (ws_bytes < L.total) return FQ_ERR_WORKSPACE;
-  const int BN = pick_bn(M);
   auto* status = reinterpret_cast<int32_t*>(ws);
   auto* z = reinterpret_cast<__nv_bfloat16*>(ws + L.z);
   auto* u = reinterpret_cast<__nv_bfloat16*>(ws + L.u);
@@ -892,6 +1409,7 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
     a[ph].cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
     a[ph].part = reinterpret_cast<float*>(ws + L.part);
   }
+  a[0].clear_status = 1;
   a[1].words = Cq.words;
   a[1].scale = reinterpret_cast<const __half*>(Cq.scale_f16);
   a[1].zero = reinterpret_cast<const __half*>(Cq.zero_f16);
@@ -905,36 +1423,14 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
     a[1].delta = delta;
   }
 
-  // maps: T_in, x, z, T_out^T, u  (A maps use 128-row boxes, B maps BN-row boxes)
+  // maps: T_in, x, z, T_out^T, u
   CUtensorMap maps[5];
-  if (!make_tmap(&maps[0], T_in, n_in, d_in, kBM) || !make_tmap(&maps[1], x, M, d_in, BN) ||
-      !make_tmap(&maps[2], z, M, n_in, BN) || !make_tmap(&maps[3], T_out_t, d_out, n_out, kBM) ||
-      !make_tmap(&maps[4], u, M, n_out, BN))
+  if (!make_tmap(&maps[0], T_in, n_in, d_in) || !make_tmap(&maps[1], x, M, d_in) ||
+      !make_tmap(&maps[2], z, M, n_in) || !make_tmap(&maps[3], T_out_t, d_out, n_out) ||
+      !make_tmap(&maps[4], u, M, n_out))
     return FQ_ERR_CUDA;
-
-  return BN == 128 ? run_forward<128>(maps, a, max_sms, act_bits, delta, s)
-                   : run_forward<256>(maps, a, max_sms, act_bits, delta, s);
+  return run_forward(maps, a, max_sms, act_bits, delta, s);
 }
-
-namespace {
-// The code product and the synthesis of the tensor-core chain, after z and one sum of z per
-// token have been written to the workspace (a[1].zsum_tiles = 1).
-template <int BN>
-fq_status run_core_synthesis(const CUtensorMap* maps, PhaseArgs* a, cudaStream_t s) {
-  const DeviceInfo d = device_info();
-  if (prepare_kernel<kCore, BN>(d.dev) != cudaSuccess ||
-      prepare_kernel<kSynthesis, BN>(d.dev) != cudaSuccess)
-    return FQ_ERR_CUDA;
-  int g[2];
-  plan_phase<kCore, BN>(a[1], d, g[0]);
-  plan_phase<kSynthesis, BN>(a[2], d, g[1]);
-  a[1].zsum_tiles = 1;
-  if (launch_phase<kCore, BN>(maps[0], maps[0], a[1], g[0], s) != cudaSuccess ||
-      launch_phase<kSynthesis, BN>(maps[1], maps[2], a[2], g[1], s) != cudaSuccess)
-    return FQ_ERR_CUDA;
-  return FQ_OK;
-}
-}  // namespace
 
 fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq,
                                  const void* T_out_t, int d_out, const float* gamma, void* y,
@@ -942,7 +1438,6 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
   const int M = d_in, n_in = Cq.n_in, n_out = Cq.n_out;
   const WsLayout L = ws_layout(M, d_in, n_in, n_out, d_out, 0);
   if (ws_bytes < L.total) return FQ_ERR_WORKSPACE;
-  const int BN = pick_bn(M);
   auto* status = reinterpret_cast<int32_t*>(ws);
   auto* z = reinterpret_cast<__nv_bfloat16*>(ws + L.z);
   auto* u = reinterpret_cast<__nv_bfloat16*>(ws + L.u);
@@ -971,8 +1466,8 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
 
   // maps: z (the code product's B; also the unused A slot), T_out^T, u
   CUtensorMap maps[3];
-  if (!make_tmap(&maps[0], z, M, n_in, BN) || !make_tmap(&maps[1], T_out_t, d_out, n_out, kBM) ||
-      !make_tmap(&maps[2], u, M, n_out, BN))
+  if (!make_tmap(&maps[0], z, M, n_in) || !make_tmap(&maps[1], T_out_t, d_out, n_out) ||
+      !make_tmap(&maps[2], u, M, n_out))
     return FQ_ERR_CUDA;
 
   unit_analysis_kernel<<<dim3(static_cast<unsigned>(ceil_div(d_in, 32)),
@@ -982,7 +1477,13 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
   unit_zsum_kernel<<<static_cast<unsigned>(ceil_div(d_in, 32)), dim3(32, 32), 0, s>>>(
       Tin, n_in, d_in, zsum, status);
   if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
-  return BN == 128 ? run_core_synthesis<128>(maps, a, s) : run_core_synthesis<256>(maps, a, s);
+  // the code product and the synthesis, with one sum of z per token
+  const DeviceInfo d = device_info();
+  a[1].zsum_tiles = 1;
+  return run_phase<kCore>(maps[0], maps[0], a[1], d, s) == cudaSuccess &&
+                 run_phase<kSynthesis>(maps[1], maps[2], a[2], d, s) == cudaSuccess
+             ? FQ_OK
+             : FQ_ERR_CUDA;
 }
 
 }  // namespace fq
