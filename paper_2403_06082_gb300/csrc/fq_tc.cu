@@ -137,6 +137,15 @@ __device__ __forceinline__ void decode_row(const uint4 w4, uint8_t* tile, int r)
   }
 }
 
+// 16 bytes of global memory that no kernel of the chain writes, not kept in L1.
+__device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
   uint32_t out;
   asm volatile(
@@ -555,32 +564,44 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
 //
 // Each CTA of the pair loads and decodes its own 128 rows of A and half of the tokens of B;
 // rank 0 issues the MMAs for both, so the barriers the MMAs wait on live in rank 0:
-//   full[s]    rank 0: one arrival (its producer, with both CTAs' bytes) and the copies of both
-//   aready[s]  rank 0: one arrival per CTA's decoder (code product)
+//   full[s]    rank 0: one arrival of its producer with both CTAs' bytes, the copies of both,
+//              and in the code product one arrival per decoder warp of both CTAs
 //   tempty[b]  rank 0: one arrival per epilogue warp of both CTAs
-// and the MMAs' completions are committed to both CTAs (empty[s], tfull[b]).  cfull[s] (code
-// blocks landed) stays local.  Ring stage s is decoded by decoder warp s.  Every producer
-// waits for the last use of each of its stages before it leaves, so no copy is in flight then.
-template <int PHASE>
+// and the MMAs' completions are committed to both CTAs (empty[s], tfull[b]).  The producer waits
+// for the last use of each of its stages before it leaves, so no copy is in flight then.
+//
+// The code product's round is a chain: stage free, codes expanded, MMAs, stage free.  So the
+// codes do not pass through shared memory: round i is expanded by decoder i mod 6 of two warps (64
+// rows each), which hold the round's codes in registers, loaded from global memory right after
+// they handed over round i - 6 (not before: the release of a hand-over waits for loads in flight).  A decoder meets a stage only in some of its rounds, but it never waits for
+// a phase more than one past the last one complete: at round i it has seen round i - 6 - S's
+// MMAs (S stages) complete, the commits are in order, and 6 <= S.
+template <int PHASE, int BN_>
 struct PairLayout {
   static constexpr bool kCodes = PHASE == kCore;
-  static constexpr int kBN = 256;                       // tokens per tile
-  static constexpr int kBTile = kBN / 2 * kBK * 2;      // this CTA's half of them: 16 KiB
-  static constexpr int kStages = 6;
+  static constexpr int kBN = BN_;                       // tokens per tile
+  static constexpr int kBTile = kBN / 2 * kBK * 2;      // this CTA's half of them
+  // analysis: [4][kBN] sums of z; code product: [kBN] sums of z
+  static constexpr int kSums = PHASE == kAnalysis ? 4 * kBN * 4 : (kCodes ? kBN * 4 : 0);
+  static constexpr int kStages = (225 * 1024 - kSums) / (kATileBytes + kBTile);
   static constexpr int kEpiWarps = 8;                   // two per TMEM quarter
   static constexpr int kEpiThreads = 32 * kEpiWarps;
-  static constexpr int kDecWarps = kCodes ? kStages : 0;
+  static constexpr int kHalf = kBN / 2;                 // columns per epilogue warp
+  static constexpr int kDecoders = 6;                   // of two warps each
+  static constexpr int kDecWarps = kCodes ? 2 * kDecoders : 0;
   static constexpr int kThreads = 64 + kEpiThreads + 32 * kDecWarps;
-  static constexpr uint32_t kTmemCols = 512;            // two accumulators of 256 columns
+  static constexpr uint32_t kTmemCols = 512;            // all, so that both CTAs' base is 0
   static constexpr int oA = 0;
   static constexpr int oB = oA + kStages * kATileBytes;
-  static constexpr int oCodes = oB + kStages * kBTile;
-  static constexpr int oBar = oCodes + (kCodes ? kStages * kCodeBytes : 0);
-  static constexpr int kNumBars = 4 * kStages + 4;
+  static constexpr int oBar = oB + kStages * kBTile;
+  static constexpr int kNumBars = 2 * kStages + 4;
   static constexpr int oMisc = oBar + kNumBars * 8;     // TMEM address, abort and last-split flags
-  static constexpr int oRed = oMisc + 16;               // analysis: [4][256] sums of z
-  static constexpr int oZsum = oRed + (PHASE == kAnalysis ? 4 * kBN * 4 : 0);   // core: [256]
-  static constexpr int kBytes = oZsum + (kCodes ? kBN * 4 : 0) + 1024;          // + alignment slack
+  static constexpr int oSums = oMisc + 16;
+  static constexpr int kBytes = oSums + kSums + 1024;   // + alignment slack
+  static_assert(kBN == 128 || kBN == 256, "tokens per tile");
+  static_assert(2 * kBN <= 512, "two accumulators");
+  static_assert(kBTile % 1024 == 0, "B tiles keep 1024-byte alignment");
+  static_assert(!kCodes || kDecoders <= kStages, "a decoder waits for a stage's latest phase only");
   static_assert(kBytes <= 227 * 1024, "shared memory");
 };
 
@@ -643,14 +664,13 @@ __device__ __forceinline__ float warp_sums16(const float (&v)[kChunk], int lane)
   return d + __shfl_xor_sync(0xffffffffu, d, 1);
 }
 
-template <int PHASE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::kThreads, 1)
+template <int PHASE, int BN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN>::kThreads, 1)
     tc_pair_kernel(const __grid_constant__ CUtensorMap tmA,
                    const __grid_constant__ CUtensorMap tmB, const PhaseArgs p) {
-  using Lo = PairLayout<PHASE>;
+  using Lo = PairLayout<PHASE, BN>;
   constexpr int S_ = Lo::kStages;
   constexpr bool kCodes = Lo::kCodes;
-  constexpr int BN = Lo::kBN;
   constexpr uint32_t kFullBytes = 2 * ((kCodes ? 0 : kATileBytes) + Lo::kBTile);
 
   extern __shared__ uint8_t smem_raw[];
@@ -658,18 +678,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sA = smem + Lo::oA;
   uint8_t* sB = smem + Lo::oB;
-  uint8_t* sCodes = smem + Lo::oCodes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + Lo::oBar);
   uint64_t* empty = full + S_;
-  uint64_t* aready = empty + S_;
-  uint64_t* cfull = aready + S_;
-  uint64_t* tfull = cfull + S_;
+  uint64_t* tfull = empty + S_;
   uint64_t* tempty = tfull + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Lo::oMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
-  float* red = reinterpret_cast<float*>(smem + Lo::oRed);
-  float* zsum_s = reinterpret_cast<float*>(smem + Lo::oZsum);
+  float* red = reinterpret_cast<float*>(smem + Lo::oSums);
+  float* zsum_s = red;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
@@ -684,10 +701,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S_; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], kCodes ? 5 : 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&aready[s], 2);
-      mbar_init(&cfull[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
@@ -713,17 +728,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
       const uint64_t pol_x = policy_evict_last();
       const bool leader = rank == 0;
       auto load_a = [&](int stage, int rt, int kb) {
-        const int rt1 = row_tile(rt);
-        if (kCodes) {
-          mbar_arrive_expect_tx(&cfull[stage], kCodeBytes);
-          bulk_load(sCodes + stage * kCodeBytes,
-                    p.words + (static_cast<int64_t>(min(rt1, p.RT1 - 1)) * p.KB + kb) * 512,
-                    kCodeBytes, &cfull[stage], pol_w);
-        } else {
-          if (leader) mbar_arrive_expect_tx(&full[stage], kFullBytes);
+        if (leader) mbar_arrive_expect_tx(&full[stage], kFullBytes);
+        if (!kCodes)
           tma_load_2d_pair(sA + stage * kATileBytes, &tmA, mapa(smem_u32(&full[stage]), 0),
-                           kb * kBK, rt1 * kBM, pol_w);
-        }
+                           kb * kBK, row_tile(rt) * kBM, pol_w);
       };
       // weight tiles of the first unit do not depend on the previous kernel: a ring of them is
       // requested, and the rest warmed in L2, before waiting for it
@@ -765,7 +773,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
             }
             load_a(stage, rt, kb);
           }
-          if (kCodes && leader) mbar_arrive_expect_tx(&full[stage], kFullBytes);
           tma_load_2d_pair(sB + stage * Lo::kBTile, &tmB, mapa(smem_u32(&full[stage]), 0),
                            kb * kBK, tt * BN + static_cast<int>(rank) * (BN / 2), pol_x);
           if (++stage == S_) stage = 0, phase ^= 1;
@@ -801,8 +808,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * BN);
         for (int kb = k0; kb < k1; ++kb) {
-          ok = mbar_wait_cluster(&full[stage], phase, abort_flag) &&
-               (!kCodes || mbar_wait_cluster(&aready[stage], phase, abort_flag));
+          ok = mbar_wait_cluster(&full[stage], phase, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
           const uint64_t adesc = umma_desc_sw128(smem_u32(sA + stage * kATileBytes));
@@ -827,7 +833,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
     // ---------------------------------------------------------------- epilogue (rows)
     constexpr int kN = Lo::kEpiThreads;
     const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
-    const int half = (warp - 2) >> 2;             // columns 128 * half .. + 127
+    const int c_lo = (warp - 2) / 4 * Lo::kHalf;  // columns c_lo .. c_hi - 1
+    const int c_hi = c_lo + Lo::kHalf;
     const int r_in_tile = quarter * 32 + lane;
     const int et = threadIdx.x - 64;
     pdl_wait();
@@ -849,12 +856,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
         // sum_j z[t][j] of the tile's tokens (one per thread), from the analysis' per-tile sums
         const int t = t0 + et;
         float s = 0.f;
-        if (t < p.M)
+        if (et < BN && t < p.M)
 #pragma unroll 8
           for (int g = 0; g < p.zsum_tiles; ++g)
             s += ldcg_f32(p.zsum_part + static_cast<int64_t>(g) * p.M + t);
         named_barrier_sync(1, kN);                // the previous unit's sums have been read
-        zsum_s[et] = s;
+        if (et < BN) zsum_s[et] = s;
       }
       const bool fail = !mbar_wait(&tfull[buf], acc_phase, abort_flag);
       if (fail) report(p.status, FQ_ERR_TIMEOUT);
@@ -900,7 +907,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
       bool finish = true;
       if (p.KS == 1) {
 #pragma unroll 1
-        for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+        for (int c = c_lo; c < c_hi; c += kChunk) {
           float v[kChunk];
           tmem_ld16(t_row + c, v);
           tmem_wait_ld();
@@ -917,7 +924,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
         const bool mine_ok = rt1 < p.RT1;
         float* mine = p.part + (t1 * p.KS + split) * BN * kBM;
 #pragma unroll 1
-        for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+        for (int c = c_lo; c < c_hi; c += kChunk) {
           float v[kChunk];
           tmem_ld16(t_row + c, v);
           tmem_wait_ld();
@@ -945,7 +952,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
         if (finish) {
           const float* all = p.part + t1 * p.KS * BN * kBM;
 #pragma unroll 1
-          for (int c = half * 128; c < half * 128 + 128; c += kChunk) {
+          for (int c = c_lo; c < c_hi; c += kChunk) {
             float v[kChunk];
 #pragma unroll
             for (int q = 0; q < kChunk; ++q) v[q] = 0.f;
@@ -962,7 +969,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
       if (PHASE == kAnalysis && !p.out32 && finish) {
         // the tile's sum of z per token, quarters added in a fixed order
         named_barrier_sync(1, kN);
-        if (rt1 < p.RT1 && t0 + et < p.M)
+        if (et < BN && rt1 < p.RT1 && t0 + et < p.M)
           p.zsum_part[static_cast<int64_t>(rt1) * p.M + t0 + et] =
               (red[et] + red[BN + et]) + (red[2 * BN + et] + red[3 * BN + et]);
         named_barrier_sync(1, kN);                   // read before the next unit's sums
@@ -980,16 +987,48 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
   } else {
     // ---------------------------------------------------------------- code decoders (core)
     if (kCodes) {
-      // decoder d expands every code block of ring stage d, four rows per lane
-      const int d = warp - 2 - Lo::kEpiWarps;
-      const uint32_t ready_bar = mapa(smem_u32(&aready[d]), 0);
-      const uint4* codes = reinterpret_cast<const uint4*>(sCodes + d * kCodeBytes);
-      uint8_t* tile_a = sA + d * kATileBytes;
-      int total = 0;                              // this pair's K blocks over all its units
-      for (int unit = pair; unit < p.units; unit += npairs) total += unit_k1(unit) - unit_k0(unit);
-      uint32_t phase = 0;
-      for (int it = d; it < total; it += S_, phase ^= 1) {
-        const bool got = mbar_wait(&cfull[d], phase, abort_flag);
+      // decoder d expands the code blocks of rounds d, d + 6, ...; its warp h rows 64 h .. + 63,
+      // two per lane
+      const int dw = warp - 2 - Lo::kEpiWarps;
+      const int d = dw >> 1, r0 = (dw & 1) * 64 + lane;
+      // the codes to load next: K block kb of `unit` (past k1: of a later unit), at src
+      int unit = pair, kb = 0, k1 = 0;
+      const uint4* src = nullptr;
+      auto enter = [&](int over) {               // K block k0 + over of the unit
+        while (unit < p.units) {
+          const int k0 = unit_k0(unit);
+          k1 = unit_k1(unit);
+          if (k0 + over < k1) {
+            kb = k0 + over;
+            const int rt1 = min(row_tile(unit_tile(unit) / p.TT), p.RT1 - 1);
+            src = reinterpret_cast<const uint4*>(
+                      p.words + (static_cast<int64_t>(rt1) * p.KB + kb) * 512) + r0;
+            return;
+          }
+          over -= k1 - k0;
+          unit += npairs;
+        }
+      };
+      enter(d);
+      uint4 codes[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+      auto fetch = [&]() -> bool {               // the next round's codes; false past the last
+        if (unit >= p.units) return false;
+        codes[0] = ldg_stream_u4(src);
+        codes[1] = ldg_stream_u4(src + 32);
+        kb += Lo::kDecoders;
+        src += Lo::kDecoders * (kCodeBytes / 16);
+        if (kb >= k1) {
+          const int over = kb - k1;
+          unit += npairs;
+          enter(over);
+        }
+        return true;
+      };
+      bool have = fetch();
+      int stage = d;                             // round mod S_
+      uint32_t phase = 0;                        // (round / S_) & 1
+      while (have) {
+        const bool got = mbar_wait(&empty[stage], phase ^ 1, abort_flag);
         if (!__all_sync(0xffffffffu, got)) {
           if (lane == 0) {
             report(p.status, FQ_ERR_TIMEOUT);
@@ -997,12 +1036,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE>::k
           }
           break;
         }
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr)
-          decode_row_fma(codes[lane + 32 * rr], tile_a, lane + 32 * rr);
+        uint8_t* tile_a = sA + stage * kATileBytes;
+        decode_row_fma(codes[0], tile_a, r0);
+        decode_row_fma(codes[1], tile_a, r0 + 32);
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(ready_bar);
+        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&full[stage]), 0));
+        have = fetch();
+        stage += Lo::kDecoders;
+        if (stage >= S_) stage -= S_, phase ^= 1;
       }
     }
   }
@@ -1113,13 +1155,13 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-// bf16 matrix rows x cols (row-major), boxes of 64 columns x 128 rows, 128-byte swizzle.
-bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols) {
+// bf16 matrix rows x cols (row-major), boxes of 64 columns x box_rows rows, 128-byte swizzle.
+bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int box_rows) {
   auto enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(kBM)};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(kBK), static_cast<cuuint32_t>(box_rows)};
   cuuint32_t estr[2] = {1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1183,11 +1225,9 @@ void plan_phase(PhaseArgs& a, const DeviceInfo& d, int& grid) {
   grid = std::min(a.units, d.sms);
 }
 
-// The same on CTA pairs: units of 256 x 256 tiles (or K splits of them), one pair per unit and
+// The same on CTA pairs: units of 256 x BN tiles (or K splits of them), one pair per unit and
 // round.  A split's partial tiles are kept per 128-row tile, in the workspace planned for those.
-template <int PHASE>
-void plan_pairs(PhaseArgs& a, int pairs, int& grid) {
-  constexpr int BN = PairLayout<PHASE>::kBN;
+void plan_pairs(PhaseArgs& a, int BN, int pairs, int& grid) {
   a.RT1 = static_cast<int>(ceil_div(a.R, kBM));
   a.RT = static_cast<int>(ceil_div(a.R, 2 * kBM));
   a.TT = static_cast<int>(ceil_div(a.M, BN));
@@ -1239,15 +1279,15 @@ WsLayout ws_layout(int M, int d_in, int n_in, int n_out, int d_out, int act_bits
 
 // CTA pairs of this kernel that fit the device at once (0 on an error); sets the kernel's shared
 // memory attribute on the device's first call.
-template <int PHASE>
+template <int PHASE, int BN>
 int resident_pairs(int dev) {
   static std::mutex mu;
   static std::map<int, int> cache;
   std::lock_guard<std::mutex> g(mu);
   const auto it = cache.find(dev);
   if (it != cache.end()) return it->second;
-  using Lo = PairLayout<PHASE>;
-  if (cudaFuncSetAttribute(tc_pair_kernel<PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  using Lo = PairLayout<PHASE, BN>;
+  if (cudaFuncSetAttribute(tc_pair_kernel<PHASE, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            Lo::kBytes) != cudaSuccess)
     return 0;
   cudaLaunchConfig_t cfg{};
@@ -1262,7 +1302,7 @@ int resident_pairs(int dev) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<PHASE>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<PHASE, BN>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1270,58 +1310,64 @@ int resident_pairs(int dev) {
   return n;
 }
 
-// One phase: plan and launch it on CTA pairs (more than 128 tokens and at least two SMs) or on
-// single SMs, chained to the previous kernel with programmatic dependent launch.
+// Launch configuration chained to the previous kernel with programmatic dependent launch.
+struct ChainedLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  ChainedLaunch(int grid, int threads, int smem, cudaStream_t s) {
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  ChainedLaunch(const ChainedLaunch&) = delete;
+};
+
+template <int PHASE, int BN>
+cudaError_t run_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs& a,
+                      const DeviceInfo& d, cudaStream_t s) {
+  const int pairs = std::min(resident_pairs<PHASE, BN>(d.dev), d.sms / 2);
+  if (pairs < 1) return cudaErrorLaunchOutOfResources;
+  int grid = 0;
+  plan_pairs(a, BN, pairs, grid);
+  using Lo = PairLayout<PHASE, BN>;
+  const ChainedLaunch l(grid, Lo::kThreads, Lo::kBytes, s);
+  return cudaLaunchKernelEx(&l.cfg, tc_pair_kernel<PHASE, BN>, tmA, tmB, a);
+}
+
+// The token operand's box rows: a CTA pair's CTAs load half of a tile's tokens each.
+int token_box(int M, const DeviceInfo& d) { return d.sms >= 2 ? pick_bn(M) / 2 : 128; }
+
+// One phase, planned and launched: on CTA pairs, or on one SM for a budget of one.
 template <int PHASE>
 cudaError_t run_phase(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs& a,
                       const DeviceInfo& d, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int grid = 0;
-  if (a.M > 128 && d.sms >= 2) {
-    const int pairs = std::min(resident_pairs<PHASE>(d.dev), d.sms / 2);
-    if (pairs < 1) return cudaErrorLaunchOutOfResources;
-    plan_pairs<PHASE>(a, pairs, grid);
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(PairLayout<PHASE>::kThreads);
-    cfg.dynamicSmemBytes = PairLayout<PHASE>::kBytes;
-    return cudaLaunchKernelEx(&cfg, tc_pair_kernel<PHASE>, tmA, tmB, a);
-  }
+  if (d.sms >= 2)
+    return pick_bn(a.M) == 128 ? run_pairs<PHASE, 128>(tmA, tmB, a, d, s)
+                               : run_pairs<PHASE, 256>(tmA, tmB, a, d, s);
   if (const cudaError_t e = prepare_kernel<PHASE, 128>(d.dev)) return e;
+  int grid = 0;
   plan_phase<PHASE, 128>(a, d, grid);
-  cfg.gridDim = dim3(static_cast<unsigned>(grid));
-  cfg.blockDim = dim3(threads_for<PHASE>());
-  cfg.dynamicSmemBytes = Layout<PHASE, 128>::kBytes;
-  return cudaLaunchKernelEx(&cfg, tc_phase_kernel<PHASE, 128>, tmA, tmB, a);
+  const ChainedLaunch l(grid, threads_for<PHASE>(), Layout<PHASE, 128>::kBytes, s);
+  return cudaLaunchKernelEx(&l.cfg, tc_phase_kernel<PHASE, 128>, tmA, tmB, a);
+}
+
+cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
+                         float* delta, __nv_bfloat16* zq, float* zsum, cudaStream_t s) {
+  const ChainedLaunch l(std::max(1, std::min(an.M, 4 * d.sms)), kQuantThreads, 0, s);
+  const float L = static_cast<float>((1 << (act_bits - 1)) - 1);
+  return cudaLaunchKernelEx(&l.cfg, ff_round_kernel, static_cast<const float*>(an.out32), an.M,
+                            n_in, L, static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
 }
 
 // maps: {T_in, x, z, T_out^T, u}.  The core phase's A operand is the packed codes, so it gets
 // an unused map in that slot.
-cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
-                         float* delta, __nv_bfloat16* zq, float* zsum, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(std::max(1, std::min(an.M, 4 * d.sms))));
-  cfg.blockDim = dim3(kQuantThreads);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const float L = static_cast<float>((1 << (act_bits - 1)) - 1);
-  return cudaLaunchKernelEx(&cfg, ff_round_kernel, static_cast<const float*>(an.out32), an.M,
-                            n_in, L, static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
-}
-
-fq_status run_forward(const CUtensorMap* maps, PhaseArgs* a, int max_sms, int act_bits,
+fq_status run_forward(const CUtensorMap* maps, PhaseArgs* a, const DeviceInfo& d, int act_bits,
                       float* delta, cudaStream_t s) {
-  DeviceInfo d = device_info();
-  if (max_sms > 0) d.sms = std::min(d.sms, max_sms);
   a[1].zsum_tiles =
       act_bits > 0 ? 1 : static_cast<int>(ceil_div(a[0].R, kBM));   // rounded: one exact sum
   if (run_phase<kAnalysis>(maps[0], maps[1], a[0], d, s) != cudaSuccess) return FQ_ERR_CUDA;
@@ -1370,8 +1416,10 @@ fq_status launch_tc_dense(const void* x, int M, int d_in, const void* W, int d_o
   a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
   a.part = reinterpret_cast<float*>(ws + L.part);
   CUtensorMap mW, mX;
-  if (!make_tmap(&mW, W, d_out, d_in) || !make_tmap(&mX, x, M, d_in)) return FQ_ERR_CUDA;
-  return run_phase<kSynthesis>(mW, mX, a, device_info(), s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
+  const DeviceInfo d = device_info();
+  if (!make_tmap(&mW, W, d_out, d_in, kBM) || !make_tmap(&mX, x, M, d_in, token_box(M, d)))
+    return FQ_ERR_CUDA;
+  return run_phase<kSynthesis>(mW, mX, a, d, s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1424,12 +1472,16 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
   }
 
   // maps: T_in, x, z, T_out^T, u
+  DeviceInfo d = device_info();
+  if (max_sms > 0) d.sms = std::min(d.sms, max_sms);
+  const int box = token_box(M, d);
   CUtensorMap maps[5];
-  if (!make_tmap(&maps[0], T_in, n_in, d_in) || !make_tmap(&maps[1], x, M, d_in) ||
-      !make_tmap(&maps[2], z, M, n_in) || !make_tmap(&maps[3], T_out_t, d_out, n_out) ||
-      !make_tmap(&maps[4], u, M, n_out))
+  if (!make_tmap(&maps[0], T_in, n_in, d_in, kBM) || !make_tmap(&maps[1], x, M, d_in, box) ||
+      !make_tmap(&maps[2], z, M, n_in, box) ||
+      !make_tmap(&maps[3], T_out_t, d_out, n_out, kBM) ||
+      !make_tmap(&maps[4], u, M, n_out, box))
     return FQ_ERR_CUDA;
-  return run_forward(maps, a, max_sms, act_bits, delta, s);
+  return run_forward(maps, a, d, act_bits, delta, s);
 }
 
 fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq,
@@ -1466,8 +1518,11 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
 
   // maps: z (the code product's B; also the unused A slot), T_out^T, u
   CUtensorMap maps[3];
-  if (!make_tmap(&maps[0], z, M, n_in) || !make_tmap(&maps[1], T_out_t, d_out, n_out) ||
-      !make_tmap(&maps[2], u, M, n_out))
+  const DeviceInfo d = device_info();
+  const int box = token_box(M, d);
+  if (!make_tmap(&maps[0], z, M, n_in, box) ||
+      !make_tmap(&maps[1], T_out_t, d_out, n_out, kBM) ||
+      !make_tmap(&maps[2], u, M, n_out, box))
     return FQ_ERR_CUDA;
 
   unit_analysis_kernel<<<dim3(static_cast<unsigned>(ceil_div(d_in, 32)),
@@ -1478,7 +1533,6 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
       Tin, n_in, d_in, zsum, status);
   if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
   // the code product and the synthesis, with one sum of z per token
-  const DeviceInfo d = device_info();
   a[1].zsum_tiles = 1;
   return run_phase<kCore>(maps[0], maps[0], a[1], d, s) == cudaSuccess &&
                  run_phase<kSynthesis>(maps[1], maps[2], a[2], d, s) == cudaSuccess
