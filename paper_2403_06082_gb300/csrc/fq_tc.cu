@@ -1061,38 +1061,66 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
 // Rounding of the frame representation of the activations (Appendix F): with the tensor's
 // step Delta = max |z| / L, L = 2^(N-1) - 1, zq = nearest integer to z / Delta (ties to even,
 // clamped to [-L, L]) as bf16 (exact: |zq| <= 127 needs 7 significant bits), and the per-token
-// sum of zq for the zero term (exact in fp32: at most 127 * 81920 < 2^24).  One block per
-// token row and round.
+// sum of zq for the zero term (exact in fp32 in any order: at most 127 * 81920 < 2^24).
+//
+// Memory-bound: 6 bytes per coefficient.  A token is rounded by one warp (kPer = 32) or one block
+// (kPer = 256), eight coefficients per thread and step (32-byte loads, one 16-byte store; n is
+// a multiple of 16).  PLACEHOLDER_ROUND
 constexpr int kQuantThreads = 256;
+constexpr int kWarpTokenMaxN = 2048;
 
+template <int kPer>
 __global__ void __launch_bounds__(kQuantThreads) ff_round_kernel(
     const float* __restrict__ z32, int M, int n, float L, const uint32_t* __restrict__ amax,
     float* __restrict__ delta, __nv_bfloat16* __restrict__ zq, float* __restrict__ zsum) {
+  constexpr int kTokens = kQuantThreads / kPer;      // tokens per block and round
   __shared__ float red[kQuantThreads / 32];
   pdl_launch_dependents();
   pdl_wait();                                   // the analysis is complete
   const float d = __uint_as_float(*reinterpret_cast<const volatile uint32_t*>(amax)) / L;
   if (blockIdx.x == 0 && threadIdx.x == 0) *delta = d;
-  for (int t = blockIdx.x; t < M; t += gridDim.x) {
-    const float* zr = z32 + static_cast<int64_t>(t) * n;
-    __nv_bfloat16* qr = zq + static_cast<int64_t>(t) * n;
+  const int sub = threadIdx.x % kPer;
+  for (int t0 = blockIdx.x * kTokens; t0 < M; t0 += gridDim.x * kTokens) {
+    const int t = t0 + threadIdx.x / kPer;
     float s = 0.f;
-    for (int j = threadIdx.x; j < n; j += kQuantThreads) {
-      float q = d > 0.f ? rintf(__fdiv_rn(__ldcg(zr + j), d)) : 0.f;
-      q = fminf(fmaxf(q, -L), L);
-      qr[j] = __float2bfloat16_rn(q);
-      s += q;
+    if (t < M) {
+      const float* zr = z32 + static_cast<int64_t>(t) * n;
+      __nv_bfloat16* qr = zq + static_cast<int64_t>(t) * n;
+#pragma unroll 2
+      for (int j = 8 * sub; j < n; j += 8 * kPer) {
+        const float4 lo = __ldcg(reinterpret_cast<const float4*>(zr + j));
+        const float4 hi = __ldcg(reinterpret_cast<const float4*>(zr + j + 4));
+        const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float q[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            q[h] = d > 0.f ? rintf(__fdiv_rn(v[2 * e + h], d)) : 0.f;
+            q[h] = fminf(fmaxf(q[h], -L), L);
+            s += q[h];
+          }
+          const __nv_bfloat162 b = __floats2bfloat162_rn(q[0], q[1]);
+          w[e] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        *reinterpret_cast<uint4*>(qr + j) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      for (int w = 0; w < kQuantThreads / 32; ++w) tot += red[w];
-      zsum[t] = tot;
+    if (kPer == 32) {
+      if (sub == 0 && t < M) zsum[t] = s;
+    } else {
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        float tot = 0.f;
+        for (int w = 0; w < kQuantThreads / 32; ++w) tot += red[w];
+        zsum[t] = tot;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
 }
 
@@ -1358,10 +1386,15 @@ cudaError_t run_phase(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs&
 
 cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
                          float* delta, __nv_bfloat16* zq, float* zsum, cudaStream_t s) {
-  const ChainedLaunch l(std::max(1, std::min(an.M, 4 * d.sms)), kQuantThreads, 0, s);
+  // one warp per token when a token has little work for a block and there are tokens for every
+  // SM's warps; one block per token otherwise
+  const bool warps = n_in <= kWarpTokenMaxN && an.M >= 8 * d.sms;
+  const int blocks = static_cast<int>(ceil_div(an.M, warps ? kQuantThreads / 32 : 1));
+  const ChainedLaunch l(std::min(blocks, 8 * d.sms), kQuantThreads, 0, s);
   const float L = static_cast<float>((1 << (act_bits - 1)) - 1);
-  return cudaLaunchKernelEx(&l.cfg, ff_round_kernel, static_cast<const float*>(an.out32), an.M,
-                            n_in, L, static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
+  return cudaLaunchKernelEx(&l.cfg, warps ? ff_round_kernel<32> : ff_round_kernel<kQuantThreads>,
+                            static_cast<const float*>(an.out32), an.M, n_in, L,
+                            static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
 }
 
 // maps: {T_in, x, z, T_out^T, u}.  The core phase's A operand is the packed codes, so it gets
