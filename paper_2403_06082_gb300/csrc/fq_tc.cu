@@ -146,6 +146,17 @@ __device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
   return v;
 }
 
+// True in one lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
   uint32_t out;
   asm volatile(
@@ -587,6 +598,7 @@ struct PairLayout {
   static constexpr int kEpiWarps = 8;                   // two per TMEM quarter
   static constexpr int kEpiThreads = 32 * kEpiWarps;
   static constexpr int kHalf = kBN / 2;                 // columns per epilogue warp
+  static constexpr int kGroups = kCodes ? 1 : 2;        // of 16 columns at a time (registers)
   static constexpr int kDecoders = 6;                   // of two warps each
   static constexpr int kDecWarps = kCodes ? 2 * kDecoders : 0;
   static constexpr int kThreads = 64 + kEpiThreads + 32 * kDecWarps;
@@ -664,6 +676,70 @@ __device__ __forceinline__ float warp_sums16(const float (&v)[kChunk], int lane)
   return d + __shfl_xor_sync(0xffffffffu, d, 1);
 }
 
+// Transposes between the lanes of a warp, so that results leave in 16-byte stores: on entry lane l
+// holds row l of 16 columns, on return rows of a group of consecutive rows.
+//   bf16:  eight rows 8 (l / 8) .. + 7 of columns column16(l) and column16(l) + 1, in w[0..3] and w[4..7]
+//   fp32:  four rows 4 (l / 4) .. + 3 of columns 8 b0 + 4 b1 + 0 .. 3 (b0, b1 the low bits of l)
+// Each step exchanges half of a lane's registers with the lane 1, 2 (, 4) away.
+__device__ __forceinline__ int column16(int lane) {
+  return 8 * (lane & 1) + 4 * ((lane >> 1) & 1) + 2 * ((lane >> 2) & 1);
+}
+
+// The registers a lane keeps (of a) and what its partner sends, in the order of the partners'
+// rows: lower rows in lo, upper rows in hi.
+template <int N>
+__device__ __forceinline__ void exchange(const uint32_t* a, int lane, int bit, uint32_t* lo,
+                                         uint32_t* hi) {
+  const bool up = lane & bit;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint32_t send = up ? a[i] : a[i + N], keep = up ? a[i + N] : a[i];
+    const uint32_t got = __shfl_xor_sync(0xffffffffu, send, bit);
+    lo[i] = up ? got : keep;
+    hi[i] = up ? keep : got;
+  }
+}
+
+__device__ __forceinline__ void transpose_bf16(const uint32_t (&h)[8], int lane,
+                                               uint32_t (&w)[8]) {
+  uint32_t lo[4], hi[4], g[8];
+  exchange<4>(h, lane, 1, lo, hi);               // pairs of columns, rows 2m and 2m + 1
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    g[2 * i] = __byte_perm(lo[i], hi[i], 0x5410);       // the even column of the pair
+    g[2 * i + 1] = __byte_perm(lo[i], hi[i], 0x7632);   // the odd one
+  }
+  exchange<4>(g, lane, 2, lo, hi);               // four columns, rows 4m .. 4m + 3
+#pragma unroll
+  for (int i = 0; i < 4; ++i) g[2 * i] = lo[i], g[2 * i + 1] = hi[i];
+  exchange<4>(g, lane, 4, lo, hi);               // two columns, rows 8m .. 8m + 7
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    w[4 * i] = lo[2 * i];
+    w[4 * i + 1] = lo[2 * i + 1];
+    w[4 * i + 2] = hi[2 * i];
+    w[4 * i + 3] = hi[2 * i + 1];
+  }
+}
+
+__device__ __forceinline__ void transpose_fp32(const float (&v)[16], int lane,
+                                               uint32_t (&w)[16]) {
+  uint32_t a[16], lo[8], hi[8];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = __float_as_uint(v[i]);
+  exchange<8>(a, lane, 1, lo, hi);               // eight columns, rows 2m and 2m + 1
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[2 * i] = lo[i], a[2 * i + 1] = hi[i];
+  exchange<8>(a, lane, 2, lo, hi);               // four columns, rows 4m .. 4m + 3
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    w[4 * i] = lo[2 * i];
+    w[4 * i + 1] = lo[2 * i + 1];
+    w[4 * i + 2] = hi[2 * i];
+    w[4 * i + 3] = hi[2 * i + 1];
+  }
+}
+
 template <int PHASE, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN>::kThreads, 1)
     tc_pair_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -688,7 +764,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
   float* red = reinterpret_cast<float*>(smem + Lo::oSums);
   float* zsum_s = red;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);   // uniform
+  const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = static_cast<int>(blockIdx.x >> 1), npairs = static_cast<int>(gridDim.x >> 1);
   // work unit u = split * tiles + tile: K blocks [split * kbs, min(KB, (split + 1) * kbs))
@@ -796,35 +873,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (rank 0)
-    if (lane == 0 && rank == 0) {
+    // The whole warp walks the rounds and one elected lane issues: the operands then are
+    // warp-uniform where they are computed, and a round's waits, MMAs and commit take fewer
+    // cycles than its MMAs (with one lane walking alone a round took 656 cycles, more than the
+    // 256 of four 256 x 128 x 16 MMAs and the 512 of 256 x 256 x 16).
+    if (rank == 0) {
       constexpr uint32_t idesc = umma_idesc_bf16(2 * kBM, BN);
+      const uint64_t a0 = umma_desc_sw128(smem_u32(sA)), b0 = umma_desc_sw128(smem_u32(sB));
+      const bool elected = elect_one();
       int stage = 0, buf = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
-      for (int unit = pair; unit < p.units && ok && !*abort_flag; unit += npairs) {
+      for (int unit = pair; unit < p.units; unit += npairs) {
         const int k0 = unit_k0(unit), k1 = unit_k1(unit);
-        ok = mbar_wait_cluster(&tempty[buf], acc_phase ^ 1, abort_flag);
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&tempty[buf], acc_phase ^ 1, abort_flag));
         if (!ok) break;
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * BN);
         for (int kb = k0; kb < k1; ++kb) {
-          ok = mbar_wait_cluster(&full[stage], phase, abort_flag);
+          ok = __all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort_flag));
           if (!ok) break;
           tc_fence_after_sync();
-          const uint64_t adesc = umma_desc_sw128(smem_u32(sA + stage * kATileBytes));
-          const uint64_t bdesc = umma_desc_sw128(smem_u32(sB + stage * Lo::kBTile));
+          if (elected) {
+            const uint64_t adesc = a0 + static_cast<uint64_t>(stage * (kATileBytes >> 4));
+            const uint64_t bdesc = b0 + static_cast<uint64_t>(stage * (Lo::kBTile >> 4));
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc,
-                           (kb > k0 || k > 0) ? 1u : 0u);
-          umma_commit_pair(&empty[stage]);
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_bf16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc,
+                             (kb > k0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(&empty[stage]);
+          }
+          __syncwarp();
           if (++stage == S_) stage = 0, phase ^= 1;
         }
         if (!ok) break;
-        umma_commit_pair(&tfull[buf]);
+        if (elected) umma_commit_pair(&tfull[buf]);
+        __syncwarp();
         if (++buf == 2) buf = 0, acc_phase ^= 1;
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         report(p.status, FQ_ERR_TIMEOUT);
         *abort_flag = 1;
       }
@@ -877,26 +964,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
       // u = Delta gamma (s acc + zero sum_j zbar_j)
       const float dl = (PHASE == kCore && p.delta) ? ldcg_f32(p.delta) : 1.f;
       float amax_t = 0.f;
-      // the finished values of columns c .. c + 15 of this thread's row
+      // the finished values of columns c .. c + 15 of this thread's row, to memory (rows of R
+      // are a multiple of 8: a group of 8 or 4 rows is stored whole or not at all)
+      const int row_w = rt1 * kBM + quarter * 32;   // the warp's first row
       auto emit = [&](int c, float (&v)[kChunk]) {
         if (PHASE == kAnalysis && p.out32) {
+          // fp32 z for the rounding kernel, and the running maximum of |z| (zero past R and M)
 #pragma unroll
-          for (int q = 0; q < kChunk; ++q) {
-            const int t = t0 + c + q;
-            if (row_ok && t < p.M) {
-              p.out32[static_cast<int64_t>(t) * p.R + row] = v[q];
-              amax_t = fmaxf(amax_t, fabsf(v[q]));
-            }
+          for (int q = 0; q < kChunk; ++q) amax_t = fmaxf(amax_t, fabsf(v[q]));
+          uint32_t w[16];
+          transpose_fp32(v, lane, w);
+          const int r = row_w + 4 * (lane >> 2);
+          const int t = t0 + c + 8 * (lane & 1) + 4 * ((lane >> 1) & 1);
+          float* dst = p.out32 + static_cast<int64_t>(t) * p.R + r;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (r < p.R && t + q < p.M)
+              *reinterpret_cast<uint4*>(dst) =
+                  make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            dst += p.R;
           }
           return;
         }
+        uint32_t h[8], w[8];
 #pragma unroll
-        for (int q = 0; q < kChunk; ++q) {
-          if (PHASE == kCore) v[q] = g_i * fmaf(s_i, v[q], z_i * zsum_s[c + q]) * dl;
-          const __nv_bfloat16 b = __float2bfloat16_rn(v[q]);
-          v[q] = row_ok ? __bfloat162float(b) : 0.f;
-          const int t = t0 + c + q;
-          if (row_ok && t < p.M) p.out[static_cast<int64_t>(t) * p.R + row] = b;
+        for (int q = 0; q < kChunk; q += 2) {
+          if (PHASE == kCore) {
+            v[q] = g_i * fmaf(s_i, v[q], z_i * zsum_s[c + q]) * dl;
+            v[q + 1] = g_i * fmaf(s_i, v[q + 1], z_i * zsum_s[c + q + 1]) * dl;
+          }
+          const __nv_bfloat162 b = __floats2bfloat162_rn(v[q], v[q + 1]);
+          h[q / 2] = *reinterpret_cast<const uint32_t*>(&b);
+          if (PHASE == kAnalysis) {
+            v[q] = row_ok ? __low2float(b) : 0.f;
+            v[q + 1] = row_ok ? __high2float(b) : 0.f;
+          }
+        }
+        transpose_bf16(h, lane, w);
+        const int r = row_w + 8 * (lane >> 3), t = t0 + c + column16(lane);
+        __nv_bfloat16* dst = p.out + static_cast<int64_t>(t) * p.R + r;
+        if (r < p.R) {
+          if (t < p.M) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+          if (t + 1 < p.M)
+            *reinterpret_cast<uint4*>(dst + p.R) = make_uint4(w[4], w[5], w[6], w[7]);
         }
         if (PHASE == kAnalysis) {
           // per-token sum over the warp's 32 rows of the bf16 z actually stored
@@ -904,67 +1014,90 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
           if ((lane & 1) == 0) red[quarter * BN + c + (lane >> 1)] = s;
         }
       };
+      // the accumulator of columns c .. c + kW - 1
+      constexpr int kG = Lo::kGroups, kW = kG * kChunk;
+      auto load = [&](int c, float (&v)[kG][kChunk]) {
+#pragma unroll
+        for (int g = 0; g < kG; ++g) tmem_ld16(t_row + c + g * kChunk, v[g]);
+        tmem_wait_ld();
+      };
+      auto release = [&]() {
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[buf]), 0));
+      };
       bool finish = true;
       if (p.KS == 1) {
 #pragma unroll 1
-        for (int c = c_lo; c < c_hi; c += kChunk) {
-          float v[kChunk];
-          tmem_ld16(t_row + c, v);
-          tmem_wait_ld();
-          emit(c, v);
+        for (int c = c_lo; c < c_hi; c += kW) {
+          float v[kG][kChunk];
+          load(c, v);
+#pragma unroll
+          for (int g = 0; g < kG; ++g) emit(c + g * kChunk, v[g]);
         }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[buf]), 0));
+        release();
       } else {
-        // Split K: this CTA's partial tile to the workspace (column-major, so a warp's 32 rows
-        // are one 128-byte line), the accumulator released, the split counted in.  The last
-        // split of the CTA's 128-row tile to arrive adds the partials in split order.
+        // Split K.  The CTAs of the 128-row tile's splits take tickets as they get here.  All
+        // but the last store their partial tile in the workspace (column-major, so a warp's 32
+        // rows are one 128-byte line) and count it in; the last waits for those counts, adds the
+        // partials in split order with its own still in TMEM, and finishes the tile.  (The
+        // CTAs it waits for are past their MMAs; the wait is bounded like every other.)
         const int64_t t1 = static_cast<int64_t>(rt1) * p.TT + tt;
         const bool mine_ok = rt1 < p.RT1;
-        float* mine = p.part + (t1 * p.KS + split) * BN * kBM;
-#pragma unroll 1
-        for (int c = c_lo; c < c_hi; c += kChunk) {
-          float v[kChunk];
-          tmem_ld16(t_row + c, v);
-          tmem_wait_ld();
-          if (mine_ok) {
-#pragma unroll
-            for (int q = 0; q < kChunk; ++q) mine[(c + q) * kBM + r_in_tile] = v[q];
-          }
-        }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[buf]), 0));
-        __threadfence();
-        named_barrier_sync(1, kN);
-        if (et == 0) {
-          bool last = false;
-          if (mine_ok) {
-            last = atomicAdd(&p.cnt[t1], 1u) == static_cast<uint32_t>(p.KS - 1);
-            if (last) p.cnt[t1] = 0;                 // ready for the next call
-            __threadfence();
-          }
-          *last_flag = last ? 1 : 0;
-        }
+        uint32_t* cnt = p.cnt + t1;              // low half: tickets, high half: stored partials
+        if (et == 0)
+          *last_flag = mine_ok ? ((atomicAdd(cnt, 1u) & 0xffffu) == static_cast<uint32_t>(p.KS - 1))
+                               : 0;
         named_barrier_sync(1, kN);
         finish = *last_flag != 0;
-        if (finish) {
-          const float* all = p.part + t1 * p.KS * BN * kBM;
+        float* part = p.part + t1 * p.KS * BN * kBM + r_in_tile;
+        if (!finish) {
+          float* mine = part + static_cast<int64_t>(split) * BN * kBM;
 #pragma unroll 1
-          for (int c = c_lo; c < c_hi; c += kChunk) {
-            float v[kChunk];
+          for (int c = c_lo; mine_ok && c < c_hi; c += kW) {
+            float v[kG][kChunk];
+            load(c, v);
 #pragma unroll
-            for (int q = 0; q < kChunk; ++q) v[q] = 0.f;
-            for (int sp = 0; sp < p.KS; ++sp) {
-#pragma unroll
-              for (int q = 0; q < kChunk; ++q)
-                v[q] += ldcg_f32(all + (static_cast<int64_t>(sp) * BN + c + q) * kBM + r_in_tile);
-            }
-            emit(c, v);
+            for (int q = 0; q < kW; ++q)
+              mine[(c + q) * kBM] = v[q / kChunk][q % kChunk];
           }
+          release();
+          __threadfence();
+          named_barrier_sync(1, kN);
+          if (et == 0 && mine_ok) {
+            __threadfence();
+            atomicAdd(cnt, 0x10000u);
+          }
+        } else {
+          if (et == 0) {
+            const uint32_t want = (static_cast<uint32_t>(p.KS - 1) << 16) | static_cast<uint32_t>(p.KS);
+            const bool all = wait_flag(cnt, want, abort_flag);
+            if (!all) {
+              report(p.status, FQ_ERR_TIMEOUT);
+              *abort_flag = 1;
+            }
+            *cnt = 0;                            // ready for the next call
+          }
+          named_barrier_sync(1, kN);
+#pragma unroll 1
+          for (int c = c_lo; c < c_hi; c += kW) {
+            float v[kG][kChunk], own[kG][kChunk];
+            load(c, own);
+#pragma unroll
+            for (int q = 0; q < kW; ++q) v[q / kChunk][q % kChunk] = 0.f;
+            for (int sp = 0; sp < p.KS; ++sp) {
+              const float* other = part + (static_cast<int64_t>(sp) * BN + c) * kBM;
+#pragma unroll
+              for (int q = 0; q < kW; ++q)
+                v[q / kChunk][q % kChunk] +=
+                    sp == split ? own[q / kChunk][q % kChunk] : ldcg_f32(other + q * kBM);
+            }
+#pragma unroll
+            for (int g = 0; g < kG; ++g) emit(c + g * kChunk, v[g]);
+          }
+          release();
         }
-        named_barrier_sync(1, kN);                   // the flag is read before it is reused
+        named_barrier_sync(1, kN);               // the flag is read before it is reused
       }
       if (PHASE == kAnalysis && !p.out32 && finish) {
         // the tile's sum of z per token, quarters added in a fixed order
