@@ -70,6 +70,7 @@ struct PhaseArgs {
   const float* gamma;
   int32_t* status;
   int clear_status;          // this launch starts a call: clear the status word
+  int transposed;            // synthesis on CTA pairs: out is [R][M] (M a multiple of 8)
   // Rounding of the frame representation of the activations (Appendix F), else all null:
   float* out32;              // analysis: z in fp32 (the bf16 z is then the rounded one)
   uint32_t* amax;            // analysis: running max |z| as float bits; the core resets it
@@ -144,17 +145,6 @@ __device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
-}
-
-// True in one lane of the (converged) warp.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r));
-  return r != 0;
 }
 
 __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
@@ -1000,6 +990,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
             v[q + 1] = row_ok ? __high2float(b) : 0.f;
           }
         }
+        if (PHASE == kSynthesis && p.transposed) {
+          // this thread's row: 16 consecutive tokens, inside M eight at a time
+          __nv_bfloat16* dst = p.out + static_cast<int64_t>(row) * p.M + t0 + c;
+          if (row_ok && t0 + c < p.M)
+            *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+          if (row_ok && t0 + c + 8 < p.M)
+            *reinterpret_cast<uint4*>(dst + 8) = make_uint4(h[4], h[5], h[6], h[7]);
+          return;
+        }
         transpose_bf16(h, lane, w);
         const int r = row_w + 8 * (lane >> 3), t = t0 + c + column16(lane);
         __nv_bfloat16* dst = p.out + static_cast<int64_t>(t) * p.R + r;
@@ -1259,44 +1258,55 @@ __global__ void __launch_bounds__(kQuantThreads) ff_round_kernel(
 
 // The analysis of the d_in unit vectors, for the weight reconstruction: unit vector e_t has
 // z = T_in e_t = column t of T_in, exact in bf16, so the analysis product is a transpose,
-// z[t][j] = T_in[j][t], through 32 x 32 shared-memory tiles.
-__global__ void unit_analysis_kernel(const __nv_bfloat16* __restrict__ T_in, int n_in, int d_in,
-                                     __nv_bfloat16* __restrict__ z) {
-  __shared__ __nv_bfloat16 tile[32][34];
-  const int t0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-  for (int dy = threadIdx.y; dy < 32; dy += 8) {
-    const int j = j0 + dy, t = t0 + threadIdx.x;
-    if (j < n_in && t < d_in) tile[dy][threadIdx.x] = T_in[static_cast<int64_t>(j) * d_in + t];
-  }
-  __syncthreads();
-  for (int dy = threadIdx.y; dy < 32; dy += 8) {
-    const int t = t0 + dy, j = j0 + threadIdx.x;
-    if (t < d_in && j < n_in) z[static_cast<int64_t>(t) * n_in + j] = tile[threadIdx.x][dy];
-  }
-}
+// z[t][j] = T_in[j][t], with the sums of z over each 128-row tile of T_in, as the analysis of
+// tokens leaves them.  Memory-bound (4 bytes per element): a block moves 128 rows x 64 columns through
+// shared memory, 16 bytes per access at both ends (a row of 68 elements puts the 16 columns x 2
+// row groups that a warp gathers into 32 different banks).  PLACEHOLDER_UNIT
+constexpr int kUnitRows = 128, kUnitCols = 64;
 
-// sum_j z[t][j] of unit vector t (the column sums of T_in), for the code product's zero term.
-// Block of 32 columns x 32 row groups: thread (x, y) adds rows j = y, y + 32, ... of column
-// t0 + x (coalesced across the warp), then the 32 partial sums of a column are added in row
-// group order.  Block 0 clears the status word of the new call.
-__global__ void __launch_bounds__(1024) unit_zsum_kernel(const __nv_bfloat16* __restrict__ T_in,
-                                                         int n_in, int d_in,
-                                                         float* __restrict__ zsum,
-                                                         int32_t* __restrict__ status) {
-  __shared__ float part[32][33];
-  if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *status = 0;
-  const int t = blockIdx.x * 32 + threadIdx.x;
-  float s = 0.f;
-  if (t < d_in)
-    for (int j = threadIdx.y; j < n_in; j += 32)
-      s += __bfloat162float(T_in[static_cast<int64_t>(j) * d_in + t]);
-  part[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && t < d_in) {
-    float tot = 0.f;
-    for (int y = 0; y < 32; ++y) tot += part[y][threadIdx.x];
-    zsum[t] = tot;
+__global__ void __launch_bounds__(256) unit_analysis_kernel(const __nv_bfloat16* __restrict__ T_in,
+                                                            int n_in, int d_in,
+                                                            __nv_bfloat16* __restrict__ z,
+                                                            float* __restrict__ zsum,
+                                                            int32_t* __restrict__ status) {
+  __shared__ __align__(16) uint16_t tile[kUnitRows][kUnitCols + 4];
+  __shared__ float part[4][kUnitCols];
+  const int t0 = blockIdx.x * kUnitCols, j0 = blockIdx.y * kUnitRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *status = 0;     // a new call
+  // d_in is a multiple of 8: eight columns are inside or outside together
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int r = 32 * it + tid / 8, c = 8 * (tid % 8);
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (j0 + r < n_in && t0 + c < d_in)
+      v = __ldg(reinterpret_cast<const uint4*>(T_in + static_cast<int64_t>(j0 + r) * d_in + t0 + c));
+    *reinterpret_cast<uint2*>(&tile[r][c]) = make_uint2(v.x, v.y);
+    *reinterpret_cast<uint2*>(&tile[r][c + 4]) = make_uint2(v.z, v.w);
   }
+  __syncthreads();
+  // a warp and step: 16 columns of T_in, 16 of its rows (n_in is a multiple of 16)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int q = warp + 8 * k;
+    const int c = 16 * (q & 3) + (lane & 15), r = 16 * (q >> 2) + 8 * (lane >> 4);
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      w[e] = tile[r + 2 * e][c] | (static_cast<uint32_t>(tile[r + 2 * e + 1][c]) << 16);
+    if (t0 + c < d_in && j0 + r < n_in)
+      *reinterpret_cast<uint4*>(z + static_cast<int64_t>(t0 + c) * n_in + j0 + r) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  const int c = tid & 63, g = tid >> 6;          // 32 rows of one column per thread
+  float s = 0.f;
+#pragma unroll 8
+  for (int r = 32 * g; r < 32 * g + 32; ++r) s += __uint_as_float(static_cast<uint32_t>(tile[r][c]) << 16);
+  part[g][c] = s;
+  __syncthreads();
+  if (g == 0 && t0 + c < d_in)
+    zsum[static_cast<int64_t>(blockIdx.y) * d_in + t0 + c] =
+        (part[0][c] + part[1][c]) + (part[2][c] + part[3][c]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1651,7 +1661,7 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
 }
 
 fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq,
-                                 const void* T_out_t, int d_out, const float* gamma, void* y,
+                                 const void* T_out_t, int d_out, const float* gamma, void* W_hat,
                                  char* ws, size_t ws_bytes, cudaStream_t s) {
   const int M = d_in, n_in = Cq.n_in, n_out = Cq.n_out;
   const WsLayout L = ws_layout(M, d_in, n_in, n_out, d_out, 0);
@@ -1665,7 +1675,7 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
   PhaseArgs a[3];
   const int R[3] = {n_in, n_out, d_out};
   const int K[3] = {d_in, n_in, n_out};
-  __nv_bfloat16* outs[3] = {z, u, reinterpret_cast<__nv_bfloat16*>(y)};
+  __nv_bfloat16* outs[3] = {z, u, reinterpret_cast<__nv_bfloat16*>(W_hat)};
   for (int ph = 1; ph < 3; ++ph) {
     a[ph] = PhaseArgs{};
     a[ph].R = R[ph];
@@ -1681,6 +1691,7 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
   a[1].scale = reinterpret_cast<const __half*>(Cq.scale_f16);
   a[1].zero = reinterpret_cast<const __half*>(Cq.zero_f16);
   a[1].gamma = gamma;
+  a[2].transposed = 1;                           // the output's rows are those of W_hat
 
   // maps: z (the code product's B; also the unused A slot), T_out^T, u
   CUtensorMap maps[3];
@@ -1691,15 +1702,11 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
       !make_tmap(&maps[2], u, M, n_out, box))
     return FQ_ERR_CUDA;
 
-  unit_analysis_kernel<<<dim3(static_cast<unsigned>(ceil_div(d_in, 32)),
-                              static_cast<unsigned>(ceil_div(n_in, 32))),
-                         dim3(32, 8), 0, s>>>(Tin, n_in, d_in, z);
+  unit_analysis_kernel<<<dim3(static_cast<unsigned>(ceil_div(d_in, kUnitCols)),
+                              static_cast<unsigned>(ceil_div(n_in, kUnitRows))),
+                         256, 0, s>>>(Tin, n_in, d_in, z, zsum, status);
   if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
-  unit_zsum_kernel<<<static_cast<unsigned>(ceil_div(d_in, 32)), dim3(32, 32), 0, s>>>(
-      Tin, n_in, d_in, zsum, status);
-  if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
-  // the code product and the synthesis, with one sum of z per token
-  a[1].zsum_tiles = 1;
+  a[1].zsum_tiles = static_cast<int>(ceil_div(n_in, kUnitRows));
   return run_phase<kCore>(maps[0], maps[0], a[1], d, s) == cudaSuccess &&
                  run_phase<kSynthesis>(maps[1], maps[2], a[2], d, s) == cudaSuccess
              ? FQ_OK
