@@ -147,18 +147,17 @@ __global__ void eye_kernel(float* __restrict__ T, int d) {
     T[static_cast<int64_t>(i) * d + i] = 1.f;
 }
 
-// C[i][j] = sum_k A[i][k] * B[j][k] (+ C if accumulate), fp32, both operands K-contiguous,
-// batched over blockIdx.z with element strides. 64 x 64 tiles, 4 x 4 outputs per thread.
+// C[i][j] = sum_k A[i][k] * B[j][k], fp32, both operands K-contiguous.  Every element is one
+// chain of fused multiply-adds in ascending k (K padded with zeros to a multiple of kGK), whichever
+// kernel computes it, so the coefficients and the codes rounded from them do not depend on the
+// choice.  Small products: 64 x 64 tiles, 4 x 4 outputs per thread.
 constexpr int kGT = 64, kGK = 16;
 __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
                                                    const float* __restrict__ B,
-                                                   float* __restrict__ C, int64_t M, int N, int K,
-                                                   int64_t sA, int64_t sB, int64_t sC) {
+                                                   float* __restrict__ C, int64_t M, int N,
+                                                   int K) {
   __shared__ float As[kGK][kGT + 4];
   __shared__ float Bs[kGK][kGT + 4];
-  A += blockIdx.z * sA;
-  B += blockIdx.z * sB;
-  C += blockIdx.z * sC;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kGT;
   const int j0 = blockIdx.y * kGT;
@@ -194,11 +193,153 @@ __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
     }
 }
 
-cudaError_t gemm_nt(const float* A, const float* B, float* C, int64_t M, int N, int K, int batch,
-                    int64_t sA, int64_t sB, int64_t sC, cudaStream_t s) {
-  dim3 grid(static_cast<unsigned>(ceil_div(M, kGT)), static_cast<unsigned>(ceil_div(N, kGT)),
-            static_cast<unsigned>(batch));
-  gemm_nt_f32<<<grid, 256, 0, s>>>(A, B, C, M, N, K, sA, sB, sC);
+// Products that fill the GPU: 128 x kBN tiles, 8 x 8 outputs per thread as 32 packed pairs
+// (fma.rn.f32x2: two ordinary fused multiply-adds per instruction, which halves the issue slots
+// of a kernel that is bound by them), the next K slice in registers while the current one is
+// multiplied, two slices in shared memory (one barrier per slice).  Both operands are kept
+// k-major; a warp's 32 x 64 outputs read 4 + 8 distinct 16-byte groups per k, broadcast.
+// PLACEHOLDER_GEMM
+constexpr int kLBM = 128;
+constexpr int64_t kLargeMinBlocks = 100;
+
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+
+template <int kBN>
+__global__ void __launch_bounds__(2 * kBN, 256 / kBN) gemm_nt_f32_large(const float* __restrict__ A,
+                                                             const float* __restrict__ B,
+                                                             float* __restrict__ C, int64_t M,
+                                                             int N, int K, int vec) {
+  constexpr int kThreads = 2 * kBN;
+  constexpr int kLA = kLBM * kGK / 4 / kThreads, kLB = kBN * kGK / 4 / kThreads;   // float4 loads
+  __shared__ __align__(16) float As[2][kGK][kLBM + 4];
+  __shared__ __align__(16) float Bs[2][kGK][kBN + 4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kLBM;
+  const int j0 = blockIdx.y * kBN;
+  // a thread's rows: r0 .. + 3 and r0 + 16 .. + 19; columns: c0 .. + 3 and c0 + 32 .. + 35
+  const int r0 = (warp % 4) * 32 + (lane >> 3) * 4, c0 = (warp / 4) * 64 + (lane & 7) * 4;
+  uint64_t acc[8][4] = {};
+  float4 ra[kLA], rb[kLB];
+  // four consecutive k of one row of an operand, zero past its edges
+  auto load4 = [&](const float* X, int64_t row, int64_t rows, int k) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < rows) {
+      const float* src = X + row * K + k;
+      if (vec && k + 3 < K) {
+        v = __ldg(reinterpret_cast<const float4*>(src));
+      } else {
+        if (k < K) v.x = src[0];
+        if (k + 1 < K) v.y = src[1];
+        if (k + 2 < K) v.z = src[2];
+        if (k + 3 < K) v.w = src[3];
+      }
+    }
+    return v;
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int l = 0; l < kLA; ++l) {
+      const int e = tid + l * kThreads;
+      ra[l] = load4(A, i0 + e / 4, M, k0 + 4 * (e % 4));
+    }
+#pragma unroll
+    for (int l = 0; l < kLB; ++l) {
+      const int e = tid + l * kThreads;
+      rb[l] = load4(B, j0 + e / 4, N, k0 + 4 * (e % 4));
+    }
+  };
+  auto stash = [&](int buf) {
+#pragma unroll
+    for (int l = 0; l < kLA; ++l) {
+      const int e = tid + l * kThreads, r = e / 4, k = 4 * (e % 4);
+      As[buf][k][r] = ra[l].x;
+      As[buf][k + 1][r] = ra[l].y;
+      As[buf][k + 2][r] = ra[l].z;
+      As[buf][k + 3][r] = ra[l].w;
+    }
+#pragma unroll
+    for (int l = 0; l < kLB; ++l) {
+      const int e = tid + l * kThreads, r = e / 4, k = 4 * (e % 4);
+      Bs[buf][k][r] = rb[l].x;
+      Bs[buf][k + 1][r] = rb[l].y;
+      Bs[buf][k + 2][r] = rb[l].z;
+      Bs[buf][k + 3][r] = rb[l].w;
+    }
+  };
+  fetch(0);
+  stash(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < K; k0 += kGK) {
+    const bool more = k0 + kGK < K;
+    if (more) fetch(k0 + kGK);
+#pragma unroll
+    for (int kk = 0; kk < kGK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][r0]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][r0 + 16]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][c0]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][c0 + 32]);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const uint64_t b[4] = {pack2(b0.x, b0.y), pack2(b0.z, b0.w), pack2(b1.x, b1.y),
+                             pack2(b1.z, b1.w)};
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        const uint64_t ap = pack2(a[p], a[p]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = fma2(ap, b[q], acc[p][q]);
+      }
+    }
+    if (more) stash(buf ^ 1);
+    __syncthreads();
+    buf ^= 1;
+  }
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int64_t gi = i0 + r0 + (p < 4 ? p : p + 12);
+    if (gi >= M) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int gj = j0 + c0 + 32 * h;
+      const float2 lo = unpack2(acc[p][2 * h]), hi = unpack2(acc[p][2 * h + 1]);
+      float* dst = C + gi * N + gj;
+      if (gj < N) dst[0] = lo.x;
+      if (gj + 1 < N) dst[1] = lo.y;
+      if (gj + 2 < N) dst[2] = hi.x;
+      if (gj + 3 < N) dst[3] = hi.y;
+    }
+  }
+}
+
+cudaError_t gemm_nt(const float* A, const float* B, float* C, int64_t M, int N, int K,
+                    cudaStream_t s) {
+  // The large tiles need about a wave of blocks to win over four times as many small ones;
+  // N <= 64 (a rotation factor) takes 64 columns so that no half of a tile is idle.
+  const int bn = N <= 64 ? 64 : 128;
+  if (ceil_div(M, kLBM) * ceil_div(N, bn) >= kLargeMinBlocks) {
+    const int vec = K % 4 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+    const dim3 grid(static_cast<unsigned>(ceil_div(M, kLBM)), static_cast<unsigned>(ceil_div(N, bn)));
+    if (bn == 64)
+      gemm_nt_f32_large<64><<<grid, 128, 0, s>>>(A, B, C, M, N, K, vec);
+    else
+      gemm_nt_f32_large<128><<<grid, 256, 0, s>>>(A, B, C, M, N, K, vec);
+    return cudaGetLastError();
+  }
+  const dim3 grid(static_cast<unsigned>(ceil_div(M, kGT)), static_cast<unsigned>(ceil_div(N, kGT)));
+  gemm_nt_f32<<<grid, 256, 0, s>>>(A, B, C, M, N, K);
   return cudaGetLastError();
 }
 
@@ -397,10 +538,10 @@ fq_status fq_frame_build(int k, int rho, int d, const fq_rotation* rot, float* T
     return FQ_ERR_CUDA;
   // X = T D (buf0 -> T as scratch), Z = X Qb^T, Zt per row, Yt = Zt Qa^T, out = permuted Y
   sign_kernel<<<grid_for(total), 256, 0, s>>>(buf0, dSg, T, total, d);
-  cudaError_t e = gemm_nt(T, dQb, buf1, n * a, b, b, 1, 0, 0, 0, s);
+  cudaError_t e = gemm_nt(T, dQb, buf1, n * a, b, b, s);
   if (e != cudaSuccess) return FQ_ERR_CUDA;
   transpose_rows_kernel<<<grid_for(total), 256, 0, s>>>(buf1, buf0, total, a, b);
-  e = gemm_nt(buf0, dQa, buf1, n * b, a, a, 1, 0, 0, 0, s);
+  e = gemm_nt(buf0, dQa, buf1, n * b, a, a, s);
   if (e != cudaSuccess) return FQ_ERR_CUDA;
   permute_kernel<<<grid_for(total), 256, 0, s>>>(buf1, dPm, T, total, a, b);
   if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
@@ -421,8 +562,8 @@ fq_status fq_coefficients(const float* W, int d_out, int d_in, const float* T_in
   if (!ws || ws_bytes < fq_coefficients_workspace_bytes(d_out, n_in)) return FQ_ERR_WORKSPACE;
   auto s = reinterpret_cast<cudaStream_t>(stream);
   float* Pt = static_cast<float*>(ws);                    // Pt = T_in W^T  (n_in x d_out)
-  if (gemm_nt(T_in, W, Pt, n_in, d_out, d_in, 1, 0, 0, 0, s) != cudaSuccess) return FQ_ERR_CUDA;
-  if (gemm_nt(T_out, Pt, C, n_out, n_in, d_out, 1, 0, 0, 0, s) != cudaSuccess)   // C = T_out Pt^T
+  if (gemm_nt(T_in, W, Pt, n_in, d_out, d_in, s) != cudaSuccess) return FQ_ERR_CUDA;
+  if (gemm_nt(T_out, Pt, C, n_out, n_in, d_out, s) != cudaSuccess)   // C = T_out Pt^T
     return FQ_ERR_CUDA;
   return FQ_OK;
 }
