@@ -13,14 +13,20 @@
 //   3. the damped Hessian H + damp mean(diag H) I and the upper factor U of its inverse,
 //      H^-1 = U^T U.  With J the exchange matrix, J H J = L L^T (lower Cholesky) gives
 //      H = (J L J)(J L J)^T, so U = (J L J)^-1 = J L^-1 J: one Cholesky and one triangular
-//      inverse, no explicit inverse of H;
+//      inverse, no explicit inverse of H.  Both go by blocks of 32: a diagonal block is factored
+//      and inverted in one warp's registers, the rest is tiled products; the inverse doubles its
+//      blocks (32, 64, ...), X_21 = -X_22 (L_21 X_11);
 //   4. the columns in blocks of 128: column j of a block is rounded to each row's grid, its
 //      rounding error e = (w_j - q_hat_j) / U_jj is spread over the block's later columns
 //      (w_k -= e U_jk), and after the block over all later columns at once (a product with
 //      U's block rows).
-// W is held transposed (column j of every row contiguous) so that one thread per row reads and
-// writes coalesced.  Inside a block the update is one rounded multiply and one rounded subtract,
+// W is held transposed (column j of every row contiguous) so that consecutive rows are read and
+// written coalesced.  Inside a block the update is one rounded multiply and one rounded subtract,
 // as the plain recursion writes it.
+//
+// What bounds it: GB300's fp64 rate (about two multiply-adds per cycle and SM), so the products
+// are cut into tiles small enough to spread evenly over all SMs, and the two serial recursions
+// (the Cholesky's pivots, a row's 128 columns) keep their chains short.  PLACEHOLDER_GPTQ
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -34,59 +40,97 @@ namespace {
 
 constexpr int kBlockCols = 128;   // columns per block of the iteration
 constexpr int kT = 256;           // threads per block of the simple kernels
+constexpr int kMaxIn = 25600;     // the largest n_in taken
 
-// ---- fp64 tiled product: C[m][n] (+)= sum_k A(m, k) B(k, n), A and B given by element strides.
-constexpr int kGM = 64, kGN = 64, kGK = 16;
+// ---- fp64 tiled product: C[m][n] = op(sum_k A(m, k) B(k, n)), A and B given by element strides;
+// every element is one chain of fused multiply-adds in ascending k from zero.  32 x 32 tiles, 2 x
+// 2 outputs per thread: at the fp64 rate a tile's shared-memory reads are far below its
+// multiply-adds, and small tiles leave the last wave of blocks short.
+constexpr int kG = 32, kGK = 16;
+enum GemmOp : int { kSet = 0, kSub = 1, kNeg = 2 };        // C = sum, C - sum, -sum
+enum GemmTri : int { kFull = 0, kALower = 1, kAUpper = 2 };  // A(m, k) = 0 for k > m, k < m
 
-__global__ void __launch_bounds__(256) gemm_f64_kernel(
-    const double* __restrict__ A, int64_t a_m, int64_t a_k, const double* __restrict__ B,
-    int64_t b_k, int64_t b_n, double* __restrict__ C, int64_t ldc, int M, int N, int K,
-    int subtract) {
-  __shared__ double As[kGK][kGM + 1];
-  __shared__ double Bs[kGK][kGN + 1];
+struct GemmShape {
+  int64_t a_m, a_k, b_k, b_n, ldc;
+  int M, N, K;
+  int op, tri;
+  int lower;                        // only tiles on or below the diagonal
+  int mirror;                       // and their transposes are stored too
+};
+
+__device__ __forceinline__ void gemm_f64_tile(const double* __restrict__ A,
+                                              const double* __restrict__ B,
+                                              double* __restrict__ C, const GemmShape& g) {
+  __shared__ double As[kGK][kG + 1];
+  __shared__ double Bs[kGK][kG + 1];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int m0 = blockIdx.y * kGM, n0 = blockIdx.x * kGN;
-  double acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += kGK) {
-    for (int t = threadIdx.x; t < kGM * kGK; t += 256) {
-      // A: m fastest within a k row of the tile; B: n fastest
-      const int r = t % kGM, kk = t / kGM;
-      const int gm = m0 + r, gk = k0 + kk, gn = n0 + r;
-      As[kk][r] = (gm < M && gk < K) ? A[gm * a_m + gk * a_k] : 0.0;
-      Bs[kk][r] = (gn < N && gk < K) ? B[gk * b_k + gn * b_n] : 0.0;
+  const int m0 = blockIdx.y * kG, n0 = blockIdx.x * kG;
+  if (m0 >= g.M || n0 >= g.N || (g.lower && m0 < n0)) return;
+  const int k_lo = g.tri == kAUpper ? m0 : 0;
+  const int k_hi = g.tri == kALower ? min(g.K, m0 + kG) : g.K;
+  // a thread's two elements of each operand slice, consecutive threads along the contiguous side
+  int am[2], ak[2], bn[2], bk[2];
+#pragma unroll
+  for (int l = 0; l < 2; ++l) {
+    const int t = threadIdx.x + 256 * l;
+    am[l] = g.a_m == 1 ? t % kG : t / kGK;
+    ak[l] = g.a_m == 1 ? t / kG : t % kGK;
+    bn[l] = g.b_n == 1 ? t % kG : t / kGK;
+    bk[l] = g.b_n == 1 ? t / kG : t % kGK;
+  }
+  double acc[2][2] = {}, ra[2], rb[2];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      ra[l] = (m0 + am[l] < g.M && k0 + ak[l] < k_hi)
+                  ? A[(m0 + am[l]) * g.a_m + (k0 + ak[l]) * g.a_k] : 0.0;
+      rb[l] = (n0 + bn[l] < g.N && k0 + bk[l] < k_hi)
+                  ? B[(k0 + bk[l]) * g.b_k + (n0 + bn[l]) * g.b_n] : 0.0;
+    }
+  };
+  fetch(k_lo);
+  for (int k0 = k_lo; k0 < k_hi; k0 += kGK) {
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      As[ak[l]][am[l]] = ra[l];
+      Bs[bk[l]][bn[l]] = rb[l];
     }
     __syncthreads();
+    if (k0 + kGK < k_hi) fetch(k0 + kGK);
 #pragma unroll
     for (int kk = 0; kk < kGK; ++kk) {
-      double a[4], b[4];
+      const double a[2] = {As[kk][ty], As[kk][ty + 16]}, b[2] = {Bs[kk][tx], Bs[kk][tx + 16]};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = As[kk][ty + 16 * q], b[q] = Bs[kk][tx + 16 * q];
+      for (int p = 0; p < 2; ++p)
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+        for (int q = 0; q < 2; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
+  for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       const int gm = m0 + ty + 16 * p, gn = n0 + tx + 16 * q;
-      if (gm < M && gn < N) {
-        double* c = C + gm * ldc + gn;
-        *c = subtract ? *c - acc[p][q] : acc[p][q];
+      if (gm < g.M && gn < g.N) {
+        double* c = C + gm * g.ldc + gn;
+        *c = g.op == kSub ? *c - acc[p][q] : (g.op == kNeg ? -acc[p][q] : acc[p][q]);
+        if (g.mirror && m0 > n0) C[gn * g.ldc + gm] = acc[p][q];
       }
     }
 }
 
-cudaError_t gemm_f64(const double* A, int64_t a_m, int64_t a_k, const double* B, int64_t b_k,
-                     int64_t b_n, double* C, int64_t ldc, int M, int N, int K, bool subtract,
+__global__ void __launch_bounds__(256) gemm_f64_kernel(const double* __restrict__ A,
+                                                       const double* __restrict__ B,
+                                                       double* __restrict__ C, GemmShape g) {
+  gemm_f64_tile(A, B, C, g);
+}
+
+cudaError_t gemm_f64(const double* A, const double* B, double* C, const GemmShape& g,
                      cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  const dim3 grid(static_cast<unsigned>(ceil_div(N, kGN)), static_cast<unsigned>(ceil_div(M, kGM)));
-  gemm_f64_kernel<<<grid, 256, 0, s>>>(A, a_m, a_k, B, b_k, b_n, C, ldc, M, N, K,
-                                       subtract ? 1 : 0);
+  if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  const dim3 grid(static_cast<unsigned>(ceil_div(g.N, kG)), static_cast<unsigned>(ceil_div(g.M, kG)));
+  gemm_f64_kernel<<<grid, 256, 0, s>>>(A, B, C, g);
   return cudaGetLastError();
 }
 
@@ -223,85 +267,157 @@ __global__ void damp_reverse_kernel(const double* __restrict__ H, int n, double 
   }
 }
 
-// Right-looking Cholesky, step j: K[i][k] -= K[i][j] K[k][j] / K[j][j] for j < k <= i.  The
-// columns are scaled at the end (L[i][j] = K[i][j] / sqrt(K[j][j])).
-__global__ void chol_step_kernel(double* __restrict__ K, int n, int j) {
-  const int k = j + 1 + blockIdx.x * 16 + threadIdx.x;
-  const int i = j + 1 + blockIdx.y * 16 + threadIdx.y;
-  if (k >= n || i >= n || k > i) return;
-  const double piv = K[static_cast<int64_t>(j) * n + j];
-  K[static_cast<int64_t>(i) * n + k] -=
-      K[static_cast<int64_t>(i) * n + j] * K[static_cast<int64_t>(k) * n + j] / piv;
-}
+// ---- blocked right-looking Cholesky of K (lower triangle) with the inverses of its diagonal blocks
+constexpr int kNB = 32;           // block: a warp's lanes
 
-// L[i][j] = K[i][j] / sqrt(K[j][j]) below the diagonal (the diagonal itself is replaced by the
-// next kernel, so every pivot is read here unchanged); a pivot that is not positive means the
-// damped H was not positive definite
-__global__ void chol_scale_kernel(double* __restrict__ K, int n, int32_t* __restrict__ status) {
-  const int64_t total = static_cast<int64_t>(n) * n;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(kT) + threadIdx.x; e < total;
-       e += static_cast<int64_t>(gridDim.x) * kT) {
-    const int i = static_cast<int>(e / n), j = static_cast<int>(e % n);
-    const double piv = K[static_cast<int64_t>(j) * n + j];
-    if (i == j && !(piv > 0.0)) report(status, FQ_ERR_DEVICE_CHECK);
-    if (j < i) K[e] = K[e] / sqrt(piv);
+// Block column b .. b + nb - 1: factor the diagonal block, K_bb = L L^T, and solve L Y = B by forward
+// substitution, a column of B per lane: CTA 0 for B = I, the inverse of L, which goes to X; CTA c > 0
+// for B = the transpose of 32 rows below the block, K_ib <- K_ib L^-T in place.  Every CTA factors
+// the diagonal block for itself (one warp, a row per lane: a pivot's chain is a division and the
+// row's multiply-adds, no barriers), which saves a launch and its latency per block; nothing
+// rewrites the diagonal block.  Loops stay rolled: unrolled code runs once per launch and waits
+// for its instructions.
+__global__ void __launch_bounds__(256) chol_panel_kernel(double* __restrict__ K, int n, int b,
+                                                         int nb, double* __restrict__ X,
+                                                         int32_t* __restrict__ status) {
+  __shared__ double D[kNB][kNB + 1];      // the block, then its factor
+  __shared__ double Y[kNB][kNB + 1];      // the right-hand sides, a column per lane
+  __shared__ double inv_s[kNB];
+  const int tid = threadIdx.x, lane = tid & 31, wr = tid >> 5;
+  const bool inverse = blockIdx.x == 0;
+  const int r0 = b + nb + (static_cast<int>(blockIdx.x) - 1) * kNB;   // this CTA's rows
+  for (int e = tid; e < kNB * kNB; e += 256) {
+    const int i = e / kNB, j = e % kNB;
+    // past nb: the identity, so that a short last block needs no case of its own
+    D[i][j] = i < nb ? (j <= i ? K[static_cast<int64_t>(b + i) * n + b + j] : 0.0)
+                     : (i == j ? 1.0 : 0.0);
+    if (inverse)
+      Y[i][j] = i == j ? 1.0 : 0.0;
+    else
+      Y[j][i] = (r0 + i < n && j < nb) ? K[static_cast<int64_t>(r0 + i) * n + b + j] : 0.0;
   }
-}
-
-__global__ void chol_diag_kernel(double* __restrict__ K, int n) {
-  for (int j = blockIdx.x * kT + threadIdx.x; j < n; j += gridDim.x * kT)
-    K[static_cast<int64_t>(j) * n + j] = sqrt(K[static_cast<int64_t>(j) * n + j]);
-}
-
-// X = L^-1 (lower), one block per column c: x_c = 1 / L_cc, x_i = -(sum_{c<=k<i} L_ik x_k) / L_ii.
-// Written straight into U = J X J: U[n-1-i][n-1-c] = X[i][c].
-__global__ void __launch_bounds__(kT) tri_inverse_kernel(const double* __restrict__ L, int n,
-                                                         double* __restrict__ U) {
-  extern __shared__ double xs[];                 // x_c .. x_{n-1}
-  __shared__ double red[kT];
-  const int c = blockIdx.x;
-  if (threadIdx.x == 0) xs[0] = 1.0 / L[static_cast<int64_t>(c) * n + c];
   __syncthreads();
-  for (int i = c + 1; i < n; ++i) {
-    const double* Li = L + static_cast<int64_t>(i) * n;
-    double s = 0.0;
-    for (int k = c + threadIdx.x; k < i; k += kT) s += Li[k] * xs[k - c];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = kT / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-      __syncthreads();
+  if (tid < 32) {
+    // right-looking, unscaled: D_ik -= D_ij D_kj / piv_j
+    for (int j = 0; j < kNB; ++j) {
+      const double m = D[lane][j] * (1.0 / D[j][j]);
+#pragma unroll 4
+      for (int k = j + 1; k < kNB; ++k)
+        if (lane >= k) D[lane][k] = fma(-m, D[k][j], D[lane][k]);
+      __syncwarp();
     }
-    if (threadIdx.x == 0) xs[i - c] = -red[0] / Li[i];
+    // a pivot that is not positive: the damped H was not positive definite
+    const double piv = D[lane][lane];
+    if (inverse && !(piv > 0.0)) report(status, FQ_ERR_DEVICE_CHECK);
+    inv_s[lane] = 1.0 / sqrt(piv);
+  }
+  __syncthreads();
+  // columns scaled: L_ij = D_ij / sqrt(piv_j)
+  for (int i = wr; i < kNB; i += 8)
+    if (lane <= i) D[i][lane] *= inv_s[lane];
+  __syncthreads();
+  // x_k = y_k / L_kk, then y_i -= L_ik x_k for every later row i, the rows split over the warps
+  // (y_k itself is left to the end, so that a row costs one barrier)
+  for (int k = 0; k < kNB; ++k) {
+    const double x = Y[k][lane] * inv_s[k];
+    for (int i = wr; i < kNB; i += 8)
+      if (i > k) Y[i][lane] = fma(-D[i][k], x, Y[i][lane]);
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n; i += kT) {
-    const double x = i < c ? 0.0 : xs[i - c];
-    U[static_cast<int64_t>(n - 1 - i) * n + (n - 1 - c)] = x;
+  for (int e = tid; e < kNB * kNB; e += 256) {
+    const int i = e / kNB, j = e % kNB;
+    if (inverse) {
+      if (i < nb && j < nb)
+        X[static_cast<int64_t>(b + i) * n + b + j] = j <= i ? Y[i][j] * inv_s[i] : 0.0;
+    } else if (r0 + i < n && j < nb) {
+      K[static_cast<int64_t>(r0 + i) * n + b + j] = Y[j][i] * inv_s[j];
+    }
   }
 }
 
-// Block b0 .. b1-1 of the iteration, one thread per row i of W (WT column i).
-__global__ void __launch_bounds__(kT) gptq_block_kernel(double* __restrict__ WT, int n_out,
+// One doubling of the inverse for all pairs of s x s blocks (blockIdx.z = pair): T = L_21 X_11, kept
+// transposed in the upper triangle of L's matrix, which nothing else uses (step 0), then
+// X_21 = -X_22 T (step 1).
+__global__ void __launch_bounds__(256) tri_double_kernel(double* __restrict__ L,
+                                                         double* __restrict__ X, int n, int s,
+                                                         int step) {
+  const int o = 2 * s * blockIdx.z, rows = min(s, n - o - s);   // rows of the lower block
+  if (rows <= 0) return;
+  const int64_t at = static_cast<int64_t>(o) * n + o, below = static_cast<int64_t>(s) * n;
+  double* Tt = L + at + s;                                      // Tt[c][r] = T[r][c], s x rows
+  const int64_t N = n;
+  if (step == 0)   // Tt[c][r] = sum_{k >= c} X_11[k][c] L_21[r][k]
+    gemm_f64_tile(X + at, L + at + below, Tt,
+                  GemmShape{1, N, 1, N, N, s, rows, s, kSet, kAUpper, 0, 0});
+  else             // X_21[r][c] = -sum_{k <= r} X_22[r][k] Tt[c][k]
+    gemm_f64_tile(X + at + below + s, Tt, X + at + below,
+                  GemmShape{N, 1, 1, N, N, rows, s, rows, kNeg, kALower, 0, 0});
+}
+
+// U = J X J in place: the n^2 entries in reverse order.
+__global__ void reverse_kernel(double* __restrict__ X, int64_t total) {
+  for (int64_t e = blockIdx.x * static_cast<int64_t>(kT) + threadIdx.x; e < total / 2;
+       e += static_cast<int64_t>(gridDim.x) * kT) {
+    const double lo = X[e], hi = X[total - 1 - e];
+    X[e] = hi;
+    X[total - 1 - e] = lo;
+  }
+}
+
+// Block b0 .. b1-1 of the iteration.  A CTA keeps `rows` rows of the block's columns and the
+// block of U in shared memory.  Warp 0 carries the serial chain, a row per lane: column j with the
+// last error e_(j-1) applied, rounded, its error e_j.  Meanwhile the other warps apply e_(j-1) to
+// the columns after j, so every element takes the errors in ascending order, and the chain of
+// one column costs one barrier.
+constexpr int kIterRows = 32;     // most rows per CTA
+constexpr int kIterSmem = (kBlockCols * kBlockCols + kIterRows * (kBlockCols + 1) + 2 * kIterRows) * 8;
+
+__global__ void __launch_bounds__(kT) gptq_block_kernel(const double* __restrict__ WT, int n_out,
                                                         int n_in, const double* __restrict__ U,
                                                         const double* __restrict__ s64,
                                                         const double* __restrict__ z64, int b0,
-                                                        int b1, uint8_t* __restrict__ codesT,
+                                                        int b1, int rows,
+                                                        uint8_t* __restrict__ codesT,
                                                         double* __restrict__ ET) {
-  const int i = blockIdx.x * kT + threadIdx.x;
-  if (i >= n_out) return;
+  extern __shared__ double iter_smem[];
+  double(*Us)[kBlockCols] = reinterpret_cast<double(*)[kBlockCols]>(iter_smem);
+  double(*W)[kBlockCols + 1] =
+      reinterpret_cast<double(*)[kBlockCols + 1]>(iter_smem + kBlockCols * kBlockCols);
+  double* E = iter_smem + kBlockCols * kBlockCols + kIterRows * (kBlockCols + 1);   // [2][rows]
+  const int nb = b1 - b0, i0 = blockIdx.x * rows, nr = min(rows, n_out - i0);
+  const int tid = threadIdx.x;
+  for (int e = tid; e < nb * nb; e += kT) {
+    const int j = e / nb, k = e % nb;
+    if (k >= j) Us[j][k] = U[static_cast<int64_t>(b0 + j) * n_in + b0 + k];
+  }
+  for (int e = tid; e < nb * nr; e += kT) {
+    const int j = e / nr, r = e % nr;
+    W[r][j] = WT[static_cast<int64_t>(b0 + j) * n_out + i0 + r];
+  }
+  __syncthreads();
+  const bool chain = tid < 32 && tid < nr;
+  const int i = i0 + (chain ? tid : 0);
   const double s = s64[i], z = z64[i];
-  for (int j = b0; j < b1; ++j) {
-    const double w = WT[static_cast<int64_t>(j) * n_out + i];
-    const double q = fmin(fmax(rint((w - z) / s), 0.0), 3.0);
-    codesT[static_cast<int64_t>(j) * n_out + i] = static_cast<uint8_t>(q);
-    const double* Uj = U + static_cast<int64_t>(j) * n_in;
-    const double e = (w - __dadd_rn(__dmul_rn(s, q), z)) / Uj[j];
-    ET[static_cast<int64_t>(j - b0) * n_out + i] = e;
-    for (int k = j + 1; k < b1; ++k) {
-      double* wk = WT + static_cast<int64_t>(k) * n_out + i;
-      *wk = __dsub_rn(*wk, __dmul_rn(e, Uj[k]));
+  double e_prev = 0.0;
+  // the other warps: row r, columns in steps of ncg
+  const int t = tid - 32, r = t >= 0 ? t % nr : 0, cg = t >= 0 ? t / nr : 0, ncg = (kT - 32) / nr;
+  const bool bulk = t >= 0 && cg < ncg;
+  for (int j = 0; j < nb; ++j) {
+    if (chain) {
+      double w = W[tid][j];
+      if (j > 0) w = __dsub_rn(w, __dmul_rn(e_prev, Us[j - 1][j]));
+      const double q = fmin(fmax(rint((w - z) / s), 0.0), 3.0);
+      const double e = (w - __dadd_rn(__dmul_rn(s, q), z)) / Us[j][j];
+      E[(j & 1) * kIterRows + tid] = e;
+      e_prev = e;
+      codesT[static_cast<int64_t>(b0 + j) * n_out + i] = static_cast<uint8_t>(q);
+      ET[static_cast<int64_t>(j) * n_out + i] = e;
+    } else if (bulk && j > 0) {
+      const double e = E[((j - 1) & 1) * kIterRows + r];
+      for (int k = j + 1 + cg; k < nb; k += ncg)
+        W[r][k] = __dsub_rn(W[r][k], __dmul_rn(e, Us[j - 1][k]));
     }
+    __syncthreads();
   }
 }
 
@@ -364,7 +480,9 @@ fq_status fq_gptq_hessian(const double* Z, int N, int n_in, double* H, fq_stream
   if (!Z || !H || N <= 0 || n_in <= 0) return FQ_ERR_INVALID_ARG;
   if (!a8(Z) || !a8(H)) return FQ_ERR_ALIGNMENT;
   // H[i][j] = sum_t Z[t][i] Z[t][j]: A(i, t) = Z[t n_in + i], B(t, j) = Z[t n_in + j]
-  return gemm_f64(Z, 1, n_in, Z, n_in, 1, H, n_in, n_in, n_in, N, false,
+  // (symmetric: the same chains of multiply-adds, so half of the tiles are computed)
+  const int64_t ld = n_in;
+  return gemm_f64(Z, Z, H, GemmShape{1, ld, ld, 1, ld, n_in, n_in, N, kSet, kFull, 1, 1},
                   reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess
              ? FQ_OK
              : FQ_ERR_CUDA;
@@ -387,6 +505,7 @@ fq_status fq_quantize_gptq(const double* C, int n_out, int n_in, const double* H
   if ((reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return FQ_ERR_ALIGNMENT;
   const GptqWs L = gptq_ws(n_out, n_in);
   if (ws_bytes < L.total) return FQ_ERR_WORKSPACE;
+  if (n_in > kMaxIn) return FQ_ERR_UNSUPPORTED;
   auto s = reinterpret_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   auto* status = reinterpret_cast<int32_t*>(w + L.status);
@@ -418,29 +537,43 @@ fq_status fq_quantize_gptq(const double* C, int n_out, int n_in, const double* H
       z64, gamma);
   // 3. U with H^-1 = U^T U
   damp_reverse_kernel<<<grid_cap(nH), kT, 0, s>>>(H, n_in, damp, K);
-  for (int j = 0; j + 1 < n_in; ++j) {
-    const int t = n_in - j - 1;
-    const dim3 g(static_cast<unsigned>(ceil_div(t, 16)), static_cast<unsigned>(ceil_div(t, 16)));
-    chol_step_kernel<<<g, dim3(16, 16), 0, s>>>(K, n_in, j);
+  if (cudaMemsetAsync(U, 0, static_cast<size_t>(nH) * 8, s) != cudaSuccess) return FQ_ERR_CUDA;
+  const int64_t ld = n_in;
+  for (int b = 0; b < n_in; b += kNB) {
+    const int nb = std::min(kNB, n_in - b), below = n_in - b - nb;
+    chol_panel_kernel<<<static_cast<unsigned>(1 + ceil_div(below, kNB)), 256, 0, s>>>(
+        K, n_in, b, nb, U, status);
+    // K_ik -= L_ib L_kb^T for the rows and columns below the block, lower triangle
+    const double* P = K + (b + nb) * ld + b;
+    if (gemm_f64(P, P, K + (b + nb) * ld + b + nb,
+                 GemmShape{ld, 1, 1, ld, ld, below, below, nb, kSub, kFull, 1, 0},
+                 s) != cudaSuccess)
+      return FQ_ERR_CUDA;
   }
-  chol_scale_kernel<<<grid_cap(nH), kT, 0, s>>>(K, n_in, status);
-  chol_diag_kernel<<<grid_cap(n_in), kT, 0, s>>>(K, n_in);
-  const size_t xs_bytes = static_cast<size_t>(n_in) * 8;
-  if (xs_bytes > 200 * 1024) return FQ_ERR_UNSUPPORTED;
-  if (xs_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(tri_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(xs_bytes)) != cudaSuccess)
+  for (int w32 = kNB; w32 < n_in; w32 *= 2) {
+    const dim3 g(static_cast<unsigned>(w32 / kG), static_cast<unsigned>(w32 / kG),
+                 static_cast<unsigned>(ceil_div(n_in, 2 * w32)));
+    tri_double_kernel<<<g, 256, 0, s>>>(K, U, n_in, w32, 0);
+    tri_double_kernel<<<g, 256, 0, s>>>(K, U, n_in, w32, 1);
+  }
+  reverse_kernel<<<grid_cap(nH / 2), kT, 0, s>>>(U, nH);
+  // 4. the columns, block by block; the rows spread evenly over the SMs
+  if (cudaFuncSetAttribute(gptq_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           kIterSmem) != cudaSuccess)
     return FQ_ERR_CUDA;
-  tri_inverse_kernel<<<static_cast<unsigned>(n_in), kT, xs_bytes, s>>>(K, n_in, U);
-  // 4. the columns, block by block
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return FQ_ERR_CUDA;
+  const int64_t waves = ceil_div(n_out, static_cast<int64_t>(kIterRows) * sms);
+  const int rows = static_cast<int>(std::max<int64_t>(1, ceil_div(n_out, waves * sms)));
   for (int b0 = 0; b0 < n_in; b0 += kBlockCols) {
     const int b1 = std::min(n_in, b0 + kBlockCols);
-    gptq_block_kernel<<<static_cast<unsigned>(ceil_div(n_out, kT)), kT, 0, s>>>(
-        WT, n_out, n_in, U, s64, z64, b0, b1, codesT, ET);
+    gptq_block_kernel<<<static_cast<unsigned>(ceil_div(n_out, rows)), kT, kIterSmem, s>>>(
+        WT, n_out, n_in, U, s64, z64, b0, b1, rows, codesT, ET);
     // WT[k][i] -= sum_jj U[b0 + jj][k] ET[jj][i] for k >= b1
-    if (b1 < n_in &&
-        gemm_f64(U + static_cast<int64_t>(b0) * n_in + b1, 1, n_in, ET, n_out, 1,
-                 WT + static_cast<int64_t>(b1) * n_out, n_out, n_in - b1, n_out, b1 - b0, true,
+    if (gemm_f64(U + b0 * ld + b1, ET, WT + static_cast<int64_t>(b1) * n_out,
+                 GemmShape{1, ld, n_out, 1, n_out, n_in - b1, n_out, b1 - b0, kSub, kFull, 0, 0},
                  s) != cudaSuccess)
       return FQ_ERR_CUDA;
   }
