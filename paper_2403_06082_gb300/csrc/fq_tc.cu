@@ -138,15 +138,6 @@ __device__ __forceinline__ void decode_row(const uint4 w4, uint8_t* tile, int r)
   }
 }
 
-// 16 bytes of global memory that no kernel of the chain writes, not kept in L1.
-__device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-
 __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
   uint32_t out;
   asm volatile(
@@ -786,7 +777,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
   cluster_sync();       // both CTAs' barriers and TMEM exist before either signals the other
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
+  // (Not from the kernel that writes a rebuilt weight: the next kernel may be one of this library
+  // that reads the weight as its A operand before its own wait.)
+  if (!p.transposed) pdl_launch_dependents();
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
