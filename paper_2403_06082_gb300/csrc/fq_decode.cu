@@ -24,16 +24,23 @@
 // next tasks (and warms L2 with this CTA's later code blocks, and with its synthesis tiles when
 // the layer is small enough) while activations are still being produced.
 //
-// sum(z), needed by the core's zero term, is taken by the core's epilogue over the bf16 z of its
-// own K range, read from global memory once the slices' ready flags are seen (this runs while
-// the task's MMAs are in flight, and keeps the analysis epilogue, which every core task waits
-// for, short).
+// sum(z), needed by the core's zero term: in launches whose core tasks have more than
+// kSumMmaBlocks K blocks per CTA it comes from the tensor cores (kSums), whose core rounds issue
+// their MMAs once more with a constant A tile of ones, into columns beside the accumulator, so
+// that every accumulator row also holds the token sums over the CTA's K range.  Shorter tasks
+// take it in the epilogue over the bf16 z of their K range, read from global memory once the
+// slices' ready flags are seen, which costs them less than the extra MMAs and accumulator reads.
+// The two are separate kernels: a small launch is bound by latency, and carrying the other's
+// code cost it 2-8%.  Measured, us per call (epilogue sums, tensor-core sums): 4096 x 4096 at 24
+// tokens 30.4, 28.4; 11008 x 4096 at 48 tokens 97.3, 84.7; q|k|v at 16 tokens 51.1, 48.2; with 8 K
+// blocks per CTA at 34 tokens 35.1, 37.0.
 //
 // The workspace header holds the generation counter and the tiles' ready flags; a zero-filled
 // header is a valid start and every call leaves it valid for the next (flags keep
 // generations that are all in the past; the last CTA to finish advances the generation).
 //
 // Warps: 0 weight (A) producer, 1 TMEM owner + MMA issuer 0, 2-5 epilogue (thread = tile row),
+// 11 the tile of ones,
 // 6 activation (B) producer, 7-10 code decoders (ring stage s -> decoder s mod 4; one per SM
 // sub-partition, since the decode is issue-bound), and for 16 or 32 tokens 12, 14, 15 MMA
 // issuers 1-3 (one issuer per SM sub-partition).
@@ -43,8 +50,9 @@
 // every one of its phases that follows a phase they wait for:
 //   empty[s]  (the round's MMAs completed)  the weight and the activation producers, which
 //             both fill every round of the stage;
-//   cfull[s]  (a core round's code block landed)  decoder s mod 4, whose arrival on fullA[s]
-//             the round's MMAs (and so the next code load into the stage) wait for;
+//   cfull[s]  (a core round has the stage: the weight producer saw it empty)  decoder s mod 4,
+//             whose arrival on fullA[s] the round's MMAs (and so the stage's next core round)
+//             wait for;
 //   fullA[s]  (the A tile is in place: the weight tile's bytes, or the decoder's arrival in
 //             core rounds), fullB[s]  the issuer that owns s, which commits empty[s].
 #include <cuda.h>
@@ -66,7 +74,7 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kBK = 64;
 constexpr int kATile = kBM * kBK * 2;      // 16 KiB
-constexpr int kCodeBytes = kBM * kBK / 4;  // 2 KiB
+constexpr int kCodeBytes = kBM * kBK / 4;  // 2 KiB of packed codes per K block
 constexpr int kMaxSplit = 8;
 static_assert(kMaxSplit <= kWsSlices, "one ready flag per slice");
 constexpr int kEpi = 128;
@@ -154,38 +162,43 @@ struct DecSched {
   uint16_t task[kMaxSched];          // layer << 14 | phase << 12 | row tile
 };
 
-template <int BN>
+template <int BN, bool kSums>
 struct DecLayout {
   static constexpr int kBTile = BN * kBK * 2;
-  static constexpr int kStage = kATile + kBTile + kCodeBytes;
+  static constexpr int kStage = kATile + kBTile;
   static constexpr int kRecvRow = BN + 4;                     // floats per received row
   static constexpr int kRecv = kBM * kRecvRow * 4;            // [S][128/S][BN + 4] fp32
   static constexpr int NI = DecCfg<BN>::NI;
   // a multiple of NI: issuer q owns stages q, q + NI, ...
   static constexpr int kStages =
-      std::min(12, (216 * 1024 - 4096 - 2 * kRecv) / kStage) / NI * NI;
-  static constexpr int kAccCols = 2 * NI * BN;               // [2 buffers][NI issuers][BN]
-  static constexpr uint32_t kTmemCols =
-      kAccCols <= 32 ? 32 : (kAccCols <= 64 ? 64 : (kAccCols <= 128 ? 128 : 256));
+      std::min(12, (227 * 1024 - 5120 - 2 * kRecv - (kSums ? kATile : 0)) / kStage) / NI * NI;
+  // accumulators [2 buffers][NI issuers][BN], then (kSums) the core's sums of z likewise
+  static constexpr int kSumCol = 2 * NI * BN;
+  static constexpr int kAccCols = (kSums ? 2 : 1) * kSumCol;
+  static constexpr uint32_t kTmemCols = kAccCols <= 128 ? 128 : (kAccCols <= 256 ? 256 : 512);
   static constexpr int oA = 0;
   static constexpr int oB = oA + kStages * kATile;
-  static constexpr int oC = oB + kStages * kBTile;
-  static constexpr int oRecv = oC + kStages * kCodeBytes;    // two receive buffers
+  static constexpr int oOnes = oB + kStages * kBTile;        // kSums: an A tile of ones
+  static constexpr int oRecv = oOnes + (kSums ? kATile : 0);   // two receive buffers
   static constexpr int oBar = oRecv + 2 * kRecv;
-  static constexpr int kBars = 4 * kStages + 10;
+  static constexpr int kBars = 4 * kStages + 11;
   static constexpr int oMisc = oBar + kBars * 8;
   static constexpr int oZs = oMisc + 32;                     // [BN] floats
   static constexpr int oZsPart = oZs + BN * 4;               // [128] floats
   static constexpr int kBytes = oZsPart + kEpi * 4 + 1024;
   static_assert(kBTile % 1024 == 0, "B tiles keep 1024-byte alignment");
   static_assert(kStages >= 3 && kStages % NI == 0, "pipeline depth, stage ownership");
-  static_assert(kAccCols <= 256, "accumulator columns");
+  static_assert(kAccCols <= 512, "accumulator columns");
   static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
 };
 
 __device__ __forceinline__ uint4 ldcg_u4(const __nv_bfloat16* p) {
   return __ldcg(reinterpret_cast<const uint4*>(p));
 }
+
+// Launches whose core tasks have more than this many K blocks per CTA take sum(z) from the tensor
+// cores (kSums).
+constexpr int kSumMmaBlocks = 8;
 
 struct Task {
   int l, p, tile;
@@ -254,11 +267,11 @@ __device__ __forceinline__ void note_timeout(int32_t* status, int role, int task
   }
 }
 
-template <int BN>
+template <int BN, bool kSums>
 __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
     decode_layer_kernel(const __grid_constant__ DecMaps maps, const __grid_constant__ DecArgs a,
                         const __grid_constant__ DecSched sched) {
-  using Lo = DecLayout<BN>;
+  using Lo = DecLayout<BN, kSums>;
   constexpr int S_ = Lo::kStages;
   constexpr int kBTile = Lo::kBTile;
   constexpr int NI = Lo::NI;
@@ -268,7 +281,6 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sA = smem + Lo::oA;
   uint8_t* sB = smem + Lo::oB;
-  uint8_t* sC = smem + Lo::oC;
   float* recv_buf = reinterpret_cast<float*>(smem + Lo::oRecv);
   // fullA, fullB and empty complete once in every round of their stage, cfull[s] in core
   // rounds only (its waiters keep one parity bit per stage)
@@ -280,13 +292,15 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
   uint64_t* tempty = tfull + 2;
   uint64_t* mma_done = tempty + 2;     // [4] one per issuer
   uint64_t* recv_bar = mma_done + 4;   // [2] the peers' partials of this CTA's slice arrived
+  uint64_t* ones_bar = recv_bar + 2;   // the tile of ones is written
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Lo::oMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* gen_s = tmem_slot + 2;
   float* zs_s = reinterpret_cast<float*>(smem + Lo::oZs);
   float* zs_part = reinterpret_cast<float*>(smem + Lo::oZsPart);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);   // uniform
+  const int lane = threadIdx.x & 31;
   const int S = a.S;
   const bool clustered = S > 1;
   uint32_t rank = 0, cid = blockIdx.x, ncl = gridDim.x;
@@ -300,7 +314,7 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
 
   if (warp == 0) {
     // the barriers, initialised lane-parallel: fullA, fullB, empty, cfull (count 1), tfull[2]
-    // (one commit per issuer), tempty[2] (kEpi), mma_done[4] (1), recv_bar[2] (1)
+    // (one commit per issuer), tempty[2] (kEpi), mma_done[4] (1), recv_bar[2] (1), ones_bar (1)
     // fullA takes two arrivals per round when a stage has two decoders: the weight
     // producer's two (with the tile's bytes), or one from each decoder
     constexpr uint32_t kFullA = DecCfg<BN>::kPairs ? 2u : 1u;
@@ -374,15 +388,13 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
                        "r"(static_cast<uint32_t>(b1 - o < 65536 ? b1 - o : 65536))
                        : "memory");
       };
-      // bit s: stage s filled / its last fill a code block / parity of that fill's phase of
-      // fullA (weight tile) or cfull (code block)
-      uint32_t used = 0, last_code = 0, last_par = 0, cpar = 0;
+      // bit s: stage s's last fill was a weight tile / parity of that fill's phase of fullA
+      uint32_t used = 0, last_par = 0;
       bool wok = true;
       for (int i = t_lo; i < t_hi && wok; ++i) {
         if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
         const Task t = task_at(sched, i);
         const DecPhase ph = phase_of(a, t.l, t.p);
-        const uint32_t* words = a.L[t.l].words;
         const CUtensorMap* tmA = &maps.m[t.l][t.p == 0 ? kMapTin : kMapTout];
         int k0, k1;
         krange(ph, t.tile, k0, k1);
@@ -428,17 +440,10 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
             break;
           }
           const uint32_t bit = 1u << stage;
-          used |= bit;
           if (t.p == 1) {
-            if (lane == 0) {
-              mbar_arrive_expect_tx(&cfull[stage], kCodeBytes);
-              bulk_load(sC + stage * kCodeBytes,
-                        words + (static_cast<int64_t>(t.tile) * ph.KB + kb) * 512,
-                        kCodeBytes, &cfull[stage], pol_w);
-            }
-            last_code |= bit;
-            last_par = (last_par & ~bit) | (cpar & bit);
-            cpar ^= bit;
+            // the stage is free: its decoder may write the A tile
+            if (lane == 0) mbar_arrive(&cfull[stage]);
+            used &= ~bit;
           } else {
             if (lane == 0) {
               mbar_arrive_expect_tx(&fullA[stage], kATile);
@@ -451,7 +456,7 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
                 tma_load_2d(sA + stage * kATile, tmA, &fullA[stage], kb * kBK, t.tile * kBM,
                             pol_w);
             }
-            last_code &= ~bit;
+            used |= bit;
             last_par = (last_par & ~bit) | (phase << stage);
           }
           if (++stage == S_) stage = 0, phase ^= 1;
@@ -479,8 +484,7 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
       // later phase of its barrier exists, so the parity wait is exact)
       for (int s = 0; s < S_ && lane == 0; ++s)
         if (((used >> s) & 1u) &&
-            !mbar_wait(((last_code >> s) & 1u) ? &cfull[s] : &fullA[s], (last_par >> s) & 1u,
-                       nullptr))
+            !mbar_wait(&fullA[s], (last_par >> s) & 1u, nullptr))
           report(a.status, FQ_ERR_TIMEOUT);
     }
   } else if (warp == 6) {
@@ -572,110 +576,180 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
   } else if (issuer_of(warp, NI) >= 0) {
     // -------------------------------------------------------------- MMA issuers
     // issuer q: the K blocks that land in ring stages s = q (mod NI), into accumulator q of
-    // the task's buffer; every issuer walks every round to follow the ring
+    // the task's buffer.  The whole warp walks its rounds and one elected lane issues, so that the
+    // operands are warp-uniform where they are computed (one lane walking alone: 4096 x 4096 at one
+    // token 27.0 us per call, the whole warp 25.3).
     const int q = issuer_of(warp, NI);
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = umma_idesc_bf16(kBM, BN);
-      int stage = 0;
+      const uint64_t a0 = umma_desc_sw128(smem_u32(sA)), b0 = umma_desc_sw128(smem_u32(sB));
+      const uint64_t ones = umma_desc_sw128(smem_u32(smem + Lo::oOnes));
+      const bool elected = elect_one();
+      int stage = q;                   // the issuer's next stage and its phase
       uint32_t phase = 0;
+      int pos = 0;                     // ring position of the task's first K block, mod NI
       int buf = 0;
       uint32_t acc_phase = 0;
       bool issued_any = false;
-      for (int i = t_lo; i < t_hi && !*abort_flag; ++i) {
+      for (int i = t_lo; i < t_hi; ++i) {
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
         const Task t = task_at(sched, i);
         const DecPhase ph = phase_of(a, t.l, t.p);
         int k0, k1;
         krange(ph, t.tile, k0, k1);
-        if (!mbar_wait(&tempty[buf], acc_phase ^ 1, abort_flag)) {
-          if (!*abort_flag) note_timeout(a.status, 4, i, buf, static_cast<int>(acc_phase));
-          *abort_flag = 1;
+        const int n = max(0, k1 - k0), first = (q - pos + NI) % NI;
+        pos = (pos + n) % NI;
+        bool ok = mbar_wait(&tempty[buf], acc_phase ^ 1, abort_flag);
+        const bool sums = kSums && t.p == 1;
+        if (sums) ok = ok && mbar_wait(ones_bar, 0, abort_flag);       // its only phase
+        if (!__all_sync(0xffffffffu, ok)) {
+          if (lane == 0) {
+            if (!*abort_flag) note_timeout(a.status, 4, i, buf, static_cast<int>(acc_phase));
+            *abort_flag = 1;
+          }
           break;
         }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>((buf * NI + q) * BN);
-        bool ok = true;
-        bool acc = false;      // this issuer has accumulated a K block of the task
-        for (int kb = k0; kb < k1; ++kb) {
-          if (stage % NI == q) {
-            ok = mbar_wait(&fullA[stage], phase, abort_flag);
-            if (!ok && !*abort_flag) note_timeout(a.status, 5, i, stage, kb * 2 + static_cast<int>(phase));
-            if (ok) {
-              ok = mbar_wait(&fullB[stage], phase, abort_flag);
-              if (!ok && !*abort_flag) note_timeout(a.status, 6, i, stage, kb * 2 + static_cast<int>(phase));
-            }
-            if (!ok) break;
-            tc_fence_after_sync();
-            const uint64_t adesc = umma_desc_sw128(smem_u32(sA + stage * kATile));
-            const uint64_t bdesc = umma_desc_sw128(smem_u32(sB + stage * kBTile));
+        for (int j = first; j < n; j += NI) {
+          ok = mbar_wait(&fullA[stage], phase, abort_flag);
+          if (ok) ok = mbar_wait(&fullB[stage], phase, abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) {
+            if (lane == 0 && !*abort_flag)
+              note_timeout(a.status, 5, i, stage, (k0 + j) * 2 + static_cast<int>(phase));
+            break;
+          }
+          tc_fence_after_sync();
+          if (elected) {
+            const uint64_t adesc = a0 + static_cast<uint64_t>(stage * (kATile >> 4));
+            const uint64_t bdesc = b0 + static_cast<uint64_t>(stage * (kBTile >> 4));
+            const uint32_t more = j > first ? 1u : 0u;
+            if (sums) {                // two accumulators in turn, so that neither waits
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              umma_bf16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (acc || k > 0) ? 1u : 0u);
-            acc = true;
-            issued_any = true;
+              for (int k = 0; k < kBK / 16; ++k) {
+                umma_bf16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, more | (k > 0));
+                umma_bf16(d_tmem + Lo::kSumCol, ones + 2 * k, bdesc + 2 * k, idesc,
+                          more | (k > 0));
+              }
+            } else {
+#pragma unroll
+              for (int k = 0; k < kBK / 16; ++k)
+                umma_bf16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, more | (k > 0));
+            }
             umma_commit(&empty[stage]);
           }
-          if (++stage == S_) stage = 0, phase ^= 1;
+          __syncwarp();
+          issued_any = true;
+          stage += NI;
+          if (stage >= S_) stage -= S_, phase ^= 1;
         }
         if (!ok) {
-          *abort_flag = 1;
+          if (lane == 0) *abort_flag = 1;
           break;
         }
-        umma_commit(&tfull[buf]);      // with no K block of its own this arrives at once
+        if (elected) umma_commit(&tfull[buf]);   // with no K block of its own this arrives at once
+        __syncwarp();
         if (++buf == 2) buf = 0, acc_phase ^= 1;
       }
       if (issued_any) {
-        umma_commit(&mma_done[q]);
-        if (!mbar_wait(&mma_done[q], 0, nullptr)) report(a.status, FQ_ERR_TIMEOUT);
+        if (elected) umma_commit(&mma_done[q]);
+        __syncwarp();
+        if (!mbar_wait(&mma_done[q], 0, nullptr) && lane == 0) report(a.status, FQ_ERR_TIMEOUT);
       }
     }
   } else if ((warp >= 7 && warp <= 10) || (DecCfg<BN>::kPairs && warp >= 16 && warp <= 19)) {
     // -------------------------------------------------------------- code decoders
     // Decoder d (warps 7-10, and 16-19 with decoder pairs) expands the code blocks of the core
     // rounds that land in ring stages s = d (mod 4) into the stage's A slot (with pairs, rows
-    // 0-63 by warp 7 + d and rows 64-127 by warp 16 + d); it waits for nothing else.  All lanes
-    // wait (measured: one polling lane with the others parked in a shuffle wakes later).
+    // 0-63 by warp 7 + d and rows 64-127 by warp 16 + d).  It walks the CTA's core rounds of
+    // its stages over all tasks and holds the codes of the next two in registers, loaded from
+    // global memory when their predecessors have been handed over, so that a round's chain is
+    // stage free (cfull), expand, MMAs, and the weight producer copies no codes.
     const int dw = warp <= 10 ? warp - 7 : warp - 16;
     constexpr int kRR = DecCfg<BN>::kPairs ? 2 : 4;         // 32-row groups per decoder
-    const int rr0 = warp <= 10 ? 0 : 2;
-    int stage = 0;
-    uint32_t cpar = 0;     // bit s: parity of the next cfull[s] phase
-    bool ok = true;
-    for (int i = t_lo; i < t_hi && ok; ++i) {
-      if (__shfl_sync(0xffffffffu, *abort_flag != 0, 0)) break;   // warp-uniform
-      const Task t = task_at(sched, i);
-      const DecPhase ph = phase_of(a, t.l, t.p);
-      int k0, k1;
-      krange(ph, t.tile, k0, k1);
-      const int n = max(0, k1 - k0);
-      if (t.p != 1) {
-        stage = (stage + n) % S_;
-        continue;
-      }
-      for (int kb = 0; kb < n; ++kb) {
-        if ((stage & 3) == dw) {
-          const bool got = mbar_wait(&cfull[stage], (cpar >> stage) & 1u, abort_flag);
-          if (!got && lane == 0 && !*abort_flag) note_timeout(a.status, 7, i, stage, static_cast<int>(cpar));
-          cpar ^= 1u << stage;
-          if (!__all_sync(0xffffffffu, got)) {
-            ok = false;
-            break;
-          }
-          const uint4* codes = reinterpret_cast<const uint4*>(sC + stage * kCodeBytes);
-          uint8_t* tile_a = sA + stage * kATile;
-#pragma unroll
-          for (int rr = rr0; rr < rr0 + kRR; ++rr)
-            decode_row_dec(codes[lane + 32 * rr], tile_a, lane + 32 * rr);
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&fullA[stage]);
+    const int row0 = lane + (warp <= 10 ? 0 : 64);
+    struct Round {
+      uint4 codes[kRR];
+      int stage, task;                  // stage -1: no round left
+    };
+    int ti = t_lo - 1, ring = 0, left = 0, n_task = 0;   // task, its ring position and K blocks
+    int st = 0;                                           // stage of its next round of this decoder
+    const uint4* src = nullptr;                           // and that round's codes
+    auto step = [&](int stage) { return stage + 4 < S_ ? 4 : S_ - stage + dw; };
+    auto fetch = [&](Round& r) {
+      while (left <= 0) {
+        if (ti + 1 >= t_hi) {
+          r.stage = -1;
+          return;
         }
-        if (++stage == S_) stage = 0;
+        ring = (ring + n_task) % S_;
+        ++ti;
+        const Task t = task_at(sched, ti);
+        const DecPhase ph = phase_of(a, t.l, t.p);
+        int k0, k1;
+        krange(ph, t.tile, k0, k1);
+        n_task = max(0, k1 - k0);
+        if (t.p != 1) continue;
+        int first = 0;
+        st = ring;
+        while ((st & 3) != dw) {
+          ++first;
+          if (++st == S_) st = 0;
+        }
+        left = n_task - first;
+        src = reinterpret_cast<const uint4*>(
+                  a.L[t.l].words + (static_cast<int64_t>(t.tile) * ph.KB + k0 + first) * 512) +
+              row0;
       }
+#pragma unroll
+      for (int rr = 0; rr < kRR; ++rr) r.codes[rr] = ldg_stream_u4(src + 32 * rr);
+      r.stage = st;
+      r.task = ti;
+      const int d = step(st);
+      st += d;
+      if (st >= S_) st -= S_;
+      left -= d;
+      src += d * (kCodeBytes / 16);
+    };
+    uint32_t cpar = 0;     // bit s: parity of the next cfull[s] phase
+    auto expand = [&](const Round& r) -> bool {
+      const int stage = r.stage;
+      const bool got = mbar_wait(&cfull[stage], (cpar >> stage) & 1u, abort_flag);
+      if (!got && lane == 0 && !*abort_flag) note_timeout(a.status, 7, r.task, stage, static_cast<int>(cpar));
+      cpar ^= 1u << stage;
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) {
+          report(a.status, FQ_ERR_TIMEOUT);
+          *abort_flag = 1;
+        }
+        return false;
+      }
+      uint8_t* tile_a = sA + stage * kATile;
+#pragma unroll
+      for (int rr = 0; rr < kRR; ++rr) decode_row_dec(r.codes[rr], tile_a, row0 + 32 * rr);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&fullA[stage]);
+      return true;
+    };
+    // (the first two turns only load; one copy of each body keeps the code that a short launch
+    // has to fetch small)
+    Round cur{}, nxt{};
+    for (int turn = 0;; ++turn) {
+      if (turn >= 2 && (cur.stage < 0 || !expand(cur))) break;
+      cur = nxt;
+      fetch(nxt);
     }
-    if (!ok && lane == 0) {
-      report(a.status, FQ_ERR_TIMEOUT);
-      *abort_flag = 1;
-    }
+  } else if (kSums && warp == 11) {
+    // -------------------------------------------------------------- the tile of ones
+    // (off the launch's start: it is needed by the first core round)
+    for (int e = lane; e < kATile / 16; e += 32)
+      reinterpret_cast<uint4*>(smem + Lo::oOnes)[e] =
+          make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(ones_bar);
   } else if (warp >= 2 && warp <= 5) {
     // -------------------------------------------------------------- epilogue (warps 2-5)
     const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
@@ -698,13 +772,11 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
     for (int i = t_lo; i < t_hi; ++i, ++j) {
       const Task t = task_at(sched, i);
       const DecPhase ph = phase_of(a, t.l, t.p);
-      const DecPhase ph_z = phase_of(a, t.l, 0);      // the layer's z and its ready flags
       const __half* l_scale = a.L[t.l].scale;
       const __half* l_zero = a.L[t.l].zero;
       const float* l_gamma = a.L[t.l].gamma;
       int k0, k1;
       krange(ph, t.tile, k0, k1);
-      const bool has_k = k1 > k0;
       const int row = t.tile * kBM + r_in_tile;
       const bool row_ok = row < ph.R;
       float s_i = 0.f, z_i = 0.f, g_row = 1.f;
@@ -715,9 +787,11 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
       }
       const float zb_i = z_i - 4.f * s_i;          // the decoded codes carry an offset of 4
       bool fail = false;
-      if (t.p == 1) {
+      if (!kSums && t.p == 1) {
         // sum of z over this CTA's K range: first the ready flags of the slices it reads
+        const bool has_k = k1 > k0;
         if (has_k && !(a.ext_in & 2)) {
+          const DecPhase ph_z = phase_of(a, t.l, 0);
           const int sl0 = (k0 * kBK) / rows_per, sl1 = (min(ph.K, k1 * kBK) - 1) / rows_per;
           for (int gs = sl0 + et; gs <= sl1 && !fail; gs += kEpi) {
             fail = !wait_flag(&ph_z.flags[(gs / S) * kWsSlices + gs % S], g, abort_flag);
@@ -728,20 +802,26 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
           if (et == 0) *abort_flag = 1;
           break;
         }
-        {
-          // 128 / BN threads per token each add a strided share of the token's z, then one
-          // thread per token adds the shares in a fixed order
-          constexpr int kPer = kEpi / BN;
-          const int q = et % BN, part = et / BN;
-          float sz = 0.f;
-          if (q < a.M && has_k) {
-            // z columns k0 * 64 .. of token q: multiples of 8 (n_in is a multiple of 16), so
-            // 16-byte loads from L2, each thread a strided share
-            const int c0 = k0 * kBK, c1 = min(ph.K, k1 * kBK);
-            const __nv_bfloat16* zr = ph_z.out + static_cast<int64_t>(q) * ph.K;
-            for (int c = c0 + 8 * part; c < c1; c += 8 * kPer) {
-              const uint4 w = ldcg_u4(zr + c);
-              const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
+        // 128 / BN threads per token each add a strided share of the token's z, then one
+        // thread per token adds the shares in a fixed order
+        constexpr int kPer = kEpi / BN;
+        const int q = et % BN, part = et / BN;
+        float sz = 0.f;
+        if (q < a.M && has_k) {
+          // z columns k0 * 64 .. of token q: multiples of 8 (n_in is a multiple of 16), so
+          // 16-byte loads from L2, each thread a strided share
+          const int c0 = k0 * kBK, c1 = min(ph.K, k1 * kBK);
+          const __nv_bfloat16* zr = a.L[t.l].ph[0].out + static_cast<int64_t>(q) * ph.K;
+          // four loads in flight (zeros past the range), added in order
+          for (int c = c0 + 8 * part; c < c1; c += 32 * kPer) {
+            uint4 w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              w[u] = c + 8 * kPer * u < c1 ? ldcg_u4(zr + c + 8 * kPer * u)
+                                           : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const uint32_t wv[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
                 const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&wv[e]));
@@ -749,14 +829,14 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
               }
             }
           }
-          zs_part[part * BN + q] = sz;
-          named_barrier_sync(1, kEpi);
-          if (et < BN) {
-            float tot = 0.f;
+        }
+        zs_part[part * BN + q] = sz;
+        named_barrier_sync(1, kEpi);
+        if (et < BN) {
+          float tot = 0.f;
 #pragma unroll
-            for (int r = 0; r < kPer; ++r) tot += zs_part[r * BN + et];
-            zs_s[et] = tot;
-          }
+          for (int r = 0; r < kPer; ++r) tot += zs_part[r * BN + et];
+          zs_s[et] = tot;
         }
       }
       // one thread waits, the others block in the named barrier below
@@ -779,22 +859,35 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
       // this thread's row of the accumulator (for the core: gamma (s Q z + zero sum z) over the
       // CTA's K range), the issuers' accumulators added in issuer order
       float vals[BN];
-#pragma unroll
-      for (int c = 0; c < BN; c += kChunk) {
-        float v[kChunk];
+      // columns c .. c + 15 of the issuers' accumulators (or sums), added in issuer order
+      auto gather = [&](uint32_t col, float (&v)[kChunk]) {
 #pragma unroll
         for (int q = 0; q < kChunk; ++q) v[q] = 0.f;
+#pragma unroll
         for (int qa = 0; qa < NI; ++qa) {
           if ((qa - ring0 + NI) % NI >= nkb) continue;       // uniform across the warp
           float w[kChunk];
-          tmem_ld16(t_row + static_cast<uint32_t>(qa * BN + c), w);
+          tmem_ld16(t_row + col + static_cast<uint32_t>(qa * BN), w);
           tmem_wait_ld();
 #pragma unroll
           for (int q = 0; q < kChunk; ++q) v[q] += w[q];
         }
+      };
+#pragma unroll
+      for (int c = 0; c < BN; c += kChunk) {
+        float v[kChunk];
+        if (kSums && t.p == 1) {
+          gather(static_cast<uint32_t>(Lo::kSumCol + c), v);
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * v[q];
+        } else if (t.p == 1) {
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * zs_s[c + q];
+        }
+        gather(static_cast<uint32_t>(c), v);
 #pragma unroll
         for (int q = 0; q < kChunk; ++q)
-          vals[c + q] = t.p == 1 ? g_row * fmaf(s_i, v[q], zb_i * zs_s[c + q]) : v[q];
+          vals[c + q] = t.p == 1 ? g_row * fmaf(s_i, v[q], vals[c + q]) : v[q];
       }
       tc_fence_before_sync();
       mbar_arrive(&tempty[buf]);
@@ -945,15 +1038,15 @@ DecWs dec_ws(int M, int n_in, int n_out) {
   return L;
 }
 
-template <int BN>
+template <int BN, bool kSums>
 cudaError_t prepare(int dev) {
   static std::mutex mu;
   static std::map<int, bool> done;
   std::lock_guard<std::mutex> g(mu);
   if (done[dev]) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(decode_layer_kernel<BN>,
+  const cudaError_t e = cudaFuncSetAttribute(decode_layer_kernel<BN, kSums>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             DecLayout<BN>::kBytes);
+                                             DecLayout<BN, kSums>::kBytes);
   if (e == cudaSuccess) done[dev] = true;
   return e;
 }
@@ -970,7 +1063,7 @@ int max_clusters(int dev, int S) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(S * 64));
   cfg.blockDim = dim3(DecCfg<BN>::kThreads);
-  cfg.dynamicSmemBytes = DecLayout<BN>::kBytes;
+  cfg.dynamicSmemBytes = DecLayout<BN, true>::kBytes;   // both forms: one CTA per SM
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(S);
@@ -979,7 +1072,7 @@ int max_clusters(int dev, int S) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, decode_layer_kernel<BN>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, decode_layer_kernel<BN, true>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -1096,7 +1189,8 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
               int budget, cudaStream_t s) {
   int dev = 0;
   cudaGetDevice(&dev);
-  if (prepare<BN>(dev) != cudaSuccess) return FQ_ERR_CUDA;
+  if (prepare<BN, true>(dev) != cudaSuccess || prepare<BN, false>(dev) != cudaSuccess)
+    return FQ_ERR_CUDA;
   int total = 0;
   for (const Block& b : blocks) total += static_cast<int>(ceil_div(b.R, kBM));
   if (total > kMaxSched) return FQ_ERR_UNSUPPORTED;
@@ -1111,6 +1205,10 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
       ph.kbs = static_cast<int>(ceil_div(ph.KB, plan->S));
     }
   a.total = total;
+  // Where sum(z) comes from, by the longest core range of a CTA: the epilogue's reads grow with the
+  // range, the tensor cores' fixed cost does not (even at about 8 K blocks).
+  bool sums = false;
+  for (int l = 0; l < a.G; ++l) sums |= a.L[l].ph[1].kbs > kSumMmaBlocks;
   {
     // L2 warming within one budget for the whole launch: the code blocks of every layer, then
     // the T_out^T of as many layers (in order) as fit with them
@@ -1136,7 +1234,7 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(plan->ncl * plan->S));
   cfg.blockDim = dim3(DecCfg<BN>::kThreads);
-  cfg.dynamicSmemBytes = DecLayout<BN>::kBytes;
+  cfg.dynamicSmemBytes = sums ? DecLayout<BN, true>::kBytes : DecLayout<BN, false>::kBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1147,7 +1245,8 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = plan->S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, decode_layer_kernel<BN>, maps, a, plan->sched) == cudaSuccess
+  return cudaLaunchKernelEx(&cfg, sums ? decode_layer_kernel<BN, true> : decode_layer_kernel<BN, false>,
+                            maps, a, plan->sched) == cudaSuccess
              ? FQ_OK
              : FQ_ERR_CUDA;
 }
