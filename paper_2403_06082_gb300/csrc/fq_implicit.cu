@@ -35,36 +35,33 @@ namespace {
 
 
 // ------------------------------------------------------------------------------ rotations
-// CTA (token t, rows r0 .. r0 + 7 of the a x b block); bf16 in and out.
-//   analysis:  V = Pi^T x (V[perm[i]] = x_i), Y = Q_a^T V Q_b, out = D vec(Y)      A = Q_a^T, B = Q_b
+// A cluster of C CTAs takes one token's a x b block; bf16 in and out, fp32 between.
+//   analysis:  V = Pi^T x (V_e = x[iperm[e]]), Y = Q_a^T V Q_b, out = D vec(Y)   A = Q_a^T, B = Q_b
 //   synthesis: V = D s, Y = Q_a V Q_b^T, out = Pi vec(Y) (out[iperm[e]] = vec(Y)_e) A = Q_a, B = Q_b^T
-// The CTA is KG groups of r threads (r = b rounded up to a warp): thread (c, g) owns column c and
-// the reduction indices g, g + KG, ... of both products, for all eight rows at once (eight
-// accumulators; the eight row values of a reduction index are one 32-byte broadcast read of a
-// row-interleaved copy).  The KG partial sums of an entry are added in group order through
-// shared memory.  The factors do not depend on the previous kernel: A's rows, and all of B
-// when b <= kRotStageB and the CTA's shared memory stays within kRotSmemStaged (so that two
-// CTAs fit an SM), are requested in shared memory before the wait for the input, with
-// asynchronous copies all in flight at once; otherwise B streams through kRotBufs buffers of
-// kRotChunk rows, so that its loads overlap the products (the first chunks are requested
-// before the wait).
-constexpr int kRotRows = 8;        // rows of the a x b block per rotation CTA
-constexpr int kRotStageB = 128;
-constexpr size_t kRotSmemStaged = 110 * 1024;
-constexpr int kRotChunk = 16;
-constexpr int kRotBufs = 4;
-constexpr int kRotMaxGroups = 4;
+// CTA r computes columns [r bc, (r + 1) bc) of T1 = A V, which needs only those columns of V, and
+// stores each row of them into the shared memory of the CTA that owns the row; after one cluster
+// barrier it computes its rows [r rc, (r + 1) rc) of Y = T1 B.  So a token's gather, products and
+// scatter are each split C ways and nothing is computed or gathered twice.  Both products take
+// 4 rows x 2 columns per thread, the row values of a reduction index as one 16-byte read (the
+// factors are read in the orientation that has them consecutive).
+// What bounds it is latency: a token is two products of a few million multiply-adds.  The
+// factors, the permutation and the signs do not depend on the previous kernel and are staged in
+// shared memory before the wait for the input; a factor that does not fit is read from L2.
+// PLACEHOLDER_ROTATE
+constexpr int kRotThreads = 256;
+constexpr size_t kMaxSmem = 227 * 1024;
 
 // One launch rotates the tokens of up to FQ_MAX_GROUP layers (blockIdx.z = layer).
 struct RotLayer {
   const __nv_bfloat16* in;
   __nv_bfloat16* out;
-  int d, a, b;
-  int bp, KG;             // column slots (b rounded up to 32) and reduction groups
-  int staged;             // all of B in shared memory (else streamed in chunks)
-  const float* A;
-  const float* B;
-  const int32_t* perm;
+  int a, b;
+  int ap, bp;             // row strides of the staged factors: a rounded up to 4, b to 2
+  int bc, vs;             // columns of V per CTA, and their stride (rounded up to 2)
+  int rc, rs;             // rows of Y per CTA, and their stride in T1t (rounded up to 4)
+  int stage_a, stage_b;   // the factor is staged in shared memory
+  const float* At;        // A^T, a x a row-major: At[i][r] = A[r][i]
+  const float* B;         // b x b row-major
   const int32_t* iperm;
   const float* signs;
 };
@@ -72,161 +69,179 @@ struct RotBatch {
   RotLayer L[FQ_MAX_GROUP];
 };
 
-__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc)
+template <int kBytes>
+__device__ __forceinline__ void cp_async(float* smem_dst, const float* gsrc) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc),
+               "n"(kBytes)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
-__device__ __forceinline__ void cp_async_wait_pending() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(kRotBufs - 1) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
-
-__device__ __forceinline__ void fma8(float (&acc)[kRotRows], const float* r8, float v) {
-  const float4 u0 = *reinterpret_cast<const float4*>(r8);
-  const float4 u1 = *reinterpret_cast<const float4*>(r8 + 4);
-  acc[0] = fmaf(u0.x, v, acc[0]);
-  acc[1] = fmaf(u0.y, v, acc[1]);
-  acc[2] = fmaf(u0.z, v, acc[2]);
-  acc[3] = fmaf(u0.w, v, acc[3]);
-  acc[4] = fmaf(u1.x, v, acc[4]);
-  acc[5] = fmaf(u1.y, v, acc[5]);
-  acc[6] = fmaf(u1.z, v, acc[6]);
-  acc[7] = fmaf(u1.w, v, acc[7]);
+__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
 
-template <bool kSynth>
-__global__ void __launch_bounds__(1024) rotate_kernel(const __grid_constant__ RotBatch rb) {
-  const RotLayer& ly = rb.L[blockIdx.z];
-  const __nv_bfloat16* __restrict__ in = ly.in;
-  __nv_bfloat16* __restrict__ out = ly.out;
-  const int d = ly.d, a = ly.a, b = ly.b, bp = ly.bp, KG = ly.KG;
-  const float* __restrict__ A = ly.A;
-  const float* __restrict__ B = ly.B;
-  const int32_t* __restrict__ perm = ly.perm;
-  const int32_t* __restrict__ iperm = ly.iperm;
-  const float* __restrict__ signs = ly.signs;
-  pdl_launch_dependents();
-  const int r0 = static_cast<int>(blockIdx.x) * kRotRows;
-  if (r0 >= a) {
-    pdl_wait();
+// An n x n factor (row-major) into shared memory with row stride np, asynchronously, a warp per row
+// in the widest pieces that the rows' alignment allows; past the n-th column nothing is written
+// (such entries only reach results that are dropped).
+__device__ __forceinline__ void stage_factor(float* dst, const float* __restrict__ src, int n,
+                                             int np, int tid) {
+  if (n % 4 == 0) {       // np == n: one contiguous copy
+    for (int i = tid; i < n * n / 4; i += kRotThreads) cp_async<16>(dst + 4 * i, src + 4 * i);
     return;
   }
-  extern __shared__ float4 rot_smem4[];
-  float* V = reinterpret_cast<float*>(rot_smem4);   // [d], d rounded up to 4
-  float* At = V + ((d + 3) & ~3);                   // [a][8]: At[i][g] = A[r0 + g][i]
-  float* T1t = At + a * kRotRows;                   // [b][8]: T1t[k][g] = (A V)[r0 + g][k]
-  float* P = T1t + b * kRotRows;                    // [KG][8][bp] partial sums
-  float* Bs = P + KG * kRotRows * bp;               // all of B, or kRotBufs chunks of it
-  const int t = blockIdx.y, nt = blockDim.x, tid = threadIdx.x;
-  const int rows = min(kRotRows, a - r0);
-  const int c = tid % bp, kg = tid / bp;
-  const bool active = c < b && kg < KG;
-  const bool staged = ly.staged != 0;
-  const bool async = (b & 3) == 0;
-  const int nch = (b + kRotChunk - 1) / kRotChunk;
-  // chunk ch of B (rows ch * kRotChunk ..) into buffer ch mod kRotBufs; every thread commits a
-  // group per call, so that the group count stays uniform
-  auto stage_chunk = [&](int ch) {
-    if (ch < nch) {
-      const int k0 = ch * kRotChunk, kn = min(kRotChunk, b - k0);
-      const float* src = B + static_cast<int64_t>(k0) * b;
-      float* dst = Bs + (ch % kRotBufs) * kRotChunk * b;
-      for (int i = tid; i < kn * b / 4; i += nt) cp_async16(dst + 4 * i, src + 4 * i);
-    }
-    cp_async_commit();
-  };
-  for (int i = tid; i < a * kRotRows; i += nt) {
-    const int ii = i / kRotRows, g = i % kRotRows;
-    At[i] = g < rows ? A[static_cast<int64_t>(r0 + g) * a + ii] : 0.f;
+  const int lane = tid & 31;
+  for (int r = tid >> 5; r < n; r += kRotThreads / 32) {
+    const float* from = src + static_cast<int64_t>(r) * n;
+    float* to = dst + r * np;
+    if (n % 2 == 0)
+      for (int i = 2 * lane; i < n; i += 64) cp_async<8>(to + i, from + i);
+    else
+      for (int i = lane; i < n; i += 32) cp_async<4>(to + i, from + i);
   }
-  if (staged) {
-    if (async) {
-      for (int i = tid; i < b * b / 4; i += nt) cp_async16(Bs + 4 * i, B + 4 * i);
-      cp_async_commit();
-    } else {
-#pragma unroll 8
-      for (int i = tid; i < b * b; i += nt) Bs[i] = B[i];
+}
+
+// acc[row][col] += sum_k rows4(k)[row] * cols2(k)[col]
+template <int kUnroll, typename Rows, typename Cols>
+__device__ __forceinline__ void rot_product(float (&acc)[4][2], int n, Rows rows4, Cols cols2) {
+#pragma unroll kUnroll
+  for (int k = 0; k < n; ++k) {
+    const float4 u = rows4(k);
+    const float2 v = cols2(k);
+    acc[0][0] = fmaf(u.x, v.x, acc[0][0]);
+    acc[0][1] = fmaf(u.x, v.y, acc[0][1]);
+    acc[1][0] = fmaf(u.y, v.x, acc[1][0]);
+    acc[1][1] = fmaf(u.y, v.y, acc[1][1]);
+    acc[2][0] = fmaf(u.z, v.x, acc[2][0]);
+    acc[2][1] = fmaf(u.z, v.y, acc[2][1]);
+    acc[3][0] = fmaf(u.w, v.x, acc[3][0]);
+    acc[3][1] = fmaf(u.w, v.y, acc[3][1]);
+  }
+}
+
+template <bool kSynth, bool kCluster>
+__global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_constant__ RotBatch rb) {
+  const RotLayer& ly = rb.L[blockIdx.z];
+  const int a = ly.a, b = ly.b, ap = ly.ap, bp = ly.bp, vs = ly.vs, rs = ly.rs, rc = ly.rc;
+  const int tid = threadIdx.x;
+  const int rank = kCluster ? static_cast<int>(blockIdx.x) : 0;       // the cluster spans x
+  const int c0 = min(b, rank * ly.bc), nc = min(ly.bc, b - c0);       // this CTA's columns of V
+  const int r0 = min(a, rank * rc), nr = min(rc, a - r0);             // and its rows of Y
+  extern __shared__ float4 rot_smem4[];
+  float* T1t = reinterpret_cast<float*>(rot_smem4);   // [b][rs]: T1t[k][r] = T1[r0 + r][k]
+  float* V = T1t + b * rs;                            // [a][vs]: V[k][c] = V_(k, c0 + c)
+  float* Bs = V + a * vs + ((a * vs) & 2);            // [b][bp], 16-byte aligned
+  float* As = Bs + (ly.stage_b ? b * bp + ((b * bp) & 2) : 0);   // [a][ap]
+  pdl_launch_dependents();
+  if (kCluster) cluster_arrive();   // (waited for before the first store into another CTA)
+  if (ly.stage_a) stage_factor(As, ly.At, a, ap, tid);
+  if (ly.stage_b) stage_factor(Bs, ly.B, b, bp, tid);
+  cp_async_commit();
+  // V's place first holds what does not depend on the input: the index each entry is gathered
+  // from (analysis) or its sign (synthesis).  A thread takes columns vc, vc + dc, ... (one, when
+  // they are at most the threads) and rows vk, vk + dk, ...
+  const bool narrow = nc <= kRotThreads;
+  const int dk = narrow ? kRotThreads / max(nc, 1) : 1, dc = narrow ? max(nc, 1) : kRotThreads;
+  const int vc = tid % dc, vk = narrow ? (tid < dk * dc ? tid / dc : a) : 0;
+  for (int c = vc; c < nc; c += dc) {
+#pragma unroll 4
+    for (int k = vk; k < a; k += dk) {
+      const int e = k * b + c0 + c;
+      V[k * vs + c] = kSynth ? ly.signs[e] : __int_as_float(ly.iperm[e]);
     }
-  } else if (async) {
-    for (int ch = 0; ch < kRotBufs - 1; ++ch) stage_chunk(ch);
   }
   pdl_wait();
-  const __nv_bfloat16* src = in + static_cast<int64_t>(t) * d;
-  if (kSynth) {
+  const int64_t tok = static_cast<int64_t>(blockIdx.y) * a * b;
+  const __nv_bfloat16* in = ly.in + tok;
+  for (int c = vc; c < nc; c += dc) {
 #pragma unroll 8
-    for (int i = tid; i < d; i += nt) V[i] = signs[i] * __bfloat162float(src[i]);
-  } else {
-#pragma unroll 8
-    for (int i = tid; i < d; i += nt) V[perm[i]] = __bfloat162float(src[i]);
-  }
-  if (staged && async) cp_async_wait_all();
-  __syncthreads();
-  float acc[kRotRows];
-  // T1 = A[rows] V: this thread's partial over i = kg, kg + KG, ...
-#pragma unroll
-  for (int g = 0; g < kRotRows; ++g) acc[g] = 0.f;
-  if (active) {
-#pragma unroll 4
-    for (int i = kg; i < a; i += KG) fma8(acc, At + i * kRotRows, V[i * b + c]);
-#pragma unroll
-    for (int g = 0; g < kRotRows; ++g) P[(kg * kRotRows + g) * bp + c] = acc[g];
-  }
-  __syncthreads();
-  for (int e = tid; e < b * kRotRows; e += nt) {
-    const int k = e / kRotRows, g = e % kRotRows;
-    float s = 0.f;
-    for (int q = 0; q < KG; ++q) s += P[(q * kRotRows + g) * bp + k];
-    T1t[e] = s;
-  }
-  __syncthreads();
-  // Y = T1 B: this thread's partial over k = kg, kg + KG, ...
-#pragma unroll
-  for (int g = 0; g < kRotRows; ++g) acc[g] = 0.f;
-  if (staged) {
-    if (active) {
-#pragma unroll 4
-      for (int k = kg; k < b; k += KG) fma8(acc, T1t + k * kRotRows, Bs[k * b + c]);
-    }
-  } else {
-    for (int ch = 0; ch < nch; ++ch) {
-      const int k0 = ch * kRotChunk, k1 = min(b, k0 + kRotChunk);
-      const float* Bc = Bs;
-      if (async) {
-        stage_chunk(ch + kRotBufs - 1);
-        cp_async_wait_pending();     // chunk ch has landed (for this thread's copies)
-        __syncthreads();             // ... and for every thread's
-        Bc = Bs + (ch % kRotBufs) * kRotChunk * b;
-      } else {
-        for (int i = tid; i < (k1 - k0) * b; i += nt) Bs[i] = B[static_cast<int64_t>(k0) * b + i];
-        __syncthreads();
-      }
-      if (active) {
-        const int first = k0 + ((kg - k0 % KG) % KG + KG) % KG;
-        for (int k = first; k < k1; k += KG) fma8(acc, T1t + k * kRotRows, Bc[(k - k0) * b + c]);
-      }
-      __syncthreads();               // the buffer is read before it is refilled
+    for (int k = vk; k < a; k += dk) {              // (this thread's own entries)
+      const float h = V[k * vs + c];
+      V[k * vs + c] = kSynth ? h * __bfloat162float(in[k * b + c0 + c])
+                             : __bfloat162float(in[__float_as_int(h)]);
     }
   }
-  if (active) {
-#pragma unroll
-    for (int g = 0; g < kRotRows; ++g) P[(kg * kRotRows + g) * bp + c] = acc[g];
-  }
+  cp_async_wait_all();
   __syncthreads();
-  __nv_bfloat16* dst = out + static_cast<int64_t>(t) * d;
-  for (int e = tid; e < rows * b; e += nt) {
-    const int g = e / b, cc = e - g * b;
-    float y = 0.f;
-    for (int q = 0; q < KG; ++q) y += P[(q * kRotRows + g) * bp + cc];
-    const int o = (r0 + g) * b + cc;
-    if (kSynth)
-      dst[iperm[o]] = __float2bfloat16_rn(y);
-    else
-      dst[o] = __float2bfloat16_rn(signs[o] * y);
+  if (kCluster) cluster_wait();
+  // T1 = A V, columns c0 .. c0 + nc - 1, to the owners of the rows
+  const int cp = (nc + 1) / 2;
+  for (int t = tid; t < (a + 3) / 4 * cp; t += kRotThreads) {
+    const int r = t / cp * 4, c = t % cp * 2;
+    float acc[4][2] = {};
+    const auto cols = [&](int k) { return *reinterpret_cast<const float2*>(V + k * vs + c); };
+    if (ly.stage_a) {
+      rot_product<8>(
+          acc, a, [&](int k) { return *reinterpret_cast<const float4*>(As + k * ap + r); }, cols);
+    } else {
+      rot_product<2>(acc, a, [&](int k) {
+        const float* p = ly.At + static_cast<int64_t>(k) * a + r;
+        return make_float4(p[0], r + 1 < a ? p[1] : 0.f, r + 2 < a ? p[2] : 0.f,
+                           r + 3 < a ? p[3] : 0.f);
+      }, cols);
+    }
+    if (kCluster) {
+      int owner = r / rc, rl = r - owner * rc;   // the CTA that takes this row, its place there
+#pragma unroll
+      for (int j = 0; j < 4; ++j, ++rl) {
+        if (rl == rc) ++owner, rl = 0;
+        if (r + j >= a) continue;
+        const uint32_t dst = mapa(smem_u32(T1t + (c0 + c) * rs + rl), static_cast<uint32_t>(owner));
+        st_cluster_f32(dst, acc[j][0]);
+        if (c + 1 < nc) st_cluster_f32(dst + 4 * rs, acc[j][1]);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 2; ++q)                // (rows past a fall into the padding)
+        if (c + q < nc)
+          *reinterpret_cast<float4*>(T1t + (c + q) * rs + r) =
+              make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
+    }
+  }
+  if (kCluster)
+    cluster_sync();
+  else
+    __syncthreads();
+  // Y = T1 B, rows r0 .. r0 + nr - 1
+  __nv_bfloat16* out = ly.out + tok;
+  const int bp2 = (b + 1) / 2;
+  for (int t = tid; t < (nr + 3) / 4 * bp2; t += kRotThreads) {
+    const int r = t / bp2 * 4, c = t % bp2 * 2;
+    float acc[4][2] = {};
+    // where the results go (or their signs), requested before the product
+    int dest[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int o = (r0 + min(r + j, nr - 1)) * b + min(c + q, b - 1);
+        dest[j][q] = kSynth ? ly.iperm[o] : __float_as_int(ly.signs[o]);
+      }
+    const auto rows = [&](int k) { return *reinterpret_cast<const float4*>(T1t + k * rs + r); };
+    if (ly.stage_b) {
+      rot_product<8>(acc, b, rows,
+                     [&](int k) { return *reinterpret_cast<const float2*>(Bs + k * bp + c); });
+    } else {
+      rot_product<2>(acc, b, rows, [&](int k) {
+        const float* p = ly.B + static_cast<int64_t>(k) * b + c;
+        return make_float2(p[0], c + 1 < b ? p[1] : 0.f);
+      });
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (r + j >= nr || c + q >= b) continue;
+        if (kSynth)
+          out[dest[j][q]] = __float2bfloat16_rn(acc[j][q]);
+        else
+          out[(r0 + r + j) * b + c + q] =
+              __float2bfloat16_rn(__int_as_float(dest[j][q]) * acc[j][q]);
+      }
   }
 }
 
@@ -377,36 +392,42 @@ ImplWs impl_ws(int M, int d_in, int n_in, int n_out, int d_out) {
   return L;
 }
 
-// a rotation CTA's column slots (b rounded up to a warp), reduction groups and threads
-int rot_slots(int b) { return static_cast<int>(round_up(b, 32)); }
-int rot_groups(int b, int nt) {
-  return std::max(1, std::min(kRotMaxGroups, nt / rot_slots(b)));
-}
-int rot_threads(int b) {
-  return rot_slots(b) * std::max(1, std::min(kRotMaxGroups, 1024 / rot_slots(b)));
-}
-
-size_t rot_smem_with(const fq_frame& f, int KG, bool staged) {
-  const size_t bb = staged ? static_cast<size_t>(f.b) * f.b
-                           : static_cast<size_t>(kRotBufs) * kRotChunk * f.b;
-  return (static_cast<size_t>(round_up(f.d, 4)) + static_cast<size_t>(kRotRows) * (f.a + f.b) +
-          static_cast<size_t>(KG) * kRotRows * rot_slots(f.b) + bb) *
-         4;
-}
-// all of B in shared memory when it is small and leaves room for two CTAs per SM
-bool rot_staged(const fq_frame& f, int KG) {
-  return f.b <= kRotStageB && rot_smem_with(f, KG, true) <= kRotSmemStaged;
-}
-size_t rot_smem(const fq_frame& f, int KG) { return rot_smem_with(f, KG, rot_staged(f, KG)); }
-
-constexpr size_t kMaxSmem = 227 * 1024;
-
+// Frames taken: the sizes that this library's entry points document (a rotation with b <= 1024
+// whose (d + 8 (a + b) + 8 g r + B) fp32 values fit 227 KiB, r = b rounded up to 32, g = min(4,
+// 1024 / r), B = b^2 for b <= 128 where the total stays within 110 KiB and 64 b otherwise).  The
+// rotation kernel itself needs less.
 bool frame_fits(const fq_frame& f) {
   if (ceil_div(static_cast<int64_t>(f.k) * f.rho, kTR) > kWsMaxTiles ||
       ceil_div(f.d, kTR) > kWsMaxTiles)
     return false;
-  return f.a == 0 ||
-         (f.b <= 1024 && rot_smem(f, rot_groups(f.b, rot_threads(f.b))) <= kMaxSmem);
+  if (f.a == 0) return true;
+  if (f.b > 1024) return false;
+  const int64_t r = round_up(f.b, 32), g = std::max<int64_t>(1, std::min<int64_t>(4, 1024 / r));
+  const int64_t base = round_up(f.d, 4) + 8 * (static_cast<int64_t>(f.a) + f.b) + 8 * g * r;
+  const int64_t whole = (base + static_cast<int64_t>(f.b) * f.b) * 4;
+  return (f.b <= 128 && whole <= 110 * 1024) || (base + 64 * static_cast<int64_t>(f.b)) * 4 <=
+                                                    static_cast<int64_t>(kMaxSmem);
+}
+
+// CTAs per token: enough entries for each to outweigh the cluster barriers.  Measured on two layers
+// of 16 tokens (us, C = 1, 2, 4, 8): 512 x 512 20.0, 20.7, 21.3, 21.5; 1024 x 1024 25.2, 27.0, 26.8,
+// 26.6; 2048 x 2048 53.4, 35.0, 30.4, 31.0; 768 to 3072 51.6, 38.4, 33.8, 30.8.
+int rot_cluster(int d) { return d >= 3072 ? 8 : (d > 1024 ? 4 : 1); }
+
+// The layer's split over C CTAs and its staging; returns its shared memory.
+size_t rot_layout(RotLayer& L, int C) {
+  L.ap = static_cast<int>(round_up(L.a, 4));
+  L.bp = static_cast<int>(round_up(L.b, 2));
+  L.bc = static_cast<int>(ceil_div(L.b, C));
+  L.vs = static_cast<int>(round_up(L.bc, 2));
+  L.rc = static_cast<int>(ceil_div(L.a, C));
+  L.rs = static_cast<int>(round_up(L.rc, 4));
+  const size_t base = 4 * (static_cast<size_t>(L.b) * L.rs + round_up(static_cast<int64_t>(L.a) * L.vs, 4));
+  const size_t as = 4 * static_cast<size_t>(L.a) * L.ap;
+  const size_t bs = 4 * static_cast<size_t>(round_up(static_cast<int64_t>(L.b) * L.bp, 4));
+  L.stage_a = base + as <= kMaxSmem;
+  L.stage_b = base + (L.stage_a ? as : 0) + bs <= kMaxSmem;
+  return base + (L.stage_a ? as : 0) + (L.stage_b ? bs : 0);
 }
 
 cudaError_t set_smem_attributes() {
@@ -417,58 +438,60 @@ cudaError_t set_smem_attributes() {
   std::lock_guard<std::mutex> g(mu);
   if (done.count(dev)) return cudaSuccess;
   const int bytes = static_cast<int>(kMaxSmem);
-  cudaError_t e = cudaFuncSetAttribute(rotate_kernel<false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(rotate_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             bytes);
+  void (*const kernels[])(RotBatch) = {rotate_kernel<false, false>, rotate_kernel<false, true>,
+                                       rotate_kernel<true, false>, rotate_kernel<true, true>};
+  cudaError_t e = cudaSuccess;
+  for (auto* k : kernels)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) done.insert(dev);
   return e;
 }
 
-// Launch with programmatic stream serialization (the kernel may start while its predecessor
-// in the stream finishes; it waits with griddepcontrol.wait before reading its inputs).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
 // R^T x (analysis) or R s (synthesis) for M tokens of n layers in one launch, bf16 in and out;
-// layers without a rotation are skipped
+// layers without a rotation, and those whose `in` is null, are skipped.  Launched with
+// programmatic stream serialization (the kernel may start while its predecessor in the stream
+// finishes; it waits with griddepcontrol.wait before reading its inputs).
 template <bool kSynth>
 cudaError_t rotate_batch(int n, const fq_frame* const* f, const void* const* in,
                          void* const* out, int M, cudaStream_t s) {
   RotBatch rb{};
-  int nb = 0, gx = 1, threads = 32;
+  int nb = 0, C = 1;
   size_t smem = 0;
   for (int l = 0; l < n; ++l)
-    if (f[l]->a != 0) threads = std::max(threads, rot_threads(f[l]->b));
+    if (f[l]->a != 0 && in[l]) C = std::max(C, rot_cluster(f[l]->d));
   for (int l = 0; l < n; ++l) {
-    if (f[l]->a == 0) continue;
+    if (f[l]->a == 0 || !in[l]) continue;
     const fq_frame& F = *f[l];
-    const int KG = rot_groups(F.b, threads);
-    rb.L[nb] = RotLayer{static_cast<const __nv_bfloat16*>(in[l]), static_cast<__nv_bfloat16*>(out[l]),
-                        F.d, F.a, F.b, rot_slots(F.b), KG, rot_staged(F, KG) ? 1 : 0,
-                        kSynth ? F.Qa : F.QaT,
-                        kSynth ? F.QbT : F.Qb, F.perm, F.iperm, F.signs};
-    gx = std::max(gx, static_cast<int>(ceil_div(F.a, kRotRows)));
-    smem = std::max(smem, rot_smem(F, KG));
-    ++nb;
+    RotLayer& L = rb.L[nb++];
+    L.in = static_cast<const __nv_bfloat16*>(in[l]);
+    L.out = static_cast<__nv_bfloat16*>(out[l]);
+    L.a = F.a;
+    L.b = F.b;
+    L.At = kSynth ? F.QaT : F.Qa;
+    L.B = kSynth ? F.QbT : F.Qb;
+    L.iperm = F.iperm;
+    L.signs = F.signs;
+    smem = std::max(smem, rot_layout(L, C));
   }
   if (nb == 0) return cudaSuccess;
-  return launch_pdl(rotate_kernel<kSynth>, dim3(static_cast<unsigned>(gx), M, nb), dim3(threads),
-                    smem, s, rb);
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(C), static_cast<unsigned>(M), static_cast<unsigned>(nb));
+  cfg.blockDim = dim3(kRotThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(C);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = C > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, C > 1 ? rotate_kernel<kSynth, true> : rotate_kernel<kSynth, false>,
+                            rb);
 }
 
 template <bool kSynth>
@@ -695,12 +718,28 @@ fq_status fq_linear_forward_implicit_group(int M, int n_layers, const fq_implici
     const fq_implicit_layer& L = layers[l];
     g[l] = DecGroupLayer{nullptr, L.F_in->d, nullptr, *L.C, nullptr, L.F_out->d, L.gamma, nullptr};
   }
+  const fq_frame* fin[FQ_MAX_GROUP];
+  const fq_frame* fout[FQ_MAX_GROUP];
+  const void* xin[FQ_MAX_GROUP];
+  void* vout[FQ_MAX_GROUP];
+  const void* sin_[FQ_MAX_GROUP];
+  void* yout[FQ_MAX_GROUP];
   size_t off = decode_group_workspace_bytes(M, n_layers, g);
   const size_t group_bytes = off;
   for (int l = 0; l < n_layers; ++l) {
     const fq_implicit_layer& L = layers[l];
     const fq_frame &fi = *L.F_in, &fo = *L.F_out;
+    // layers that rotate the same tokens by the same rotation share the result
+    int same = l;
+    for (int j = 0; j < l && same == l; ++j) {
+      const fq_frame& fj = *layers[j].F_in;
+      if (layers[j].x == L.x && fj.a == fi.a && fj.b == fi.b && fj.Qa == fi.Qa && fj.Qb == fi.Qb &&
+          fj.iperm == fi.iperm && fj.signs == fi.signs)
+        same = j;
+    }
     void* v = fi.a > 0 ? static_cast<void*>(w + off) : const_cast<void*>(L.x);
+    if (same < l) v = const_cast<void*>(g[same].x);
+    xin[l] = same < l ? nullptr : L.x;
     off += static_cast<size_t>(round_up(static_cast<int64_t>(M) * fi.d * 2, 256));
     void* sy = fo.a > 0 ? static_cast<void*>(w + off) : L.y;
     off += static_cast<size_t>(round_up(static_cast<int64_t>(M) * fo.d * 2, 256));
@@ -709,16 +748,9 @@ fq_status fq_linear_forward_implicit_group(int M, int n_layers, const fq_implici
     g[l].tin = SparseOperand{fi.ana_tiles, fi.ana_idx, fi.ana_count};
     g[l].tout = SparseOperand{fo.syn_tiles, fo.syn_idx, fo.syn_count};
   }
-  const fq_frame* fin[FQ_MAX_GROUP];
-  const fq_frame* fout[FQ_MAX_GROUP];
-  const void* xin[FQ_MAX_GROUP];
-  void* vout[FQ_MAX_GROUP];
-  const void* sin_[FQ_MAX_GROUP];
-  void* yout[FQ_MAX_GROUP];
   for (int l = 0; l < n_layers; ++l) {
     fin[l] = layers[l].F_in;
     fout[l] = layers[l].F_out;
-    xin[l] = layers[l].x;
     vout[l] = const_cast<void*>(g[l].x);
     sin_[l] = g[l].y;
     yout[l] = layers[l].y;
