@@ -60,7 +60,10 @@ struct PhaseArgs {
   int RT1;                   // 128-row tiles
   int KS, kbs, units;        // K splits per tile, K blocks per split, tiles * KS work units
   float* part;               // KS > 1: fp32 partial tiles [tile][split][BN][128]
-  uint32_t* cnt;             // KS > 1: arrivals per tile (the last resets it to 0)
+  int64_t part_floats;       // what `part` and `cnt` hold (host)
+  int cnt_slots;
+  uint32_t* cnt;             // KS > 1: arrivals per tile (the last resets it to 0; on CTA pairs
+                             // 16 bits for each CTA's half)
   const uint32_t* words;     // core: packed codes
   __nv_bfloat16* out;        // [M][R]
   float* zsum_part;          // analysis writes [RT][M] sums of z; the core reads them
@@ -563,11 +566,15 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
 // for the last use of each of its stages before it leaves, so no copy is in flight then.
 //
 // The code product's round is a chain: stage free, codes expanded, MMAs, stage free.  So the
-// codes do not pass through shared memory: round i is expanded by decoder i mod 6 of two warps (64
-// rows each), which hold the round's codes in registers, loaded from global memory right after
-// they handed over round i - 6 (not before: the release of a hand-over waits for loads in flight).  A decoder meets a stage only in some of its rounds, but it never waits for
-// a phase more than one past the last one complete: at round i it has seen round i - 6 - S's
-// MMAs (S stages) complete, the commits are in order, and 6 <= S.
+// codes do not pass through shared memory: round i is expanded by decoder i mod D, which holds the
+// round's codes in registers, loaded from global memory right after it handed over round i - D
+// (not earlier: the release of a hand-over to the other CTA, about 1500 cycles, waits for loads
+// in flight).  For 256 tokens six decoders of two warps keep up with the MMAs' 512 cycles per
+// round; for 128 tokens nine of one warp are faster (2.4% on 8192 x 8192 at 128 tokens, 9% on 4096 x
+// 4096 at 100), since two warps wait for the same release, and slower for 256 (0.7 to 3%).  A
+// decoder meets a stage only in some of its rounds, but it never waits for a phase more than one
+// past the last one complete: at round i it has seen round i - D - S's MMAs (S stages) complete,
+// the commits are in order, and D <= S.
 template <int PHASE, int BN_>
 struct PairLayout {
   static constexpr bool kCodes = PHASE == kCore;
@@ -580,8 +587,9 @@ struct PairLayout {
   static constexpr int kEpiThreads = 32 * kEpiWarps;
   static constexpr int kHalf = kBN / 2;                 // columns per epilogue warp
   static constexpr int kGroups = kCodes ? 1 : 2;        // of 16 columns at a time (registers)
-  static constexpr int kDecoders = 6;                   // of two warps each
-  static constexpr int kDecWarps = kCodes ? 2 * kDecoders : 0;
+  static constexpr int kDecoders = kBN == 256 ? 6 : kStages;
+  static constexpr int kWarpsPer = kBN == 256 ? 2 : 1;  // warps per decoder
+  static constexpr int kDecWarps = kCodes ? kDecoders * kWarpsPer : 0;
   static constexpr int kThreads = 64 + kEpiThreads + 32 * kDecWarps;
   static constexpr uint32_t kTmemCols = 512;            // all, so that both CTAs' base is 0
   static constexpr int oA = 0;
@@ -589,12 +597,12 @@ struct PairLayout {
   static constexpr int oBar = oB + kStages * kBTile;
   static constexpr int kNumBars = 2 * kStages + 4;
   static constexpr int oMisc = oBar + kNumBars * 8;     // TMEM address, abort and last-split flags
-  static constexpr int oSums = oMisc + 16;
+  static constexpr int oSums = (oMisc + 16 + 15) & ~15;
   static constexpr int kBytes = oSums + kSums + 1024;   // + alignment slack
   static_assert(kBN == 128 || kBN == 256, "tokens per tile");
   static_assert(2 * kBN <= 512, "two accumulators");
-  static_assert(kBTile % 1024 == 0, "B tiles keep 1024-byte alignment");
   static_assert(!kCodes || kDecoders <= kStages, "a decoder waits for a stage's latest phase only");
+  static_assert(kBTile % 1024 == 0, "B tiles keep 1024-byte alignment");
   static_assert(kBytes <= 227 * 1024, "shared memory");
 };
 
@@ -759,7 +767,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S_; ++s) {
-      mbar_init(&full[s], kCodes ? 5 : 1);
+      mbar_init(&full[s], kCodes ? 1 + 2 * Lo::kWarpsPer : 1);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -970,12 +978,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
           return;
         }
         uint32_t h[8], w[8];
+        if (PHASE == kCore) {
+#pragma unroll
+          for (int q = 0; q < kChunk; q += 4) {
+            const float4 zs = *reinterpret_cast<const float4*>(zsum_s + c + q);
+            v[q] = g_i * fmaf(s_i, v[q], z_i * zs.x) * dl;
+            v[q + 1] = g_i * fmaf(s_i, v[q + 1], z_i * zs.y) * dl;
+            v[q + 2] = g_i * fmaf(s_i, v[q + 2], z_i * zs.z) * dl;
+            v[q + 3] = g_i * fmaf(s_i, v[q + 3], z_i * zs.w) * dl;
+          }
+        }
 #pragma unroll
         for (int q = 0; q < kChunk; q += 2) {
-          if (PHASE == kCore) {
-            v[q] = g_i * fmaf(s_i, v[q], z_i * zsum_s[c + q]) * dl;
-            v[q + 1] = g_i * fmaf(s_i, v[q + 1], z_i * zsum_s[c + q + 1]) * dl;
-          }
           const __nv_bfloat162 b = __floats2bfloat162_rn(v[q], v[q + 1]);
           h[q / 2] = *reinterpret_cast<const uint32_t*>(&b);
           if (PHASE == kAnalysis) {
@@ -1036,9 +1050,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
         // CTAs it waits for are past their MMAs; the wait is bounded like every other.)
         const int64_t t1 = static_cast<int64_t>(rt1) * p.TT + tt;
         const bool mine_ok = rt1 < p.RT1;
-        uint32_t* cnt = p.cnt + t1;              // low half: tickets, high half: stored partials
+        uint32_t* cnt = p.cnt + tile;            // this half's bits: 0-7 tickets, 8-15 stored partials
+        const uint32_t shift = 16 * rank;
         if (et == 0)
-          *last_flag = mine_ok ? ((atomicAdd(cnt, 1u) & 0xffffu) == static_cast<uint32_t>(p.KS - 1))
+          *last_flag = mine_ok ? (((atomicAdd(cnt, 1u << shift) >> shift) & 0xffu) ==
+                                  static_cast<uint32_t>(p.KS - 1))
                                : 0;
         named_barrier_sync(1, kN);
         finish = *last_flag != 0;
@@ -1058,17 +1074,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
           named_barrier_sync(1, kN);
           if (et == 0 && mine_ok) {
             __threadfence();
-            atomicAdd(cnt, 0x10000u);
+            atomicAdd(cnt, 0x100u << shift);
           }
         } else {
           if (et == 0) {
-            const uint32_t want = (static_cast<uint32_t>(p.KS - 1) << 16) | static_cast<uint32_t>(p.KS);
-            const bool all = wait_flag(cnt, want, abort_flag);
-            if (!all) {
-              report(p.status, FQ_ERR_TIMEOUT);
-              *abort_flag = 1;
+            const uint32_t want = (static_cast<uint32_t>(p.KS - 1) << 8) | static_cast<uint32_t>(p.KS);
+            const long long w0 = clock64();
+            while (((ld_acquire_gpu(cnt) >> shift) & 0xffffu) != want) {
+              if (clock64() - w0 > kWaitLimitCycles || *abort_flag) {
+                report(p.status, FQ_ERR_TIMEOUT);
+                *abort_flag = 1;
+                break;
+              }
             }
-            *cnt = 0;                            // ready for the next call
+            atomicAnd(cnt, ~(0xffffu << shift));   // ready for the next call
           }
           named_barrier_sync(1, kN);
 #pragma unroll 1
@@ -1112,10 +1131,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
   } else {
     // ---------------------------------------------------------------- code decoders (core)
     if (kCodes) {
-      // decoder d expands the code blocks of rounds d, d + 6, ...; its warp h rows 64 h .. + 63,
-      // two per lane
+      // decoder d expands the code blocks of rounds d, d + D, ..., its warps 128 / W rows each
+      constexpr int D = Lo::kDecoders, W = Lo::kWarpsPer, kRows = 4 / W;   // rows per lane
       const int dw = warp - 2 - Lo::kEpiWarps;
-      const int d = dw >> 1, r0 = (dw & 1) * 64 + lane;
+      const int d = dw / W, row0 = dw % W * (128 / W) + lane;
       // the codes to load next: K block kb of `unit` (past k1: of a later unit), at src
       int unit = pair, kb = 0, k1 = 0;
       const uint4* src = nullptr;
@@ -1127,7 +1146,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
             kb = k0 + over;
             const int rt1 = min(row_tile(unit_tile(unit) / p.TT), p.RT1 - 1);
             src = reinterpret_cast<const uint4*>(
-                      p.words + (static_cast<int64_t>(rt1) * p.KB + kb) * 512) + r0;
+                      p.words + (static_cast<int64_t>(rt1) * p.KB + kb) * 512) + row0;
             return;
           }
           over -= k1 - k0;
@@ -1135,13 +1154,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
         }
       };
       enter(d);
-      uint4 codes[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+      uint4 codes[kRows] = {};
       auto fetch = [&]() -> bool {               // the next round's codes; false past the last
         if (unit >= p.units) return false;
-        codes[0] = ldg_stream_u4(src);
-        codes[1] = ldg_stream_u4(src + 32);
-        kb += Lo::kDecoders;
-        src += Lo::kDecoders * (kCodeBytes / 16);
+#pragma unroll
+        for (int rr = 0; rr < kRows; ++rr) codes[rr] = ldg_stream_u4(src + 32 * rr);
+        kb += D;
+        src += D * (kCodeBytes / 16);
         if (kb >= k1) {
           const int over = kb - k1;
           unit += npairs;
@@ -1162,13 +1181,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
           break;
         }
         uint8_t* tile_a = sA + stage * kATileBytes;
-        decode_row_fma(codes[0], tile_a, r0);
-        decode_row_fma(codes[1], tile_a, r0 + 32);
+#pragma unroll
+        for (int rr = 0; rr < kRows; ++rr) decode_row_fma(codes[rr], tile_a, row0 + 32 * rr);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&full[stage]), 0));
         have = fetch();
-        stage += Lo::kDecoders;
+        stage += D;
         if (stage >= S_) stage -= S_, phase ^= 1;
       }
     }
@@ -1333,7 +1352,7 @@ bool make_tmap(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tokens per tile: one-SM tiles of 128 x 128 up to 128 tokens, CTA pairs with 256 x 256 above.
+// The token tile that the workspace's partial tiles are sized by.
 int pick_bn(int M) { return M <= 128 ? 128 : 256; }
 
 struct DeviceInfo {
@@ -1390,22 +1409,50 @@ void plan_phase(PhaseArgs& a, const DeviceInfo& d, int& grid) {
 }
 
 // The same on CTA pairs: units of 256 x BN tiles (or K splits of them), one pair per unit and
-// round.  A split's partial tiles are kept per 128-row tile, in the workspace planned for those.
-void plan_pairs(PhaseArgs& a, int BN, int pairs, int& grid) {
+// round.  BN and the K split are those with the least estimated time, in cycles: waves of units,
+// each a K block at a time (256 tokens: the MMAs' 512 cycles and a little; 128: 24 KiB of operands
+// per CTA from L2), the last tile's epilogue, and for a split the partial tiles' way through L2.
+// Measured (us per call; 256-token tiles and every split that fits, then this rule): 768 x 768 at
+// 700 tokens 61, 22; 4096 x 4096 at 200 tokens 88, 52, at 300 tokens 77, 68, at 1000 tokens 93, 94;
+// 2048 x 2048 at 200 tokens 75, 35; 8192 x 8192 at 256 tokens 116, 114 (128-token tiles: 133).
+constexpr int kRoundCycles[2] = {440, 540};       // per K block, BN = 128, 256
+constexpr int kEpilogueCycles[2] = {6000, 11000};
+constexpr int kSplitFixed[2] = {5000, 10000};     // a split tile, and each of its splits
+constexpr int kSplitEach[2] = {1500, 3000};
+
+int plan_pairs(PhaseArgs& a, int pairs) {
   a.RT1 = static_cast<int>(ceil_div(a.R, kBM));
   a.RT = static_cast<int>(ceil_div(a.R, 2 * kBM));
-  a.TT = static_cast<int>(ceil_div(a.M, BN));
   a.KB = static_cast<int>(ceil_div(a.K, kBK));
-  a.tiles = a.RT * a.TT;
-  a.KS = split_for(a.tiles, a.KB, std::min(pairs, kMaxSplitSms / 2));
-  a.kbs = static_cast<int>(ceil_div(a.KB, a.KS));
-  a.KS = static_cast<int>(ceil_div(a.KB, a.kbs));
+  int64_t best = INT64_MAX;
+  int best_bn = 128;
+  for (int w = 0; w < 2; ++w) {
+    const int bn = 128 << w, tt = static_cast<int>(ceil_div(a.M, bn)), tiles = a.RT * tt;
+    for (int ks = 1; ks <= std::min(kMaxSplits, a.KB / kMinSplitBlocks) || ks == 1; ++ks) {
+      const int kbs = static_cast<int>(ceil_div(a.KB, ks));
+      if (ks > 1 && (ceil_div(a.KB, kbs) != ks || tiles * ks > pairs || tiles > a.cnt_slots ||
+                     static_cast<int64_t>(a.RT1) * tt * ks * bn * kBM > a.part_floats))
+        continue;
+      const int64_t cost = ceil_div(static_cast<int64_t>(tiles) * ks, pairs) * kbs * kRoundCycles[w] +
+                           kEpilogueCycles[w] + (ks > 1 ? kSplitFixed[w] + ks * kSplitEach[w] : 0);
+      if (cost < best) {
+        best = cost;
+        best_bn = bn;
+        a.TT = tt;
+        a.tiles = tiles;
+        a.KS = ks;
+        a.kbs = kbs;
+      }
+    }
+  }
   a.units = a.tiles * a.KS;
-  grid = 2 * std::min(a.units, pairs);
+  return best_bn;
 }
 
 struct WsLayout {
   size_t z, u, zsum, cnt, part, z32, total;
+  int64_t part_floats;       // sizes of part and cnt
+  int cnt_slots;
 };
 
 // Partial tiles for split K, sized for any device with at most kMaxSplitSms SMs: a phase with
@@ -1434,6 +1481,8 @@ WsLayout ws_layout(int M, int d_in, int n_in, int n_out, int d_out, int act_bits
   L.cnt = off;
   off += round_up(max_tiles * 4, 256);
   L.part = off;
+  L.part_floats = slots * BN * kBM;
+  L.cnt_slots = static_cast<int>(round_up(max_tiles * 4, 256) / 4);
   off += static_cast<size_t>(slots) * BN * kBM * 4;
   L.z32 = off;
   if (act_bits > 0) off += round_up(static_cast<int64_t>(M) * n_in * 4, 256);
@@ -1491,33 +1540,51 @@ struct ChainedLaunch {
   ChainedLaunch(const ChainedLaunch&) = delete;
 };
 
-template <int PHASE, int BN>
-cudaError_t run_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs& a,
-                      const DeviceInfo& d, cudaStream_t s) {
-  const int pairs = std::min(resident_pairs<PHASE, BN>(d.dev), d.sms / 2);
-  if (pairs < 1) return cudaErrorLaunchOutOfResources;
-  int grid = 0;
-  plan_pairs(a, BN, pairs, grid);
-  using Lo = PairLayout<PHASE, BN>;
-  const ChainedLaunch l(grid, Lo::kThreads, Lo::kBytes, s);
-  return cudaLaunchKernelEx(&l.cfg, tc_pair_kernel<PHASE, BN>, tmA, tmB, a);
+// One phase of a call, planned with its tensor maps before anything is launched.
+struct PhasePlan {
+  CUtensorMap A, B;
+  int bn;                    // tokens per tile on CTA pairs; 0: the one-SM kernel
+  int grid;
+};
+
+// A: the weight operand (R x K; not used by the code product), B: the tokens (M x K).  CTA pairs for
+// budgets of two SMs and more.
+template <int PHASE>
+bool plan_call_phase(PhasePlan& pl, PhaseArgs& a, const void* A, const void* B,
+                     const DeviceInfo& d) {
+  if (d.sms >= 2) {
+    const int pairs = std::min({resident_pairs<PHASE, 128>(d.dev), resident_pairs<PHASE, 256>(d.dev),
+                                d.sms / 2});
+    if (pairs < 1) return false;
+    pl.bn = plan_pairs(a, pairs);
+    pl.grid = 2 * std::min(a.units, pairs);
+  } else {
+    if (prepare_kernel<PHASE, 128>(d.dev) != cudaSuccess) return false;
+    pl.bn = 0;
+    plan_phase<PHASE, 128>(a, d, pl.grid);
+  }
+  // a pair's CTAs load half of a tile's tokens each
+  if (!make_tmap(&pl.B, B, a.M, a.K, pl.bn ? pl.bn / 2 : 128)) return false;
+  if (PHASE == kCore) {
+    pl.A = pl.B;
+    return true;
+  }
+  return make_tmap(&pl.A, A, a.R, a.K, kBM);
 }
 
-// The token operand's box rows: a CTA pair's CTAs load half of a tile's tokens each.
-int token_box(int M, const DeviceInfo& d) { return d.sms >= 2 ? pick_bn(M) / 2 : 128; }
+template <int PHASE, int BN>
+cudaError_t launch_pairs(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s) {
+  using Lo = PairLayout<PHASE, BN>;
+  const ChainedLaunch l(pl.grid, Lo::kThreads, Lo::kBytes, s);
+  return cudaLaunchKernelEx(&l.cfg, tc_pair_kernel<PHASE, BN>, pl.A, pl.B, a);
+}
 
-// One phase, planned and launched: on CTA pairs, or on one SM for a budget of one.
 template <int PHASE>
-cudaError_t run_phase(const CUtensorMap& tmA, const CUtensorMap& tmB, PhaseArgs& a,
-                      const DeviceInfo& d, cudaStream_t s) {
-  if (d.sms >= 2)
-    return pick_bn(a.M) == 128 ? run_pairs<PHASE, 128>(tmA, tmB, a, d, s)
-                               : run_pairs<PHASE, 256>(tmA, tmB, a, d, s);
-  if (const cudaError_t e = prepare_kernel<PHASE, 128>(d.dev)) return e;
-  int grid = 0;
-  plan_phase<PHASE, 128>(a, d, grid);
-  const ChainedLaunch l(grid, threads_for<PHASE>(), Layout<PHASE, 128>::kBytes, s);
-  return cudaLaunchKernelEx(&l.cfg, tc_phase_kernel<PHASE, 128>, tmA, tmB, a);
+cudaError_t launch_phase(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s) {
+  if (pl.bn == 128) return launch_pairs<PHASE, 128>(pl, a, s);
+  if (pl.bn == 256) return launch_pairs<PHASE, 256>(pl, a, s);
+  const ChainedLaunch l(pl.grid, threads_for<PHASE>(), Layout<PHASE, 128>::kBytes, s);
+  return cudaLaunchKernelEx(&l.cfg, tc_phase_kernel<PHASE, 128>, pl.A, pl.B, a);
 }
 
 cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
@@ -1531,22 +1598,6 @@ cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const Devi
   return cudaLaunchKernelEx(&l.cfg, warps ? ff_round_kernel<32> : ff_round_kernel<kQuantThreads>,
                             static_cast<const float*>(an.out32), an.M, n_in, L,
                             static_cast<const uint32_t*>(an.amax), delta, zq, zsum);
-}
-
-// maps: {T_in, x, z, T_out^T, u}.  The core phase's A operand is the packed codes, so it gets
-// an unused map in that slot.
-fq_status run_forward(const CUtensorMap* maps, PhaseArgs* a, const DeviceInfo& d, int act_bits,
-                      float* delta, cudaStream_t s) {
-  a[1].zsum_tiles =
-      act_bits > 0 ? 1 : static_cast<int>(ceil_div(a[0].R, kBM));   // rounded: one exact sum
-  if (run_phase<kAnalysis>(maps[0], maps[1], a[0], d, s) != cudaSuccess) return FQ_ERR_CUDA;
-  if (act_bits > 0 && launch_round(a[0], a[1].K, act_bits, d, delta, a[0].out, a[0].zsum_part,
-                                   s) != cudaSuccess)
-    return FQ_ERR_CUDA;
-  if (run_phase<kCore>(maps[1], maps[2], a[1], d, s) != cudaSuccess ||
-      run_phase<kSynthesis>(maps[3], maps[4], a[2], d, s) != cudaSuccess)
-    return FQ_ERR_CUDA;
-  return FQ_OK;
 }
 
 // The dense product of the weight-reconstruction path: one synthesis-phase kernel with the
@@ -1566,6 +1617,8 @@ WsLayout dense_ws_layout(int M, int d_out) {
   L.cnt = off;
   off += round_up(max_tiles * 4, 256);
   L.part = off;
+  L.part_floats = slots * BN * kBM;
+  L.cnt_slots = static_cast<int>(round_up(max_tiles * 4, 256) / 4);
   off += static_cast<size_t>(slots) * BN * kBM * 4;
   L.total = off;
   return L;
@@ -1584,11 +1637,11 @@ fq_status launch_tc_dense(const void* x, int M, int d_in, const void* W, int d_o
   a.status = reinterpret_cast<int32_t*>(ws);
   a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
   a.part = reinterpret_cast<float*>(ws + L.part);
-  CUtensorMap mW, mX;
-  const DeviceInfo d = device_info();
-  if (!make_tmap(&mW, W, d_out, d_in, kBM) || !make_tmap(&mX, x, M, d_in, token_box(M, d)))
-    return FQ_ERR_CUDA;
-  return run_phase<kSynthesis>(mW, mX, a, d, s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
+  a.part_floats = L.part_floats;
+  a.cnt_slots = L.cnt_slots;
+  PhasePlan pl;
+  if (!plan_call_phase<kSynthesis>(pl, a, W, x, device_info())) return FQ_ERR_CUDA;
+  return launch_phase<kSynthesis>(pl, a, s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1625,6 +1678,8 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
     a[ph].status = status;
     a[ph].cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
     a[ph].part = reinterpret_cast<float*>(ws + L.part);
+    a[ph].part_floats = L.part_floats;
+    a[ph].cnt_slots = L.cnt_slots;
   }
   a[0].clear_status = 1;
   a[1].words = Cq.words;
@@ -1640,17 +1695,23 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
     a[1].delta = delta;
   }
 
-  // maps: T_in, x, z, T_out^T, u
   DeviceInfo d = device_info();
   if (max_sms > 0) d.sms = std::min(d.sms, max_sms);
-  const int box = token_box(M, d);
-  CUtensorMap maps[5];
-  if (!make_tmap(&maps[0], T_in, n_in, d_in, kBM) || !make_tmap(&maps[1], x, M, d_in, box) ||
-      !make_tmap(&maps[2], z, M, n_in, box) ||
-      !make_tmap(&maps[3], T_out_t, d_out, n_out, kBM) ||
-      !make_tmap(&maps[4], u, M, n_out, box))
+  a[1].zsum_tiles =
+      act_bits > 0 ? 1 : static_cast<int>(ceil_div(n_in, kBM));   // rounded: one exact sum
+  PhasePlan pl[3];
+  if (!plan_call_phase<kAnalysis>(pl[0], a[0], T_in, x, d) ||
+      !plan_call_phase<kCore>(pl[1], a[1], nullptr, z, d) ||
+      !plan_call_phase<kSynthesis>(pl[2], a[2], T_out_t, u, d))
     return FQ_ERR_CUDA;
-  return run_forward(maps, a, d, act_bits, delta, s);
+  if (launch_phase<kAnalysis>(pl[0], a[0], s) != cudaSuccess) return FQ_ERR_CUDA;
+  if (act_bits > 0 &&
+      launch_round(a[0], n_in, act_bits, d, delta, a[0].out, a[0].zsum_part, s) != cudaSuccess)
+    return FQ_ERR_CUDA;
+  if (launch_phase<kCore>(pl[1], a[1], s) != cudaSuccess ||
+      launch_phase<kSynthesis>(pl[2], a[2], s) != cudaSuccess)
+    return FQ_ERR_CUDA;
+  return FQ_OK;
 }
 
 fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq,
@@ -1679,6 +1740,8 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
     a[ph].status = status;
     a[ph].cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
     a[ph].part = reinterpret_cast<float*>(ws + L.part);
+    a[ph].part_floats = L.part_floats;
+    a[ph].cnt_slots = L.cnt_slots;
   }
   a[1].words = Cq.words;
   a[1].scale = reinterpret_cast<const __half*>(Cq.scale_f16);
@@ -1686,22 +1749,19 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
   a[1].gamma = gamma;
   a[2].transposed = 1;                           // the output's rows are those of W_hat
 
-  // maps: z (the code product's B; also the unused A slot), T_out^T, u
-  CUtensorMap maps[3];
+  a[1].zsum_tiles = static_cast<int>(ceil_div(n_in, kUnitRows));
   const DeviceInfo d = device_info();
-  const int box = token_box(M, d);
-  if (!make_tmap(&maps[0], z, M, n_in, box) ||
-      !make_tmap(&maps[1], T_out_t, d_out, n_out, kBM) ||
-      !make_tmap(&maps[2], u, M, n_out, box))
+  PhasePlan pl[2];
+  if (!plan_call_phase<kCore>(pl[0], a[1], nullptr, z, d) ||
+      !plan_call_phase<kSynthesis>(pl[1], a[2], T_out_t, u, d))
     return FQ_ERR_CUDA;
 
   unit_analysis_kernel<<<dim3(static_cast<unsigned>(ceil_div(d_in, kUnitCols)),
                               static_cast<unsigned>(ceil_div(n_in, kUnitRows))),
                          256, 0, s>>>(Tin, n_in, d_in, z, zsum, status);
   if (cudaGetLastError() != cudaSuccess) return FQ_ERR_CUDA;
-  a[1].zsum_tiles = static_cast<int>(ceil_div(n_in, kUnitRows));
-  return run_phase<kCore>(maps[0], maps[0], a[1], d, s) == cudaSuccess &&
-                 run_phase<kSynthesis>(maps[1], maps[2], a[2], d, s) == cudaSuccess
+  return launch_phase<kCore>(pl[0], a[1], s) == cudaSuccess &&
+                 launch_phase<kSynthesis>(pl[1], a[2], s) == cudaSuccess
              ? FQ_OK
              : FQ_ERR_CUDA;
 }

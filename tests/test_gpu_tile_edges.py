@@ -95,3 +95,18 @@ def test_rounded_activations_at_both_kernel_forms(M):
     off = got != torch.round(q)
     assert ((q - torch.floor(q) - 0.5).abs()[off] < 1e-5).all()
     assert got.abs().max() == 7
+
+
+@pytest.mark.parametrize("M", [90, 150, 300])
+def test_prefill_k_splits_repeat(M):
+    """fc2 (848 and 3392 coefficients, K up to 53 blocks) at batches whose phases split K: calls on
+    one workspace repeat bitwise (the splits' counters are left at zero) and match the oracle."""
+    L = oracle_layer("vit_b16_mlp", "fc2")
+    X = activations("vit_b16_mlp", "fc2", M)
+    D = DeviceLayer(L)
+    nb = fq.fq_workspace_bytes(M, L.d_in, L.n_in, L.n_out, L.d_out)
+    ws = torch.zeros(nb, dtype=torch.uint8, device=DEV)
+    first = D.forward(X, ws=ws)
+    assert_parity(first, reference(L, X), 1e-2)
+    for _ in range(3):
+        np.testing.assert_array_equal(D.forward(X, ws=ws), first)
