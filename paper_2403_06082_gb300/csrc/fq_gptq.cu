@@ -273,16 +273,17 @@ constexpr int kNB = 32;           // block: a warp's lanes
 // Block column b .. b + nb - 1: factor the diagonal block, K_bb = L L^T, and solve L Y = B by forward
 // substitution, a column of B per lane: CTA 0 for B = I, the inverse of L, which goes to X; CTA c > 0
 // for B = the transpose of 32 rows below the block, K_ib <- K_ib L^-T in place.  Every CTA factors
-// the diagonal block for itself (one warp, a row per lane: a pivot's chain is a division and the
-// row's multiply-adds, no barriers), which saves a launch and its latency per block; nothing
-// rewrites the diagonal block.  Loops stay rolled: unrolled code runs once per launch and waits
-// for its instructions.
+// the diagonal block for itself, which saves a launch and its latency per block; nothing rewrites
+// the diagonal block.  The factorization is a chain of 32 pivots: the warp that owns column j + 1
+// updates it first and divides by its pivot while the other warps update the columns after it.
+// Loops stay rolled: unrolled code runs once per launch and waits for its instructions.
 __global__ void __launch_bounds__(256) chol_panel_kernel(double* __restrict__ K, int n, int b,
                                                          int nb, double* __restrict__ X,
                                                          int32_t* __restrict__ status) {
   __shared__ double D[kNB][kNB + 1];      // the block, then its factor
   __shared__ double Y[kNB][kNB + 1];      // the right-hand sides, a column per lane
   __shared__ double inv_s[kNB];
+  __shared__ double m_s[2][kNB];          // column j over its pivot, for the step at hand and the next
   const int tid = threadIdx.x, lane = tid & 31, wr = tid >> 5;
   const bool inverse = blockIdx.x == 0;
   const int r0 = b + nb + (static_cast<int>(blockIdx.x) - 1) * kNB;   // this CTA's rows
@@ -297,15 +298,22 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(double* __restrict__ K,
       Y[j][i] = (r0 + i < n && j < nb) ? K[static_cast<int64_t>(r0 + i) * n + b + j] : 0.0;
   }
   __syncthreads();
-  if (tid < 32) {
-    // right-looking, unscaled: D_ik -= D_ij D_kj / piv_j
-    for (int j = 0; j < kNB; ++j) {
-      const double m = D[lane][j] * (1.0 / D[j][j]);
-#pragma unroll 4
-      for (int k = j + 1; k < kNB; ++k)
-        if (lane >= k) D[lane][k] = fma(-m, D[k][j], D[lane][k]);
-      __syncwarp();
+  // right-looking, unscaled, a row per lane: D_ik -= (D_ij / piv_j) D_kj, column k by warp k mod 8
+  if (wr == 0) m_s[0][lane] = D[lane][0] * (1.0 / D[0][0]);
+  __syncthreads();
+  for (int j = 0; j < kNB; ++j) {
+    const double m = m_s[j & 1][lane];
+    const int first = j + 1 + ((wr - (j + 1)) & 7);            // this warp's first column after j
+    for (int k = first; k < kNB; k += 8) {
+      if (lane >= k) D[lane][k] = fma(-m, D[k][j], D[lane][k]);
+      if (k == j + 1) {
+        __syncwarp();
+        m_s[k & 1][lane] = D[lane][k] * (1.0 / D[k][k]);
+      }
     }
+    __syncthreads();
+  }
+  if (tid < 32) {
     // a pivot that is not positive: the damped H was not positive definite
     const double piv = D[lane][lane];
     if (inverse && !(piv > 0.0)) report(status, FQ_ERR_DEVICE_CHECK);
