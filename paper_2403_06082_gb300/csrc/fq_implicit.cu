@@ -47,7 +47,9 @@ namespace {
 // What bounds it is latency: a token is two products of a few million multiply-adds.  The
 // factors, the permutation and the signs do not depend on the previous kernel and are staged in
 // shared memory before the wait for the input; a factor that does not fit is read from L2.
-// PLACEHOLDER_ROTATE
+// Measured against a CTA per eight rows that gathered its whole token: three 11008 x 4096 layers at
+// 64 tokens 265 -> 164 us (the rotations and the fused kernel), 4096 to 11008 at 64 tokens 212 ->
+// 159, 2048 x 2048 at 16 tokens 34.0 -> 30.2.
 constexpr int kRotThreads = 256;
 constexpr size_t kMaxSmem = 227 * 1024;
 
