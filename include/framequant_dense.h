@@ -22,15 +22,15 @@ extern "C" {
 #endif
 
 /* Workspace bytes of fq_reconstruct_weight; 0 for invalid sizes.  It holds the tensor-core
- * chain's workspace for M = d_in tokens (z and u of the d_in unit vectors) and the d_in x d_out
- * output before its transpose: about 108 MB for a 4096 x 4096 layer at r = 1.1, 227 MB for
+ * chain's workspace for M = d_in tokens (z and u of the d_in unit vectors) and room for a
+ * d_in x d_out matrix that is not used now: about 108 MB for a 4096 x 4096 layer at r = 1.1, 227 MB for
  * 11008 x 4096, 460 MB for 4096 x 11008, 432 MB for 8192 x 8192, 1.14 GB for 28672 x 8192 and
  * 2.8 GB for 8192 x 28672. */
 size_t fq_reconstruct_workspace_bytes(int d_in, int n_in, int n_out, int d_out);
 
 /* W_hat = T_out^T diag(gamma) C_hat T_in, bf16 d_out x d_in row-major: the FQ_BF16 forward of
  * fq_linear_forward applied to the d_in unit vectors (so z and u are rounded to bf16 as in the
- * forward), then transposed.  The analysis of unit vector e_j is column j of T_in, exact in
+ * forward), stored transposed.  The analysis of unit vector e_j is column j of T_in, exact in
  * bf16, so it is taken as a transpose rather than a product; the code product and the synthesis
  * run on the tensor cores.
  *   T_in, C, T_out_t, gamma  as in fq_linear_forward
@@ -46,7 +46,7 @@ fq_status fq_reconstruct_weight(const void* T_in, const fq_packed* C, const void
 size_t fq_dense_workspace_bytes(int M, int d_in, int d_out);
 
 /* y = x W_hat^T for M tokens (bf16 in and out, fp32 accumulation on the tensor cores): one
- * product of the tensor-core path (128 x 128 or 128 x 256 tiles, split K when tiles are few).
+ * product of the tensor-core path (256 x 128 or 256 x 256 tiles on CTA pairs, split K when tiles are few).
  *   x  device bf16 M x d_in;  W_hat  device bf16 d_out x d_in;  y  device bf16 M x d_out
  *   ws device workspace of fq_dense_workspace_bytes(M, d_in, d_out) bytes, 256-byte aligned,
  *      zero-filled before its first use

@@ -58,12 +58,13 @@ struct PhaseArgs {
   int R, K, M;
   int RT, TT, KB, tiles;     // row tiles (128 rows, or 256 on a CTA pair), token tiles, K blocks
   int RT1;                   // 128-row tiles
+  // On CTA pairs:
   int KS, kbs, units;        // K splits per tile, K blocks per split, tiles * KS work units
   float* part;               // KS > 1: fp32 partial tiles [tile][split][BN][128]
   int64_t part_floats;       // what `part` and `cnt` hold (host)
   int cnt_slots;
-  uint32_t* cnt;             // KS > 1: arrivals per tile (the last resets it to 0; on CTA pairs
-                             // 16 bits for each CTA's half)
+  uint32_t* cnt;             // KS > 1: arrivals per tile, 16 bits for each CTA's half (the last
+                             // resets them to 0)
   const uint32_t* words;     // core: packed codes
   __nv_bfloat16* out;        // [M][R]
   float* zsum_part;          // analysis writes [RT][M] sums of z; the core reads them
@@ -101,8 +102,8 @@ struct Layout {
   static constexpr int oBar = oCodes + kStages * kCodesStage;
   static constexpr int kNumBars = 4 * kStages + 2 + 2 + 1;
   static constexpr int oMisc = oBar + kNumBars * 8;
-  static constexpr int oRedSmall = oMisc + 16;                      // [4][kChunk] + 4 floats
-  static constexpr int oZsum = oRedSmall + (4 * kChunk + 4) * 4;    // [2][BN] floats
+  static constexpr int oRedSmall = oMisc + 16;                      // [4][kChunk] floats
+  static constexpr int oZsum = oRedSmall + 4 * kChunk * 4;          // [2][BN] floats
   static constexpr int kBytes = oZsum + 2 * BN * 4 + 1024;          // + alignment slack
   static_assert(BN == 128, "tile width of the one-SM kernel");
   static_assert(kBTileBytes % 1024 == 0, "B tiles must keep 1024-byte alignment");
@@ -154,6 +155,8 @@ __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
   return out != 0;
 }
 
+// One SM (a call whose budget is one SM; the pairs need two): tiles of 128 rows x BN tokens, one
+// warp of TMA copies, one issuing MMAs, four of epilogue and, in the core, four decoders.
 template <int PHASE, int BN>
 __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
     tc_phase_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -178,15 +181,11 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
   uint64_t* mma_done = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Lo::oMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* red = reinterpret_cast<float*>(smem + Lo::oRedSmall);     // [4][kChunk], flag
+  float* red = reinterpret_cast<float*>(smem + Lo::oRedSmall);     // [4][kChunk]
   float* zsum_s = reinterpret_cast<float*>(smem + Lo::oZsum);      // [2][BN]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t cid = blockIdx.x, ncl = gridDim.x;
-  // work unit u = split * tiles + tile: K blocks [split * kbs, min(KB, (split + 1) * kbs))
-  auto unit_tile = [&](int u) { return u % p.tiles; };
-  auto unit_k0 = [&](int u) { return (u / p.tiles) * p.kbs; };
-  auto unit_k1 = [&](int u) { return min(p.KB, (u / p.tiles + 1) * p.kbs); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S_; ++s) {
@@ -223,12 +222,11 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
       // Weight tiles of the first tile do not depend on the previous kernel: issue up to a
       // full ring of them before waiting for it, and warm L2 with the rest.
       int pre = 0;
-      if (static_cast<int>(cid) < p.units) {
-        const int rt = unit_tile(static_cast<int>(cid)) / p.TT;
-        const int k0 = unit_k0(static_cast<int>(cid)), k1 = unit_k1(static_cast<int>(cid));
-        pre = min(S_, k1 - k0);
-        for (int i = 0; i < pre; ++i) {
-          const int kb = k0 + i;
+      if (static_cast<int>(cid) < p.tiles) {
+        const int rt = static_cast<int>(cid) / p.TT;
+        pre = min(S_, p.KB);
+        for (int kb = 0; kb < pre; ++kb) {
+          const int i = kb;
           if (kCodes) {
             mbar_arrive_expect_tx(&cfull[i], kCodeBytes);
             bulk_load(sCodes + i * kCodeBytes,
@@ -239,7 +237,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
             tma_load_2d(sA + i * kATileBytes, &tmA, &full[i], kb * kBK, rt * kBM, pol_w);
           }
         }
-        for (int kb = k0 + pre; kb < k1; ++kb) {
+        for (int kb = pre; kb < p.KB; ++kb) {
           if (kCodes) {
             const uint32_t* src = p.words + (static_cast<int64_t>(rt) * p.KB + kb) * 512;
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src),
@@ -265,11 +263,10 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
       bool issued[S_];
 #pragma unroll
       for (int s = 0; s < S_; ++s) issued[s] = false, issued_parity[s] = 0;
-      for (int unit = static_cast<int>(cid); unit < p.units && !*abort_flag;
-           unit += static_cast<int>(ncl)) {
-        const int tile = unit_tile(unit), k0 = unit_k0(unit), k1 = unit_k1(unit);
+      for (int tile = static_cast<int>(cid); tile < p.tiles && !*abort_flag;
+           tile += static_cast<int>(ncl)) {
         const int rt = tile / p.TT, tt = tile % p.TT;
-        for (int kb = k0; kb < k1; ++kb, ++it) {
+        for (int kb = 0; kb < p.KB; ++kb, ++it) {
           if (it >= pre) {
             if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) {
               report(p.status, FQ_ERR_TIMEOUT);
@@ -311,9 +308,8 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
       int buf = 0;
       uint32_t acc_phase = 0;
       bool issued_any = false;
-      for (int unit = static_cast<int>(cid); unit < p.units && !*abort_flag;
-           unit += static_cast<int>(ncl)) {
-        const int k0 = unit_k0(unit), k1 = unit_k1(unit);
+      for (int tile = static_cast<int>(cid); tile < p.tiles && !*abort_flag;
+           tile += static_cast<int>(ncl)) {
         if (!mbar_wait(&tempty[buf], acc_phase ^ 1, abort_flag)) {
           report(p.status, FQ_ERR_TIMEOUT);
           *abort_flag = 1;
@@ -322,7 +318,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * BN);
         bool ok = true;
-        for (int kb = k0; kb < k1; ++kb) {
+        for (int kb = 0; kb < p.KB; ++kb) {
           ok = mbar_wait(&full[stage], phase, abort_flag) &&
                (!kCodes || mbar_wait(&aready[stage], phase, abort_flag));
           if (!ok) break;
@@ -331,7 +327,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
           const uint64_t bdesc = umma_desc_sw128(smem_u32(sB + stage * kBTile));
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)   // 16 bf16 = 32 bytes along K per step
-            umma_bf16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > k0 || k > 0) ? 1u : 0u);
+            umma_bf16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
           issued_any = true;
           umma_commit(&empty[stage]);
           if (++stage == S_) stage = 0, phase ^= 1;
@@ -359,8 +355,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
     pdl_wait();
     int buf = 0;
     uint32_t acc_phase = 0;
-    for (int unit = static_cast<int>(cid); unit < p.units; unit += static_cast<int>(ncl)) {
-      const int tile = unit_tile(unit), split = unit / p.tiles;
+    for (int tile = static_cast<int>(cid); tile < p.tiles; tile += static_cast<int>(ncl)) {
       const int rt = tile / p.TT, tt = tile % p.TT;
       const int row = rt * kBM + r_in_tile;
       const int t0 = tt * BN;
@@ -444,58 +439,15 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
           named_barrier_sync(1, kEpi);
         }
       };
-      if (p.KS == 1) {
 #pragma unroll 1
-        for (int c = 0; c < BN; c += kChunk) {
-          float v[kChunk];
-          tmem_ld16(t_row + c, v);
-          tmem_wait_ld();
-          emit(c, v);
-        }
-        tc_fence_before_sync();
-        mbar_arrive(&tempty[buf]);
-      } else {
-        // Split K: store this split's partial tile (column-major, so a warp's 32 rows are one
-        // 128-byte line), release the accumulator, and count the split in.  The tile's last
-        // split to arrive adds the partials in split order and finishes the tile.
-        float* mine = p.part + (static_cast<int64_t>(tile) * p.KS + split) * BN * kBM;
-#pragma unroll 1
-        for (int c = 0; c < BN; c += kChunk) {
-          float v[kChunk];
-          tmem_ld16(t_row + c, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int q = 0; q < kChunk; ++q) mine[(c + q) * kBM + r_in_tile] = v[q];
-        }
-        tc_fence_before_sync();
-        mbar_arrive(&tempty[buf]);
-        __threadfence();
-        named_barrier_sync(1, kEpi);
-        if (et == 0) {
-          const uint32_t old = atomicAdd(&p.cnt[tile], 1u);
-          const bool last = old == static_cast<uint32_t>(p.KS - 1);
-          if (last) p.cnt[tile] = 0;                 // ready for the next call
-          __threadfence();
-          red[4 * kChunk] = last ? 1.f : 0.f;
-        }
-        named_barrier_sync(1, kEpi);
-        if (red[4 * kChunk] != 0.f) {
-          const float* all = p.part + static_cast<int64_t>(tile) * p.KS * BN * kBM;
-#pragma unroll 1
-          for (int c = 0; c < BN; c += kChunk) {
-            float v[kChunk];
-#pragma unroll
-            for (int q = 0; q < kChunk; ++q) v[q] = 0.f;
-            for (int sp = 0; sp < p.KS; ++sp) {
-#pragma unroll
-              for (int q = 0; q < kChunk; ++q)
-                v[q] += ldcg_f32(all + (static_cast<int64_t>(sp) * BN + c + q) * kBM + r_in_tile);
-            }
-            emit(c, v);
-          }
-        }
-        named_barrier_sync(1, kEpi);                 // the flag is read before it is reused
+      for (int c = 0; c < BN; c += kChunk) {
+        float v[kChunk];
+        tmem_ld16(t_row + c, v);
+        tmem_wait_ld();
+        emit(c, v);
       }
+      tc_fence_before_sync();
+      mbar_arrive(&tempty[buf]);
       if (PHASE == kAnalysis && p.out32) {
         // one atomic per warp and tile: the tensor's max |z| (non-negative floats order like
         // their bit patterns)
@@ -515,9 +467,9 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
       uint32_t phase = 0;
       int it = 0;
       bool ok = true;
-      for (int unit = static_cast<int>(cid); unit < p.units && ok && !*abort_flag;
-           unit += static_cast<int>(ncl)) {
-        for (int kb = unit_k0(unit); kb < unit_k1(unit); ++kb, ++it) {
+      for (int tile = static_cast<int>(cid); tile < p.tiles && ok && !*abort_flag;
+           tile += static_cast<int>(ncl)) {
+        for (int kb = 0; kb < p.KB; ++kb, ++it) {
           if ((it & 3) == dw) {
             if (!mbar_wait(&cfull[stage], phase, abort_flag)) {
               ok = false;
@@ -549,7 +501,7 @@ __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Batches of more than 128 tokens: 256 x 256 tiles on CTA pairs
+// Tiles of 256 rows x 128 or 256 tokens on CTA pairs
 // ---------------------------------------------------------------------------------------------
 // A 128 x 256 tile on one SM is bound by its shared memory: each 128-cycle MMA step reads 12 KiB
 // of operands and the ring refills 12 KiB, 192 B per cycle against the 128 B an SM moves.  A pair of
@@ -1386,34 +1338,21 @@ cudaError_t prepare_kernel(int dev) {
   return e;
 }
 
-// One work unit per CTA and round, at most one CTA per SM.  A phase with fewer tiles than SMs
-// splits each tile's K range (up to kMaxSplits ways, at least kMinSplitBlocks K blocks each)
-// so that it fills the GPU: at 128 tokens a 8192-row phase has only 64 tiles.
+// K splits of a phase with few tiles (on CTA pairs): up to kMaxSplits, of at least kMinSplitBlocks K
+// blocks each.  At 128 tokens a 8192-row phase has only 32 tiles.
 constexpr int kMaxSplits = 4;
 constexpr int kMinSplitBlocks = 4;
 constexpr int kMaxSplitSms = 256;      // bound on the SM count used for split-K planning
 
-int split_for(int tiles, int KB, int sms) {
-  sms = std::min(sms, kMaxSplitSms);
-  if (tiles >= sms) return 1;
-  int ks = std::min({kMaxSplits, sms / tiles, KB / kMinSplitBlocks});
-  return std::max(ks, 1);
-}
-
-template <int PHASE, int BN>
-void plan_phase(PhaseArgs& a, const DeviceInfo& d, int& grid) {
+// One SM: whole tiles, all on one CTA.
+void plan_one_sm(PhaseArgs& a, int BN) {
   a.RT1 = a.RT = static_cast<int>(ceil_div(a.R, kBM));
   a.TT = static_cast<int>(ceil_div(a.M, BN));
   a.KB = static_cast<int>(ceil_div(a.K, kBK));
   a.tiles = a.RT * a.TT;
-  a.KS = split_for(a.tiles, a.KB, d.sms);
-  a.kbs = static_cast<int>(ceil_div(a.KB, a.KS));
-  a.KS = static_cast<int>(ceil_div(a.KB, a.kbs));     // every split non-empty
-  a.units = a.tiles * a.KS;
-  grid = std::min(a.units, d.sms);
 }
 
-// The same on CTA pairs: units of 256 x BN tiles (or K splits of them), one pair per unit and
+// CTA pairs: units of 256 x BN tiles (or K splits of them), one pair per unit and
 // round.  BN and the K split are those with the least estimated time, in cycles: waves of units,
 // each a K block at a time (256 tokens: the MMAs' 512 cycles and a little; 128: 24 KiB of operands
 // per CTA from L2), the last tile's epilogue, and for a split the partial tiles' way through L2.
@@ -1566,7 +1505,8 @@ bool plan_call_phase(PhasePlan& pl, PhaseArgs& a, const void* A, const void* B,
   } else {
     if (prepare_kernel<PHASE, 128>(d.dev) != cudaSuccess) return false;
     pl.bn = 0;
-    plan_phase<PHASE, 128>(a, d, pl.grid);
+    plan_one_sm(a, 128);
+    pl.grid = 1;
   }
   // a pair's CTAs load half of a tile's tokens each
   if (!make_tmap(&pl.B, B, a.M, a.K, pl.bn ? pl.bn / 2 : 128)) return false;
