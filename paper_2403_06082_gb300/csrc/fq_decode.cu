@@ -24,26 +24,34 @@
 // next tasks (and warms L2 with this CTA's later code blocks, and with its synthesis tiles when
 // the layer is small enough) while activations are still being produced.
 //
-// sum(z), needed by the core's zero term: in launches whose core tasks have more than
-// kSumMmaBlocks K blocks per CTA it comes from the tensor cores (kSums), whose core rounds issue
-// their MMAs once more with a constant A tile of ones, into columns beside the accumulator, so
-// that every accumulator row also holds the token sums over the CTA's K range.  Shorter tasks
-// take it in the epilogue over the bf16 z of their K range, read from global memory once the
-// slices' ready flags are seen, which costs them less than the extra MMAs and accumulator reads.
-// The two are separate kernels: a small launch is bound by latency, and carrying the other's
-// code cost it 2-8%.  Measured, us per call (epilogue sums, tensor-core sums): 4096 x 4096 at 24
-// tokens 30.4, 28.4; 11008 x 4096 at 48 tokens 97.3, 84.7; q|k|v at 16 tokens 51.1, 48.2; with 8 K
-// blocks per CTA at 34 tokens 35.1, 37.0.
+// sum(z), needed by the core's zero term, has three forms (SumForm), each the fastest in its range:
+//   kSumEpilogue  (16 or 32 tokens, core tasks of at most kSumMmaBlocks K blocks per CTA) the
+//                 epilogue adds the bf16 z of its K range, read from global memory once the slices'
+//                 ready flags are seen;
+//   kSumOnes      (16 or 32 tokens, longer tasks) the core rounds issue their MMAs once more with a
+//                 constant A tile of ones, into columns beside the accumulator, so that every
+//                 accumulator row also holds the token sums over the CTA's K range;
+//   kSumWarp      (64 tokens) warp 11 adds up the z tile of every core round in shared memory (a 16
+//                 x 16 matrix instruction with ones) beside the MMAs that read the same tile.  At 64
+//                 tokens a round is bound by its MMAs, which the ones would double, and without the
+//                 ones' tile and columns there is room for a sixth stage and a second issuer.
+// They are separate kernels: a small launch is bound by latency, and carrying another's code cost
+// it 2-8%.  Measured, us per call: (kSumEpilogue, kSumOnes) 4096 x 4096 at 24 tokens 30.4, 28.4;
+// q|k|v at 16 tokens 51.1, 48.2; with 8 K blocks per CTA at 34 tokens 35.1, 37.0; (the faster of
+// those with one issuer, kSumWarp) 4096 x 4096 at 48 tokens 35.4, 33.4; 11008 x 4096 at 64 tokens
+// 85.2, 81.8; 4096 x 11008 at 40 tokens 80.1, 75.7; 768 to 3072 at 34 tokens 24.1, 23.2; (the faster,
+// kSumWarp at up to 32 tokens) 256 x 256 at 8 tokens 12.0, 12.3; 4096 x 4096 at 24 tokens 28.0, 28.3;
+// q|k|v at 16 tokens 48.1, 48.4; gate|up at 16 tokens 112.8, 111.6, at 32 tokens 116.5, 116.6.
 //
 // The workspace header holds the generation counter and the tiles' ready flags; a zero-filled
 // header is a valid start and every call leaves it valid for the next (flags keep
 // generations that are all in the past; the last CTA to finish advances the generation).
 //
 // Warps: 0 weight (A) producer, 1 TMEM owner + MMA issuer 0, 2-5 epilogue (thread = tile row),
-// 11 the tile of ones,
+// 11 the tile of ones or the sums of z,
 // 6 activation (B) producer, 7-10 code decoders (ring stage s -> decoder s mod 4; one per SM
-// sub-partition, since the decode is issue-bound), and for 16 or 32 tokens 12, 14, 15 MMA
-// issuers 1-3 (one issuer per SM sub-partition).
+// sub-partition, since the decode is issue-bound), 12 MMA issuer 1, and for 16 or 32
+// tokens 14 and 15 MMA issuers 2 and 3 (one issuer per SM sub-partition).
 //
 // Ring protocol.  A parity wait on an mbarrier is only exact when its waiter is neither ahead
 // of the barrier nor two or more phases behind it, so each barrier's waiters take part in
@@ -54,7 +62,10 @@
 //             whose arrival on fullA[s] the round's MMAs (and so the stage's next core round)
 //             wait for;
 //   fullA[s]  (the A tile is in place: the weight tile's bytes, or the decoder's arrival in
-//             core rounds), fullB[s]  the issuer that owns s, which commits empty[s].
+//             core rounds), fullB[s]  the issuer that owns s, which commits empty[s];
+//   fullB[s]  with kSumWarp also warp 11, in every round, which then arrives on empty[s] (two
+//             arrivals per phase; marking only the core rounds for it, and letting the activation
+//             producer arrive in the others, was 1 to 4% slower).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -84,19 +95,21 @@ constexpr int kChunk = 16;
 // per SM sub-partition, each own the ring stages s = q (mod NI) and accumulate their K blocks
 // into their own accumulator, which the epilogue adds.  Owning stages (not K blocks) keeps
 // every barrier of a stage waited for by one thread, in phase order.  With 64 tokens the
-// epilogue's registers do not leave room for the extra warps: one issuer.
+// epilogue's registers leave room for one more warp: two issuers.
 // With four issuers the code decode also gets a second warp per stage (warps 16-19), each of
-// a stage's two decoders expanding half of its rows; with 64 tokens neither fits.
+// a stage's two decoders expanding half of its rows.
 template <int BN>
 struct DecCfg {
-  static constexpr int NI = BN <= 32 ? 4 : 1;
+  static constexpr int NI = BN <= 32 ? 4 : 2;
   static constexpr bool kPairs = NI == 4;
-  static constexpr int kThreads = NI == 4 ? 640 : 384;
+  static constexpr int kThreads = NI == 4 ? 640 : 416;
 };
-// warp -> issuer index (warps 1, 12, 14, 15: sub-partitions 1, 0, 2, 3), -1 for other roles
+// warp -> issuer index (warps 1, 12, 14, 15, or the first two: sub-partitions 1, 0, 2, 3), -1 for
+// other roles
 __host__ __device__ constexpr int issuer_of(int warp, int ni) {
   return warp == 1 ? 0
-                   : (ni == 4 ? (warp == 12 ? 1 : (warp == 14 ? 2 : (warp == 15 ? 3 : -1))) : -1);
+                   : (ni == 4 ? (warp == 12 ? 1 : (warp == 14 ? 2 : (warp == 15 ? 3 : -1)))
+                              : (warp == 12 ? 1 : -1));
 }
 // L2 warming.  When a layer's code blocks fit kL2PrefetchBudget, each CTA prefetches the code
 // blocks of its later tasks after issuing its first task's loads.  When the code blocks and
@@ -162,8 +175,12 @@ struct DecSched {
   uint16_t task[kMaxSched];          // layer << 14 | phase << 12 | row tile
 };
 
-template <int BN, bool kSums>
+// where sum(z) comes from
+enum SumForm : int { kSumEpilogue, kSumOnes, kSumWarp };
+
+template <int BN, SumForm F>
 struct DecLayout {
+  static constexpr bool kSums = F == kSumOnes;
   static constexpr int kBTile = BN * kBK * 2;
   static constexpr int kStage = kATile + kBTile;
   static constexpr int kRecvRow = BN + 4;                     // floats per received row
@@ -181,14 +198,16 @@ struct DecLayout {
   static constexpr int oOnes = oB + kStages * kBTile;        // kSums: an A tile of ones
   static constexpr int oRecv = oOnes + (kSums ? kATile : 0);   // two receive buffers
   static constexpr int oBar = oRecv + 2 * kRecv;
-  static constexpr int kBars = 4 * kStages + 11;
+  // (kSumWarp: a spare one, so that the sums are 16-byte aligned)
+  static constexpr int kBars = 4 * kStages + (F == kSumWarp ? 12 : 11);
   static constexpr int oMisc = oBar + kBars * 8;
-  static constexpr int oZs = oMisc + 32;                     // [BN] floats
-  static constexpr int oZsPart = oZs + BN * 4;               // [128] floats
+  static constexpr int oZs = oMisc + 32;                     // [BN] floats (kSumWarp: two)
+  static constexpr int oZsPart = oZs + (F == kSumWarp ? 2 : 1) * BN * 4;   // [128] floats
   static constexpr int kBytes = oZsPart + kEpi * 4 + 1024;
   static_assert(kBTile % 1024 == 0, "B tiles keep 1024-byte alignment");
   static_assert(kStages >= 3 && kStages % NI == 0, "pipeline depth, stage ownership");
   static_assert(kAccCols <= 512, "accumulator columns");
+  static_assert(F != kSumWarp || oZs % 16 == 0, "sums read as float4");
   static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
 };
 
@@ -196,9 +215,41 @@ __device__ __forceinline__ uint4 ldcg_u4(const __nv_bfloat16* p) {
   return __ldcg(reinterpret_cast<const uint4*>(p));
 }
 
-// Launches whose core tasks have more than this many K blocks per CTA take sum(z) from the tensor
-// cores (kSums).
+// Launches of 16 or 32 tokens whose core tasks have more than this many K blocks per CTA take sum(z)
+// from the MMAs (kSumOnes).
 constexpr int kSumMmaBlocks = 8;
+
+// Adds to s[m][0] and s[m][2] the sums over K of rows 16 m + lane / 4 and + 8 of a B tile (BN rows of
+// 64 bf16, 128-byte swizzle): the product with a matrix of ones, fp32 sums, the four K steps in two
+// chains.
+template <int BN>
+__device__ __forceinline__ void add_row_sums(uint32_t tile, int lane, float (&s)[2][BN / 16][4]) {
+  const int r = lane & 15, hi = lane >> 4;             // ldmatrix: this lane's row and 16-byte half
+  constexpr int kM = BN / 16 < 2 ? 1 : 2;              // row groups at a time (registers)
+#pragma unroll
+  for (int m0 = 0; m0 < BN / 16; m0 += kM) {
+    uint32_t f[kM][4][4];
+#pragma unroll
+    for (int m = 0; m < kM; ++m)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(f[m][k][0]), "=r"(f[m][k][1]), "=r"(f[m][k][2]), "=r"(f[m][k][3])
+                     : "r"(tile + (16 * (m0 + m) + r) * 128 + (((2 * k + hi) ^ (r & 7)) << 4))
+                     : "memory");
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int m = 0; m < kM; ++m) {
+        float(&c)[4] = s[k & 1][m0 + m];
+        asm volatile(
+            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, "
+            "{%4, %5, %6, %7}, {%8, %8}, {%0, %1, %2, %3};"
+            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+            : "r"(f[m][k][0]), "r"(f[m][k][1]), "r"(f[m][k][2]), "r"(f[m][k][3]), "r"(0x3F803F80u));
+      }
+  }
+}
 
 struct Task {
   int l, p, tile;
@@ -267,11 +318,12 @@ __device__ __forceinline__ void note_timeout(int32_t* status, int role, int task
   }
 }
 
-template <int BN, bool kSums>
+template <int BN, SumForm F>
 __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
     decode_layer_kernel(const __grid_constant__ DecMaps maps, const __grid_constant__ DecArgs a,
                         const __grid_constant__ DecSched sched) {
-  using Lo = DecLayout<BN, kSums>;
+  using Lo = DecLayout<BN, F>;
+  constexpr bool kSums = Lo::kSums;
   constexpr int S_ = Lo::kStages;
   constexpr int kBTile = Lo::kBTile;
   constexpr int NI = Lo::NI;
@@ -314,15 +366,16 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
 
   if (warp == 0) {
     // the barriers, initialised lane-parallel: fullA, fullB, empty, cfull (count 1), tfull[2]
-    // (one commit per issuer), tempty[2] (kEpi), mma_done[4] (1), recv_bar[2] (1), ones_bar (1)
+    // (one commit per issuer), tempty[2] (kEpi), mma_done[4] (1), recv_bar[2] (1), ones_bar (1);
+    // with kSumWarp empty and tfull take warp 11's arrival too
     // fullA takes two arrivals per round when a stage has two decoders: the weight
     // producer's two (with the tile's bytes), or one from each decoder
     constexpr uint32_t kFullA = DecCfg<BN>::kPairs ? 2u : 1u;
     for (int b = lane; b < Lo::kBars; b += 32) {
       const int r = b - 4 * S_;
       const uint32_t cnt = b < S_ ? kFullA
-                                  : (r < 0 ? 1u
-                                           : (r < 2 ? static_cast<uint32_t>(NI)
+                                  : (r < 0 ? (F == kSumWarp && b >= 2 * S_ && b < 3 * S_ ? 2u : 1u)
+                                           : (r < 2 ? static_cast<uint32_t>(NI + (F == kSumWarp))
                                                     : (r < 4 ? static_cast<uint32_t>(kEpi)
                                                              : 1u)));
       mbar_init(&fullA[b], cnt);
@@ -750,6 +803,48 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) mbar_arrive(ones_bar);
+  } else if (F == kSumWarp && warp == 11) {
+    // -------------------------------------------------------------- the sums of z
+    // follows the activation tiles of every round, adds up those of core rounds, and hands a
+    // task's sums to the epilogue with the issuers' accumulators (tfull)
+    int stage = 0, buf = 0;
+    uint32_t phase = 0, acc_phase = 0;
+    for (int i = t_lo; i < t_hi; ++i) {
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
+      const Task t = task_at(sched, i);
+      const DecPhase ph = phase_of(a, t.l, t.p);
+      int k0, k1;
+      krange(ph, t.tile, k0, k1);
+      float sz[2][BN / 16][4] = {};
+      bool ok = true;
+      for (int kb = k0; kb < k1; ++kb) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&fullB[stage], phase, abort_flag));
+        if (!ok) break;
+        if (t.p == 1) add_row_sums<BN>(smem_u32(sB + stage * kBTile), lane, sz);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[stage]);
+        if (++stage == S_) stage = 0, phase ^= 1;
+      }
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(&tempty[buf], acc_phase ^ 1, abort_flag));
+      if (!ok) {
+        if (lane == 0) {
+          if (!*abort_flag) note_timeout(a.status, 8, i, stage, static_cast<int>(phase));
+          *abort_flag = 1;
+        }
+        break;
+      }
+      if (t.p == 1 && (lane & 3) == 0) {
+        float* zs = zs_s + buf * BN + (lane >> 2);
+#pragma unroll
+        for (int m = 0; m < BN / 16; ++m) {
+          zs[16 * m] = sz[0][m][0] + sz[1][m][0];
+          zs[16 * m + 8] = sz[0][m][2] + sz[1][m][2];
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tfull[buf]);
+      if (++buf == 2) buf = 0, acc_phase ^= 1;
+    }
   } else if (warp >= 2 && warp <= 5) {
     // -------------------------------------------------------------- epilogue (warps 2-5)
     const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
@@ -787,7 +882,7 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
       }
       const float zb_i = z_i - 4.f * s_i;          // the decoded codes carry an offset of 4
       bool fail = false;
-      if (!kSums && t.p == 1) {
+      if (F == kSumEpilogue && t.p == 1) {
         // sum of z over this CTA's K range: first the ready flags of the slices it reads
         const bool has_k = k1 > k0;
         if (has_k && !(a.ext_in & 2)) {
@@ -876,6 +971,24 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
 #pragma unroll
       for (int c = 0; c < BN; c += kChunk) {
         float v[kChunk];
+        if constexpr (F == kSumWarp) {
+          // (this order keeps 40 registers fewer alive than the one below)
+          gather(static_cast<uint32_t>(c), v);
+          if (t.p == 1) {
+            const float4* zs = reinterpret_cast<const float4*>(zs_s + buf * BN + c);
+#pragma unroll
+            for (int q = 0; q < kChunk; q += 4) {
+              const float4 z = zs[q / 4];
+              v[q] = g_row * fmaf(s_i, v[q], zb_i * z.x);
+              v[q + 1] = g_row * fmaf(s_i, v[q + 1], zb_i * z.y);
+              v[q + 2] = g_row * fmaf(s_i, v[q + 2], zb_i * z.z);
+              v[q + 3] = g_row * fmaf(s_i, v[q + 3], zb_i * z.w);
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q) vals[c + q] = v[q];
+          continue;
+        }
         if (kSums && t.p == 1) {
           gather(static_cast<uint32_t>(Lo::kSumCol + c), v);
 #pragma unroll
@@ -1038,17 +1151,23 @@ DecWs dec_ws(int M, int n_in, int n_out) {
   return L;
 }
 
-template <int BN, bool kSums>
+template <int BN, SumForm F>
 cudaError_t prepare(int dev) {
   static std::mutex mu;
   static std::map<int, bool> done;
   std::lock_guard<std::mutex> g(mu);
   if (done[dev]) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(decode_layer_kernel<BN, kSums>,
+  const cudaError_t e = cudaFuncSetAttribute(decode_layer_kernel<BN, F>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             DecLayout<BN, kSums>::kBytes);
+                                             DecLayout<BN, F>::kBytes);
   if (e == cudaSuccess) done[dev] = true;
   return e;
+}
+
+// A launch's form of sum(z): `longer` as above.
+template <int BN>
+constexpr SumForm sum_form(bool longer) {
+  return BN == 64 ? kSumWarp : (longer ? kSumOnes : kSumEpilogue);
 }
 
 // Co-resident clusters of S CTAs of this kernel on the current device (0 if none).
@@ -1063,7 +1182,8 @@ int max_clusters(int dev, int S) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(S * 64));
   cfg.blockDim = dim3(DecCfg<BN>::kThreads);
-  cfg.dynamicSmemBytes = DecLayout<BN, true>::kBytes;   // both forms: one CTA per SM
+  constexpr SumForm kF = sum_form<BN>(true);      // either form: one CTA per SM
+  cfg.dynamicSmemBytes = DecLayout<BN, kF>::kBytes;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(S);
@@ -1072,7 +1192,7 @@ int max_clusters(int dev, int S) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, decode_layer_kernel<BN, true>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, decode_layer_kernel<BN, kF>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -1189,7 +1309,8 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
               int budget, cudaStream_t s) {
   int dev = 0;
   cudaGetDevice(&dev);
-  if (prepare<BN, true>(dev) != cudaSuccess || prepare<BN, false>(dev) != cudaSuccess)
+  constexpr SumForm kLong = sum_form<BN>(true), kShort = sum_form<BN>(false);
+  if (prepare<BN, kLong>(dev) != cudaSuccess || prepare<BN, kShort>(dev) != cudaSuccess)
     return FQ_ERR_CUDA;
   int total = 0;
   for (const Block& b : blocks) total += static_cast<int>(ceil_div(b.R, kBM));
@@ -1234,7 +1355,7 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(plan->ncl * plan->S));
   cfg.blockDim = dim3(DecCfg<BN>::kThreads);
-  cfg.dynamicSmemBytes = sums ? DecLayout<BN, true>::kBytes : DecLayout<BN, false>::kBytes;
+  cfg.dynamicSmemBytes = sums ? DecLayout<BN, kLong>::kBytes : DecLayout<BN, kShort>::kBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1245,7 +1366,8 @@ fq_status run(const DecMaps& maps, DecArgs& a, const std::vector<Block>& blocks,
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = plan->S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, sums ? decode_layer_kernel<BN, true> : decode_layer_kernel<BN, false>,
+  return cudaLaunchKernelEx(&cfg,
+                            sums ? decode_layer_kernel<BN, kLong> : decode_layer_kernel<BN, kShort>,
                             maps, a, plan->sched) == cudaSuccess
              ? FQ_OK
              : FQ_ERR_CUDA;
