@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
 // of a kernel that is bound by them), the next K slice in registers while the current one is
 // multiplied, two slices in shared memory (one barrier per slice).  Both operands are kept
 // k-major; a warp's 32 x 64 outputs read 4 + 8 distinct 16-byte groups per k, broadcast.
-// The two products of a 4096 x 4096 layer (318 GFLOP) take 5.6 ms (57 TFLOP/s), 12.8 with the small
-// tiles.
+// A 4096 x 4096 layer quantized round-to-nearest (318 GFLOP of products) takes 5.8 ms (55 TFLOP/s),
+// 12.9 with the small tiles.
 constexpr int kLBM = 128;
 constexpr int64_t kLargeMinBlocks = 16;
 
