@@ -136,8 +136,9 @@ size_t fq_workspace_bytes(int M, int d_in, int n_in, int n_out, int d_out, int m
  *   y        device, M x d_out output (bf16 or fp32 by mode)
  *   ws       device workspace of at least fq_workspace_bytes(M, d_in, n_in, n_out, d_out,
  *            mode) bytes, 256-byte aligned, ZERO-FILLED BEFORE ITS FIRST USE.  Its first 64 KiB
- *            are a header at fixed offsets (status word, a call generation counter and
- *            ready flags per slice of a 128-row output tile) that every completed call leaves
+ *            are a header at fixed offsets (status word, a call generation counter, the
+ *            counters of tiles split over K and ready flags per slice of a 128-row output
+ *            tile) that every completed call leaves
  *            ready for the next, so a workspace can be reused across calls and layer shapes
  *            without being cleared again; zero it again after a call reported
  *            FQ_ERR_TIMEOUT.  Its first 4

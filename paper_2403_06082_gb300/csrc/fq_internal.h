@@ -21,15 +21,18 @@ inline int64_t round_up(int64_t a, int64_t b) { return ceil_div(a, b) * b; }
 // can serve layers of different shapes): [0] device status word, [4] generation counter,
 // [8] end-of-call ticket, [12] the activation-rounding maximum, [16..31] the first timeout's
 // role, task, stage and detail words (cleared by each call), [32] the activation-rounding step,
-// [kWsFlags] ready flags, kWsSlices per row tile of up to kWsMaxTiles
-// row tiles per phase.  A zero-filled header is a valid initial state and every completed call
-// leaves it valid for the next one.
+// [kWsCnt] the split-K counters of kWsCntSlots tiles (zero between calls), [kWsFlags] ready flags,
+// kWsSlices per row tile of up to kWsMaxTiles row tiles per phase.  A zero-filled header is a valid
+// initial state and every completed call leaves it valid for the next one; nothing past it is
+// assumed to hold anything when a call starts.
 constexpr size_t kWsHeader = 64 * 1024;
 constexpr size_t kWsGen = 4;
 constexpr size_t kWsDone = 8;
 constexpr size_t kWsAmax = 12;    // activation rounding: max |z| of the call (float bits)
 constexpr size_t kWsDelta = 32;   // activation rounding: the call's step Delta (float)
+constexpr size_t kWsCnt = 64;
 constexpr size_t kWsFlags = 1024;
+constexpr int kWsCntSlots = static_cast<int>((kWsFlags - kWsCnt) / 4);
 constexpr int kWsSlices = 8;
 constexpr int kWsMaxTiles = 640;
 static_assert(kWsFlags + 3 * kWsMaxTiles * kWsSlices * 4 <= kWsHeader, "flags fit the header");

@@ -61,10 +61,9 @@ struct PhaseArgs {
   // On CTA pairs:
   int KS, kbs, units;        // K splits per tile, K blocks per split, tiles * KS work units
   float* part;               // KS > 1: fp32 partial tiles [tile][split][BN][128]
-  int64_t part_floats;       // what `part` and `cnt` hold (host)
-  int cnt_slots;
+  int64_t part_floats;       // what `part` holds (host)
   uint32_t* cnt;             // KS > 1: arrivals per tile, 16 bits for each CTA's half (the last
-                             // resets them to 0)
+                             // resets them to 0), kWsCntSlots of them in the workspace header
   const uint32_t* words;     // core: packed codes
   __nv_bfloat16* out;        // [M][R]
   float* zsum_part;          // analysis writes [RT][M] sums of z; the core reads them
@@ -1374,7 +1373,7 @@ int plan_pairs(PhaseArgs& a, int pairs) {
     const int bn = 128 << w, tt = static_cast<int>(ceil_div(a.M, bn)), tiles = a.RT * tt;
     for (int ks = 1; ks <= std::min(kMaxSplits, a.KB / kMinSplitBlocks) || ks == 1; ++ks) {
       const int kbs = static_cast<int>(ceil_div(a.KB, ks));
-      if (ks > 1 && (ceil_div(a.KB, kbs) != ks || tiles * ks > pairs || tiles > a.cnt_slots ||
+      if (ks > 1 && (ceil_div(a.KB, kbs) != ks || tiles * ks > pairs || tiles > kWsCntSlots ||
                      static_cast<int64_t>(a.RT1) * tt * ks * bn * kBM > a.part_floats))
         continue;
       const int64_t cost = ceil_div(static_cast<int64_t>(tiles) * ks, pairs) * kbs * kRoundCycles[w] +
@@ -1394,9 +1393,8 @@ int plan_pairs(PhaseArgs& a, int pairs) {
 }
 
 struct WsLayout {
-  size_t z, u, zsum, cnt, part, z32, total;
-  int64_t part_floats;       // sizes of part and cnt
-  int cnt_slots;
+  size_t z, u, zsum, part, z32, total;
+  int64_t part_floats;       // size of part
 };
 
 // Partial tiles for split K, sized for any device with at most kMaxSplitSms SMs: a phase with
@@ -1413,20 +1411,15 @@ WsLayout ws_layout(int M, int d_in, int n_in, int n_out, int d_out, int act_bits
   const int BN = pick_bn(M);
   const int64_t TT = ceil_div(M, BN);
   const int64_t rows[3] = {n_in, n_out, d_out};
-  int64_t slots = 0, max_tiles = 0;
+  int64_t slots = 0;
   for (int64_t r : rows) {
     const int64_t tiles = ceil_div(r, kBM) * TT;
-    if (tiles < kMaxSplitSms) {
+    if (tiles < kMaxSplitSms)
       slots = std::max(slots, std::min<int64_t>(kMaxSplitSms, tiles * kMaxSplits));
-      max_tiles = std::max(max_tiles, tiles);
-    }
   }
   (void)d_in;
-  L.cnt = off;
-  off += round_up(max_tiles * 4, 256);
   L.part = off;
   L.part_floats = slots * BN * kBM;
-  L.cnt_slots = static_cast<int>(round_up(max_tiles * 4, 256) / 4);
   off += static_cast<size_t>(slots) * BN * kBM * 4;
   L.z32 = off;
   if (act_bits > 0) off += round_up(static_cast<int64_t>(M) * n_in * 4, 256);
@@ -1554,16 +1547,10 @@ WsLayout dense_ws_layout(int M, int d_out) {
   off += round_up(ceil_div(d_out, kBM) * M * 4, 256);
   const int BN = pick_bn(M);
   const int64_t tiles = ceil_div(d_out, kBM) * ceil_div(M, BN);
-  int64_t slots = 0, max_tiles = 0;
-  if (tiles < kMaxSplitSms) {
-    slots = std::min<int64_t>(kMaxSplitSms, tiles * kMaxSplits);
-    max_tiles = tiles;
-  }
-  L.cnt = off;
-  off += round_up(max_tiles * 4, 256);
+  int64_t slots = 0;
+  if (tiles < kMaxSplitSms) slots = std::min<int64_t>(kMaxSplitSms, tiles * kMaxSplits);
   L.part = off;
   L.part_floats = slots * BN * kBM;
-  L.cnt_slots = static_cast<int>(round_up(max_tiles * 4, 256) / 4);
   off += static_cast<size_t>(slots) * BN * kBM * 4;
   L.total = off;
   return L;
@@ -1580,10 +1567,9 @@ fq_status launch_tc_dense(const void* x, int M, int d_in, const void* W, int d_o
   a.out = reinterpret_cast<__nv_bfloat16*>(y);
   a.clear_status = 1;
   a.status = reinterpret_cast<int32_t*>(ws);
-  a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
+  a.cnt = reinterpret_cast<uint32_t*>(ws + kWsCnt);
   a.part = reinterpret_cast<float*>(ws + L.part);
   a.part_floats = L.part_floats;
-  a.cnt_slots = L.cnt_slots;
   PhasePlan pl;
   if (!plan_call_phase<kSynthesis>(pl, a, W, x, device_info())) return FQ_ERR_CUDA;
   return launch_phase<kSynthesis>(pl, a, s) == cudaSuccess ? FQ_OK : FQ_ERR_CUDA;
@@ -1621,10 +1607,9 @@ fq_status launch_tc_forward(const void* x, int M, int d_in, const void* T_in,
     a[ph].out = outs[ph];
     a[ph].zsum_part = zsum;
     a[ph].status = status;
-    a[ph].cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
+    a[ph].cnt = reinterpret_cast<uint32_t*>(ws + kWsCnt);
     a[ph].part = reinterpret_cast<float*>(ws + L.part);
     a[ph].part_floats = L.part_floats;
-    a[ph].cnt_slots = L.cnt_slots;
   }
   a[0].clear_status = 1;
   a[1].words = Cq.words;
@@ -1683,10 +1668,9 @@ fq_status launch_tc_unit_forward(const void* T_in, int d_in, const fq_packed& Cq
     a[ph].out = outs[ph];
     a[ph].zsum_part = zsum;
     a[ph].status = status;
-    a[ph].cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
+    a[ph].cnt = reinterpret_cast<uint32_t*>(ws + kWsCnt);
     a[ph].part = reinterpret_cast<float*>(ws + L.part);
     a[ph].part_floats = L.part_floats;
-    a[ph].cnt_slots = L.cnt_slots;
   }
   a[1].words = Cq.words;
   a[1].scale = reinterpret_cast<const __half*>(Cq.scale_f16);
