@@ -11,7 +11,8 @@
 //   synthesis  A = T_out^T (d_out x n_out), B = u, out = y (bf16)
 //
 // tc_pair_kernel runs them on CTA pairs, with tiles of 256 rows x 128 or 256 tokens.  A call with a
-// budget of one SM, which has no pair, takes tc_phase_kernel: tiles of 128 x 128 on one SM.
+// budget of one SM, which has no pair, takes tc_phase_kernel: tiles of 128 rows x 128 or 256 tokens
+// on one SM.  So does an odd budget where that is estimated to be faster (three SMs, mostly).
 //
 // Operand tiles are 64 bf16 wide in K (one 128-byte swizzle atom) and staged through a ring
 // of shared-memory stages guarded by mbarriers; accumulators are double-buffered in TMEM so
@@ -35,6 +36,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <utility>
 
 #include "fq_device.cuh"
@@ -104,7 +106,7 @@ struct Layout {
   static constexpr int oRedSmall = oMisc + 16;                      // [4][kChunk] floats
   static constexpr int oZsum = oRedSmall + 4 * kChunk * 4;          // [2][BN] floats
   static constexpr int kBytes = oZsum + 2 * BN * 4 + 1024;          // + alignment slack
-  static_assert(BN == 128, "tile width of the one-SM kernel");
+  static_assert(BN == 128 || BN == 256, "tile widths of the one-SM kernel");
   static_assert(kBTileBytes % 1024 == 0, "B tiles must keep 1024-byte alignment");
   static_assert(kBytes <= 227 * 1024, "shared memory");
   static_assert(kStages >= 2 && (!kCodes || kStages % 4 == 0), "ring depth");
@@ -154,8 +156,10 @@ __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t n, bool v) {
   return out != 0;
 }
 
-// One SM (a call whose budget is one SM; the pairs need two): tiles of 128 rows x BN tokens, one
-// warp of TMA copies, one issuing MMAs, four of epilogue and, in the core, four decoders.
+// Without pairs (a call whose budget is one SM, or an odd number of them that pairs use badly): tiles
+// of 128 rows x BN tokens, one CTA each, with one warp of TMA copies, one issuing MMAs, four of
+// epilogue and, in the core, four decoders.  BN is 256 above 128 tokens: the operands of a K block
+// then take 740 cycles for twice the tokens of 128 (600), see plan_one_sm.
 template <int PHASE, int BN>
 __global__ void __launch_bounds__(threads_for<PHASE>(), 1)
     tc_phase_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -1343,12 +1347,21 @@ constexpr int kMaxSplits = 4;
 constexpr int kMinSplitBlocks = 4;
 constexpr int kMaxSplitSms = 256;      // bound on the SM count used for split-K planning
 
-// One SM: whole tiles, all on one CTA.
-void plan_one_sm(PhaseArgs& a, int BN) {
+// Without pairs: whole tiles, a CTA per SM.  Returns the estimated time in cycles, waves of tiles a K
+// block at a time.  On one SM, 128 and 256 tokens per tile (us per call): 4096 x 4096 at 200 tokens
+// 4545, 2752, at 512 tokens 8932, 5335; 768 to 3072 at 200 tokens 1147, 772.
+constexpr int kOneSmRoundCycles[2] = {600, 740};   // per K block, BN = 128, 256
+constexpr int kOneSmEpilogueCycles[2] = {6000, 11000};
+
+int one_sm_bn(int M) { return M <= 128 ? 128 : 256; }
+
+int64_t plan_one_sm(PhaseArgs& a, int sms) {
+  const int bn = one_sm_bn(a.M), w = bn / 256;
   a.RT1 = a.RT = static_cast<int>(ceil_div(a.R, kBM));
-  a.TT = static_cast<int>(ceil_div(a.M, BN));
+  a.TT = static_cast<int>(ceil_div(a.M, bn));
   a.KB = static_cast<int>(ceil_div(a.K, kBK));
   a.tiles = a.RT * a.TT;
+  return ceil_div(a.tiles, sms) * a.KB * kOneSmRoundCycles[w] + kOneSmEpilogueCycles[w];
 }
 
 // CTA pairs: units of 256 x BN tiles (or K splits of them), one pair per unit and
@@ -1363,7 +1376,8 @@ constexpr int kEpilogueCycles[2] = {6000, 11000};
 constexpr int kSplitFixed[2] = {5000, 10000};     // a split tile, and each of its splits
 constexpr int kSplitEach[2] = {1500, 3000};
 
-int plan_pairs(PhaseArgs& a, int pairs) {
+// Returns the tokens per tile and the estimate.
+std::pair<int, int64_t> plan_pairs(PhaseArgs& a, int pairs) {
   a.RT1 = static_cast<int>(ceil_div(a.R, kBM));
   a.RT = static_cast<int>(ceil_div(a.R, 2 * kBM));
   a.KB = static_cast<int>(ceil_div(a.K, kBK));
@@ -1389,7 +1403,7 @@ int plan_pairs(PhaseArgs& a, int pairs) {
     }
   }
   a.units = a.tiles * a.KS;
-  return best_bn;
+  return {best_bn, best};
 }
 
 struct WsLayout {
@@ -1480,29 +1494,46 @@ struct ChainedLaunch {
 // One phase of a call, planned with its tensor maps before anything is launched.
 struct PhasePlan {
   CUtensorMap A, B;
-  int bn;                    // tokens per tile on CTA pairs; 0: the one-SM kernel
+  bool pairs;                // on CTA pairs, else the one-SM kernel
+  int bn;                    // tokens per tile
   int grid;
 };
 
 // A: the weight operand (R x K; not used by the code product), B: the tokens (M x K).  CTA pairs for
-// budgets of two SMs and more.
+// budgets of two SMs and more; an odd budget leaves an SM without a partner, so there the one-SM
+// kernel on all of them is taken where its estimate is lower.  At three SMs (us per call, one pair and
+// three CTAs): 4096 x 4096 at 129 tokens 1013, 949, at 512 tokens 2015, 1834; 768 to 3072 at 128
+// tokens 232, 207, at 512 tokens 595, 546.  At five, two pairs beat five CTAs: 4096 x 4096 at 512
+// tokens 1018, 1147.
 template <int PHASE>
 bool plan_call_phase(PhasePlan& pl, PhaseArgs& a, const void* A, const void* B,
                      const DeviceInfo& d) {
-  if (d.sms >= 2) {
+  int64_t cost = INT64_MAX;
+  pl.pairs = d.sms >= 2;
+  if (pl.pairs) {
     const int pairs = std::min({resident_pairs<PHASE, 128>(d.dev), resident_pairs<PHASE, 256>(d.dev),
                                 d.sms / 2});
     if (pairs < 1) return false;
-    pl.bn = plan_pairs(a, pairs);
+    std::tie(pl.bn, cost) = plan_pairs(a, pairs);
     pl.grid = 2 * std::min(a.units, pairs);
-  } else {
-    if (prepare_kernel<PHASE, 128>(d.dev) != cudaSuccess) return false;
-    pl.bn = 0;
-    plan_one_sm(a, 128);
-    pl.grid = 1;
   }
+  if (d.sms % 2 && !a.transposed) {            // (the one-SM kernel has no transposed store)
+    PhaseArgs one = a;
+    const int64_t one_cost = plan_one_sm(one, d.sms);
+    if (one_cost < cost) {
+      cost = one_cost;
+      a = one;
+      pl.pairs = false;
+      pl.bn = one_sm_bn(a.M);
+      pl.grid = std::min(a.tiles, d.sms);
+      if ((pl.bn == 128 ? prepare_kernel<PHASE, 128>(d.dev) : prepare_kernel<PHASE, 256>(d.dev)) !=
+          cudaSuccess)
+        return false;
+    }
+  }
+  if (cost == INT64_MAX) return false;
   // a pair's CTAs load half of a tile's tokens each
-  if (!make_tmap(&pl.B, B, a.M, a.K, pl.bn ? pl.bn / 2 : 128)) return false;
+  if (!make_tmap(&pl.B, B, a.M, a.K, pl.pairs ? pl.bn / 2 : pl.bn)) return false;
   if (PHASE == kCore) {
     pl.A = pl.B;
     return true;
@@ -1517,12 +1548,17 @@ cudaError_t launch_pairs(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s
   return cudaLaunchKernelEx(&l.cfg, tc_pair_kernel<PHASE, BN>, pl.A, pl.B, a);
 }
 
+template <int PHASE, int BN>
+cudaError_t launch_one_sm(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s) {
+  const ChainedLaunch l(pl.grid, threads_for<PHASE>(), Layout<PHASE, BN>::kBytes, s);
+  return cudaLaunchKernelEx(&l.cfg, tc_phase_kernel<PHASE, BN>, pl.A, pl.B, a);
+}
+
 template <int PHASE>
 cudaError_t launch_phase(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s) {
-  if (pl.bn == 128) return launch_pairs<PHASE, 128>(pl, a, s);
-  if (pl.bn == 256) return launch_pairs<PHASE, 256>(pl, a, s);
-  const ChainedLaunch l(pl.grid, threads_for<PHASE>(), Layout<PHASE, 128>::kBytes, s);
-  return cudaLaunchKernelEx(&l.cfg, tc_phase_kernel<PHASE, 128>, pl.A, pl.B, a);
+  if (pl.pairs)
+    return pl.bn == 128 ? launch_pairs<PHASE, 128>(pl, a, s) : launch_pairs<PHASE, 256>(pl, a, s);
+  return pl.bn == 128 ? launch_one_sm<PHASE, 128>(pl, a, s) : launch_one_sm<PHASE, 256>(pl, a, s);
 }
 
 cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
