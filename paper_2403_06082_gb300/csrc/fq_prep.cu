@@ -150,7 +150,9 @@ __global__ void eye_kernel(float* __restrict__ T, int d) {
 // C[i][j] = sum_k A[i][k] * B[j][k], fp32, both operands K-contiguous.  Every element is one
 // chain of fused multiply-adds in ascending k (K padded with zeros to a multiple of kGK), whichever
 // kernel computes it, so the coefficients and the codes rounded from them do not depend on the
-// choice.  Small products: 64 x 64 tiles, 4 x 4 outputs per thread.
+// choice.  Small products: 64 x 64 tiles, 4 x 4 outputs per thread, the next K slice in registers
+// while the current one is multiplied (without that a slice waits for its loads: a 256 x 256 layer
+// quantized round-to-nearest 55 us, with it 26).
 constexpr int kGT = 64, kGK = 16;
 __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
                                                    const float* __restrict__ B,
@@ -161,16 +163,26 @@ __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kGT;
   const int j0 = blockIdx.y * kGT;
-  float acc[4][4] = {};
+  float acc[4][4] = {}, ra[4], rb[4];
+  // the next K slice's elements, four of each operand per thread
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int t = threadIdx.x + 256 * l, r = t / kGK, gk = k0 + t % kGK;
+      ra[l] = (i0 + r < M && gk < K) ? A[(i0 + r) * K + gk] : 0.f;
+      rb[l] = (j0 + r < N && gk < K) ? B[static_cast<int64_t>(j0 + r) * K + gk] : 0.f;
+    }
+  };
+  fetch(0);
   for (int k0 = 0; k0 < K; k0 += kGK) {
-    for (int t = threadIdx.x; t < kGT * kGK; t += 256) {
-      const int r = t / kGK, kk = t % kGK;
-      const int64_t gi = i0 + r;
-      const int gj = j0 + r, gk = k0 + kk;
-      As[kk][r] = (gi < M && gk < K) ? A[static_cast<int64_t>(gi) * K + gk] : 0.f;
-      Bs[kk][r] = (gj < N && gk < K) ? B[static_cast<int64_t>(gj) * K + gk] : 0.f;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int t = threadIdx.x + 256 * l;
+      As[t % kGK][t / kGK] = ra[l];
+      Bs[t % kGK][t / kGK] = rb[l];
     }
     __syncthreads();
+    if (k0 + kGK < K) fetch(k0 + kGK);
 #pragma unroll
     for (int kk = 0; kk < kGK; ++kk) {
       float a[4], b[4];
@@ -198,10 +210,10 @@ __global__ void __launch_bounds__(256) gemm_nt_f32(const float* __restrict__ A,
 // of a kernel that is bound by them), the next K slice in registers while the current one is
 // multiplied, two slices in shared memory (one barrier per slice).  Both operands are kept
 // k-major; a warp's 32 x 64 outputs read 4 + 8 distinct 16-byte groups per k, broadcast.
-// A 4096 x 4096 layer quantized round-to-nearest (318 GFLOP of products) takes 5.8 ms (55 TFLOP/s),
-// 12.9 with the small tiles.
+// A 4096 x 4096 layer quantized round-to-nearest (318 GFLOP of products) takes 5.7 ms (56 TFLOP/s),
+// 8.6 with the small tiles.
 constexpr int kLBM = 128;
-constexpr int64_t kLargeMinBlocks = 16;
+constexpr int64_t kLargeMinTiles = 165;
 
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   uint64_t r;
@@ -327,12 +339,15 @@ __global__ void __launch_bounds__(2 * kBN, 256 / kBN) gemm_nt_f32_large(const fl
 
 cudaError_t gemm_nt(const float* A, const float* B, float* C, int64_t M, int N, int K,
                     cudaStream_t s) {
-  // The large tiles are ahead from about 20 blocks on, far below a wave (a layer quantized
-  // round-to-nearest, us, small and large tiles: 512 x 512 115, 114; 768 x 768 216, 163; 1152 x 1152
-  // 411, 247; 4096 x 4096 13023, 5801); N <= 64 (a rotation factor) takes 64 columns so that no
-  // half of a tile is idle.
+  // The large tiles are ahead once they occupy more than half of the SMs, from about 165 tiles of
+  // 128 x 64 (83 blocks) on; fewer leave the GPU emptier than the small ones do.  The two products of a
+  // layer quantized round-to-nearest, their tiles, us with small and with large tiles: 512 x 512, 40
+  // and 45, 48, 103; 768 x 768, 84 and 98, 111, 149; 1024 x 1024, 144 and 162, 179, 199; 768 to 1536,
+  // 168 and 196, 237, 220 (the first small, the second large: 226); 1088 x 1088, 170 and 190, 224, 208
+  // (217); 1280 x 1280, 220 and 242, 312, 243; 2048 x 2048, 1163, 873.  N <= 64 (a rotation factor)
+  // takes 64 columns so that no half of a tile is idle.
   const int bn = N <= 64 ? 64 : 128;
-  if (ceil_div(M, kLBM) * ceil_div(N, bn) >= kLargeMinBlocks) {
+  if (ceil_div(M, kLBM) * ceil_div(N, 64) >= kLargeMinTiles) {
     const int vec = K % 4 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
     const dim3 grid(static_cast<unsigned>(ceil_div(M, kLBM)), static_cast<unsigned>(ceil_div(N, bn)));
     if (bn == 64)
