@@ -36,12 +36,19 @@
 //                 tokens a round is bound by its MMAs, which the ones would double, and without the
 //                 ones' tile and columns there is room for a sixth stage and a second issuer.
 // They are separate kernels: a small launch is bound by latency, and carrying another's code cost
-// it 2-8%.  Measured, us per call: (kSumEpilogue, kSumOnes) 4096 x 4096 at 24 tokens 30.4, 28.4;
-// q|k|v at 16 tokens 51.1, 48.2; with 8 K blocks per CTA at 34 tokens 35.1, 37.0; (the faster of
-// those with one issuer, kSumWarp) 4096 x 4096 at 48 tokens 35.4, 33.4; 11008 x 4096 at 64 tokens
-// 85.2, 81.8; 4096 x 11008 at 40 tokens 80.1, 75.7; 768 to 3072 at 34 tokens 24.1, 23.2; (the faster,
-// kSumWarp at up to 32 tokens) 256 x 256 at 8 tokens 12.0, 12.3; 4096 x 4096 at 24 tokens 28.0, 28.3;
-// q|k|v at 16 tokens 48.1, 48.4; gate|up at 16 tokens 112.8, 111.6, at 32 tokens 116.5, 116.6.
+// it 2-8%.  Measured, us per call: (kSumEpilogue, kSumOnes) see kSumMmaBlocks; q|k|v at 16 tokens
+// 51.1, 48.2; (kSumEpilogue, kSumWarp) 4096 x 4096 at 48 tokens 36.6, 34.1; 2048 x 2048 at 64 tokens
+// 26.2, 24.5; 768 to 3072 at 48 tokens 23.0, 22.7; 256 x 256 at 33 to 64 tokens the same;
+// (the faster of the others, kSumWarp at up to 32 tokens) 256 x 256 at 8 tokens 12.0, 12.3;
+// 4096 x 4096 at 24 tokens 28.0, 28.3; q|k|v at 16 tokens 48.1, 48.4; gate|up at 16 tokens 112.8,
+// 111.6, at 32 tokens 116.5, 116.6.
+// All three add in fp32, kSumEpilogue with rounded additions, the others in the tensor cores'
+// accumulators.  The share of results u of a layer of Gaussian coefficients, z exact, that are not
+// the rounding to bf16 of the 64-bit value (kSumEpilogue in all launches, with one issuer at 64
+// tokens; then this rule): n_in = 4512 at 16 tokens
+// 0.070%, 0.068%, at 64 tokens 0.126%, 0.080%; n_in = 12128 at 16 tokens 0.134%, 0.105%, at 64
+// tokens 0.303%, 0.137%; no larger at any of 288 to 12128 and 1 to 64 but one (9024, 16 tokens: 0.105%,
+// 0.109%).
 //
 // The workspace header holds the generation counter and the tiles' ready flags; a zero-filled
 // header is a valid start and every call leaves it valid for the next (flags keep
@@ -216,7 +223,16 @@ __device__ __forceinline__ uint4 ldcg_u4(const __nv_bfloat16* p) {
 }
 
 // Launches of 16 or 32 tokens whose core tasks have more than this many K blocks per CTA take sum(z)
-// from the MMAs (kSumOnes).
+// from the MMAs (kSumOnes).  Us per call with kSumEpilogue and with kSumOnes, by K blocks per CTA:
+//    4 (768 to 3072)   16 tokens 16.3, 16.4   17 tokens 18.4, 19.0   32 tokens 18.7, 19.0
+//    9 (2048 x 2048)             16.3, 16.5             19.5, 20.0             19.7, 19.7
+//   11 (2560 x 2560)             18.1, 18.2             20.4, 21.2             21.3, 21.2
+//   11 (5120 x 5120)             45.0, 42.2             51.3, 49.2             53.5, 49.1
+//   14 (3072 x 3072)             19.7, 19.8             22.6, 23.0             24.0, 23.0
+//   18 (4096 x 4096)             25.5, 25.2             28.2, 27.3             29.7, 27.9
+//   20 (4608 x 4608)             29.7, 29.1             34.3, 30.9             38.9, 31.4
+// From 9 on the sums cost little where a CTA has one core task and gain where it has several (5120:
+// three), so the line lies below.
 constexpr int kSumMmaBlocks = 8;
 
 // Adds to s[m][0] and s[m][2] the sums over K of rows 16 m + lane / 4 and + 8 of a B tile (BN rows of
@@ -351,7 +367,11 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
   float* zs_s = reinterpret_cast<float*>(smem + Lo::oZs);
   float* zs_part = reinterpret_cast<float*>(smem + Lo::oZsPart);
 
-  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);   // uniform
+  // The warp's index, made uniform where that pays (us per call without and with it): 4096 to 11008 at
+  // 16 tokens 66.2, 65.2; 256 x 256 at 64 tokens 17.2, 17.7, 2048 x 2048 23.7, 24.4, 4096 to 11008
+  // 81.0, 80.2.
+  int warp = static_cast<int>(threadIdx.x >> 5);
+  if (BN < 64) warp = __shfl_sync(0xffffffffu, warp, 0);
   const int lane = threadIdx.x & 31;
   const int S = a.S;
   const bool clustered = S > 1;
@@ -989,18 +1009,27 @@ __global__ void __launch_bounds__(DecCfg<BN>::kThreads, 1)
           for (int q = 0; q < kChunk; ++q) vals[c + q] = v[q];
           continue;
         }
-        if (kSums && t.p == 1) {
-          gather(static_cast<uint32_t>(Lo::kSumCol + c), v);
+        if constexpr (kSums || BN == 16) {
+          if (kSums && t.p == 1) {
+            gather(static_cast<uint32_t>(Lo::kSumCol + c), v);
 #pragma unroll
-          for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * v[q];
-        } else if (t.p == 1) {
+            for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * v[q];
+          } else if (t.p == 1) {
 #pragma unroll
-          for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * zs_s[c + q];
+            for (int q = 0; q < kChunk; ++q) vals[c + q] = zb_i * zs_s[c + q];
+          }
+          gather(static_cast<uint32_t>(c), v);
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q)
+            vals[c + q] = t.p == 1 ? g_row * fmaf(s_i, v[q], vals[c + q]) : v[q];
+        } else {
+          // (the sums read last: read before the accumulators they cost 32 tokens of a 256 x 256
+          // layer 14.7 us instead of 13.7)
+          gather(static_cast<uint32_t>(c), v);
+#pragma unroll
+          for (int q = 0; q < kChunk; ++q)
+            vals[c + q] = t.p == 1 ? g_row * fmaf(s_i, v[q], zb_i * zs_s[c + q]) : v[q];
         }
-        gather(static_cast<uint32_t>(c), v);
-#pragma unroll
-        for (int q = 0; q < kChunk; ++q)
-          vals[c + q] = t.p == 1 ? g_row * fmaf(s_i, v[q], vals[c + q]) : v[q];
       }
       tc_fence_before_sync();
       mbar_arrive(&tempty[buf]);
