@@ -35,21 +35,21 @@ namespace {
 
 
 // ------------------------------------------------------------------------------ rotations
-// A cluster of C CTAs takes one token's a x b block; bf16 in and out, fp32 between.
-//   analysis:  V = Pi^T x (V_e = x[iperm[e]]), Y = Q_a^T V Q_b, out = D vec(Y)   A = Q_a^T, B = Q_b
+// C CTAs take one token's a x b block, each a range of the rows of Y; bf16 in and out, fp32 between.
+//   analysis:  V = Pi^T x (V[perm[i]] = x_i), Y = Q_a^T V Q_b, out = D vec(Y)    A = Q_a^T, B = Q_b
 //   synthesis: V = D s, Y = Q_a V Q_b^T, out = Pi vec(Y) (out[iperm[e]] = vec(Y)_e) A = Q_a, B = Q_b^T
-// CTA r computes columns [r bc, (r + 1) bc) of T1 = A V, which needs only those columns of V, and
-// stores each row of them into the shared memory of the CTA that owns the row; after one cluster
-// barrier it computes its rows [r rc, (r + 1) rc) of Y = T1 B.  So a token's gather, products and
-// scatter are each split C ways and nothing is computed or gathered twice.  Both products take
-// 4 rows x 2 columns per thread, the row values of a reduction index as one 16-byte read (the
-// factors are read in the orientation that has them consecutive).
-// What bounds it is latency: a token is two products of a few million multiply-adds.  The
-// factors, the permutation and the signs do not depend on the previous kernel and are staged in
-// shared memory before the wait for the input; a factor that does not fit is read from L2.
-// Measured against a CTA per eight rows that gathered its whole token: three 11008 x 4096 layers at
-// 64 tokens 265 -> 164 us (the rotations and the fused kernel), 4096 to 11008 at 64 tokens 212 ->
-// 159, 2048 x 2048 at 16 tokens 34.0 -> 30.2.
+// A CTA reads the whole token, in order, and permutes it on its way into shared memory: a gather of
+// 2-byte entries from global memory costs a sector each, ten times the conflicts of the scatter into
+// shared memory.  T1 = A V for its rows and Y = T1 B follow without the other CTAs, 4 rows x 2 columns
+// per thread, the row values of a reduction index as one 16-byte read (A is read transposed).
+// What bounds it is latency: a token is two products of a few million multiply-adds, and code that
+// runs once per launch waits for its instructions, so the loops are unrolled little.  The CTA's rows of
+// A and all of B do not depend on the previous kernel and are staged in shared memory before the
+// wait for the input; a factor that does not fit is read from L2.
+// Measured, us per call (a CTA per eight rows that staged B in chunks; a cluster per token that split
+// the gather and exchanged T1; this form): 2048 x 2048 at 4 tokens 23.1, 27.3, 22.9, at 32 tokens
+// 31.1, 32.7, 27.6; two 4096 to 11008 layers at 16 tokens 88, 82, 70; three 11008 to 4096 layers at 64
+// tokens 266, 158, 140; 28672 to 4096 at one token (B, 200 KB, read from L2) 99, 167, 103.
 constexpr int kRotThreads = 256;
 constexpr size_t kMaxSmem = 227 * 1024;
 
@@ -58,12 +58,12 @@ struct RotLayer {
   const __nv_bfloat16* in;
   __nv_bfloat16* out;
   int a, b;
-  int ap, bp;             // row strides of the staged factors: a rounded up to 4, b to 2
-  int bc, vs;             // columns of V per CTA, and their stride (rounded up to 2)
-  int rc, rs;             // rows of Y per CTA, and their stride in T1t (rounded up to 4)
-  int stage_a, stage_b;   // the factor is staged in shared memory
+  int bp;                 // row stride of V and of the staged B: b rounded up to 2
+  int rc;                 // rows of Y per CTA, a multiple of 4, and T1t's row stride
+  int stage_a, stage_b;   // (where not both factors of every layer are staged whole)
   const float* At;        // A^T, a x a row-major: At[i][r] = A[r][i]
   const float* B;         // b x b row-major
+  const int32_t* perm;
   const int32_t* iperm;
   const float* signs;
 };
@@ -83,16 +83,14 @@ __device__ __forceinline__ void cp_async_commit() {
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
-}
 
-// An n x n factor (row-major) into shared memory with row stride np, asynchronously, a warp per row
-// in the widest pieces that the rows' alignment allows; past the n-th column nothing is written
-// (such entries only reach results that are dropped).
+// `cols` columns of an n x n factor (row-major) into shared memory with row stride np, asynchronously:
+// one copy when they are whole rows without padding, else a warp per row, in the widest pieces that
+// the alignment allows (n, cols and the first column are multiples of them).  Nothing is written past
+// the last column (such entries only reach results that are dropped).
 __device__ __forceinline__ void stage_factor(float* dst, const float* __restrict__ src, int n,
-                                             int np, int tid) {
-  if (n % 4 == 0) {       // np == n: one contiguous copy
+                                             int cols, int np, int tid) {
+  if (n % 4 == 0 && cols == n) {       // np == n
     for (int i = tid; i < n * n / 4; i += kRotThreads) cp_async<16>(dst + 4 * i, src + 4 * i);
     return;
   }
@@ -101,9 +99,9 @@ __device__ __forceinline__ void stage_factor(float* dst, const float* __restrict
     const float* from = src + static_cast<int64_t>(r) * n;
     float* to = dst + r * np;
     if (n % 2 == 0)
-      for (int i = 2 * lane; i < n; i += 64) cp_async<8>(to + i, from + i);
+      for (int i = 2 * lane; i < cols; i += 64) cp_async<8>(to + i, from + i);
     else
-      for (int i = lane; i < n; i += 32) cp_async<4>(to + i, from + i);
+      for (int i = lane; i < cols; i += 32) cp_async<4>(to + i, from + i);
   }
 }
 
@@ -125,94 +123,75 @@ __device__ __forceinline__ void rot_product(float (&acc)[4][2], int n, Rows rows
   }
 }
 
-template <bool kSynth, bool kCluster>
+// kStaged: both factors of every layer of the launch are in shared memory, all of A.  Otherwise each
+// may or may not be, and of A only the CTA's columns of A^T.
+template <bool kSynth, bool kStaged>
 __global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_constant__ RotBatch rb) {
   const RotLayer& ly = rb.L[blockIdx.z];
-  const int a = ly.a, b = ly.b, ap = ly.ap, bp = ly.bp, vs = ly.vs, rs = ly.rs, rc = ly.rc;
+  const int a = ly.a, b = ly.b, bp = ly.bp, rc = ly.rc;
   const int tid = threadIdx.x;
-  const int rank = kCluster ? static_cast<int>(blockIdx.x) : 0;       // the cluster spans x
-  const int c0 = min(b, rank * ly.bc), nc = min(ly.bc, b - c0);       // this CTA's columns of V
-  const int r0 = min(a, rank * rc), nr = min(rc, a - r0);             // and its rows of Y
+  const int r0 = min(a, static_cast<int>(blockIdx.x) * rc), nr = min(rc, a - r0);   // its rows
+  const int al = kStaged ? (a + 3) & ~3 : rc, a0 = kStaged ? r0 : 0;   // As's row stride, and r0 in it
   extern __shared__ float4 rot_smem4[];
-  float* T1t = reinterpret_cast<float*>(rot_smem4);   // [b][rs]: T1t[k][r] = T1[r0 + r][k]
-  float* V = T1t + b * rs;                            // [a][vs]: V[k][c] = V_(k, c0 + c)
-  float* Bs = V + a * vs + ((a * vs) & 2);            // [b][bp], 16-byte aligned
-  float* As = Bs + (ly.stage_b ? b * bp + ((b * bp) & 2) : 0);   // [a][ap]
+  float* T1t = reinterpret_cast<float*>(rot_smem4);   // [b][rc]: T1t[k][r] = T1[r0 + r][k]
+  float* As = T1t + b * rc;                           // [a][al]: As[k][a0 + r] = A[r0 + r][k]
+  float* V = As + (kStaged || ly.stage_a ? a * al : 0);   // [a][bp]
+  float* Bs = V + a * bp + ((a * bp) & 2);            // [b][bp], 16-byte aligned
   pdl_launch_dependents();
-  if (kCluster) cluster_arrive();   // (waited for before the first store into another CTA)
-  if (ly.stage_a) stage_factor(As, ly.At, a, ap, tid);
-  if (ly.stage_b) stage_factor(Bs, ly.B, b, bp, tid);
+  if (kStaged)
+    stage_factor(As, ly.At, a, a, al, tid);
+  else if (ly.stage_a)
+    stage_factor(As, ly.At + r0, a, nr, al, tid);
+  if (kStaged || ly.stage_b) stage_factor(Bs, ly.B, b, b, bp, tid);
   cp_async_commit();
-  // V's place first holds what does not depend on the input: the index each entry is gathered
-  // from (analysis) or its sign (synthesis).  A thread takes columns vc, vc + dc, ... (one, when
-  // they are at most the threads) and rows vk, vk + dk, ...
-  const bool narrow = nc <= kRotThreads;
-  const int dk = narrow ? kRotThreads / max(nc, 1) : 1, dc = narrow ? max(nc, 1) : kRotThreads;
-  const int vc = tid % dc, vk = narrow ? (tid < dk * dc ? tid / dc : a) : 0;
-  for (int c = vc; c < nc; c += dc) {
-#pragma unroll 4
-    for (int k = vk; k < a; k += dk) {
-      const int e = k * b + c0 + c;
-      V[k * vs + c] = kSynth ? ly.signs[e] : __int_as_float(ly.iperm[e]);
-    }
-  }
   pdl_wait();
   const int64_t tok = static_cast<int64_t>(blockIdx.y) * a * b;
-  const __nv_bfloat16* in = ly.in + tok;
-  for (int c = vc; c < nc; c += dc) {
-#pragma unroll 8
-    for (int k = vk; k < a; k += dk) {              // (this thread's own entries)
-      const float h = V[k * vs + c];
-      V[k * vs + c] = kSynth ? h * __bfloat162float(in[k * b + c0 + c])
-                             : __bfloat162float(in[__float_as_int(h)]);
+  // four entries of the token at a time (a b is a multiple of 8)
+  const uint2* in = reinterpret_cast<const uint2*>(ly.in + tok);
+  const float4* side = reinterpret_cast<const float4*>(kSynth ? ly.signs
+                                                              : reinterpret_cast<const float*>(ly.perm));
+#pragma unroll 4
+  for (int i = tid; i < a * b / 4; i += kRotThreads) {
+    const uint2 w = in[i];
+    const float4 h = side[i];
+    const float x[4] = {__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                        __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u)};
+    const float sv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = kSynth ? 4 * i + j : __float_as_int(sv[j]);
+      V[bp == b ? e : e + e / b] = kSynth ? sv[j] * x[j] : x[j];
     }
   }
   cp_async_wait_all();
   __syncthreads();
-  if (kCluster) cluster_wait();
-  // T1 = A V, columns c0 .. c0 + nc - 1, to the owners of the rows
-  const int cp = (nc + 1) / 2;
-  for (int t = tid; t < (a + 3) / 4 * cp; t += kRotThreads) {
-    const int r = t / cp * 4, c = t % cp * 2;
+  // T1 = A V, then Y = T1 B, rows r0 .. r0 + nr - 1; task: 4 rows x 2 columns
+  const int pairs = (b + 1) / 2, tasks = (nr + 3) / 4 * pairs;
+  for (int t = tid; t < tasks; t += kRotThreads) {
+    const int r = t / pairs * 4, c = t % pairs * 2;
     float acc[4][2] = {};
-    const auto cols = [&](int k) { return *reinterpret_cast<const float2*>(V + k * vs + c); };
-    if (ly.stage_a) {
-      rot_product<8>(
-          acc, a, [&](int k) { return *reinterpret_cast<const float4*>(As + k * ap + r); }, cols);
+    const auto cols = [&](int k) { return *reinterpret_cast<const float2*>(V + k * bp + c); };
+    if (kStaged || ly.stage_a) {
+      rot_product<4>(acc, a, [&](int k) {
+        return *reinterpret_cast<const float4*>(As + k * al + a0 + r);
+      }, cols);
     } else {
-      rot_product<2>(acc, a, [&](int k) {
-        const float* p = ly.At + static_cast<int64_t>(k) * a + r;
-        return make_float4(p[0], r + 1 < a ? p[1] : 0.f, r + 2 < a ? p[2] : 0.f,
-                           r + 3 < a ? p[3] : 0.f);
+      rot_product<8>(acc, a, [&](int k) {
+        const float* p = ly.At + static_cast<int64_t>(k) * a + r0 + r;
+        return make_float4(p[0], r + 1 < nr ? p[1] : 0.f, r + 2 < nr ? p[2] : 0.f,
+                           r + 3 < nr ? p[3] : 0.f);
       }, cols);
     }
-    if (kCluster) {
-      int owner = r / rc, rl = r - owner * rc;   // the CTA that takes this row, its place there
 #pragma unroll
-      for (int j = 0; j < 4; ++j, ++rl) {
-        if (rl == rc) ++owner, rl = 0;
-        if (r + j >= a) continue;
-        const uint32_t dst = mapa(smem_u32(T1t + (c0 + c) * rs + rl), static_cast<uint32_t>(owner));
-        st_cluster_f32(dst, acc[j][0]);
-        if (c + 1 < nc) st_cluster_f32(dst + 4 * rs, acc[j][1]);
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 2; ++q)                // (rows past a fall into the padding)
-        if (c + q < nc)
-          *reinterpret_cast<float4*>(T1t + (c + q) * rs + r) =
-              make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
-    }
+    for (int q = 0; q < 2; ++q)                  // (rows past nr fall into the padding)
+      if (c + q < b)
+        *reinterpret_cast<float4*>(T1t + (c + q) * rc + r) =
+            make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
   }
-  if (kCluster)
-    cluster_sync();
-  else
-    __syncthreads();
-  // Y = T1 B, rows r0 .. r0 + nr - 1
+  __syncthreads();
   __nv_bfloat16* out = ly.out + tok;
-  const int bp2 = (b + 1) / 2;
-  for (int t = tid; t < (nr + 3) / 4 * bp2; t += kRotThreads) {
-    const int r = t / bp2 * 4, c = t % bp2 * 2;
+  for (int t = tid; t < tasks; t += kRotThreads) {
+    const int r = t / pairs * 4, c = t % pairs * 2;
     float acc[4][2] = {};
     // where the results go (or their signs), requested before the product
     int dest[4][2];
@@ -223,12 +202,16 @@ __global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_consta
         const int o = (r0 + min(r + j, nr - 1)) * b + min(c + q, b - 1);
         dest[j][q] = kSynth ? ly.iperm[o] : __float_as_int(ly.signs[o]);
       }
-    const auto rows = [&](int k) { return *reinterpret_cast<const float4*>(T1t + k * rs + r); };
-    if (ly.stage_b) {
-      rot_product<8>(acc, b, rows,
+    const auto rows = [&](int k) { return *reinterpret_cast<const float4*>(T1t + k * rc + r); };
+    if (kStaged || ly.stage_b) {
+      rot_product<4>(acc, b, rows,
                      [&](int k) { return *reinterpret_cast<const float2*>(Bs + k * bp + c); });
+    } else if (bp == b) {                        // (many loads in flight for their latency)
+      rot_product<32>(acc, b, rows, [&](int k) {
+        return __ldg(reinterpret_cast<const float2*>(ly.B + static_cast<int64_t>(k) * b + c));
+      });
     } else {
-      rot_product<2>(acc, b, rows, [&](int k) {
+      rot_product<8>(acc, b, rows, [&](int k) {
         const float* p = ly.B + static_cast<int64_t>(k) * b + c;
         return make_float2(p[0], c + 1 < b ? p[1] : 0.f);
       });
@@ -411,25 +394,68 @@ bool frame_fits(const fq_frame& f) {
                                                     static_cast<int64_t>(kMaxSmem);
 }
 
-// CTAs per token: enough entries for each to outweigh the cluster barriers.  Measured on two layers
-// of 16 tokens (us, C = 1, 2, 4, 8): 512 x 512 20.0, 20.7, 21.3, 21.5; 1024 x 1024 25.2, 27.0, 26.8,
-// 26.6; 2048 x 2048 53.4, 35.0, 30.4, 31.0; 768 to 3072 51.6, 38.4, 33.8, 30.8.
-int rot_cluster(int d) { return d >= 3072 ? 8 : (d > 1024 ? 4 : 1); }
+// A layer's split over C CTAs per token, and its shared memory with both factors staged whole, or
+// (`whole` false) with what of them fits; above kMaxSmem when it does not fit.
+size_t rot_layout(RotLayer& L, int C, bool whole) {
+  const int64_t a = L.a, b = L.b;
+  L.bp = static_cast<int>(round_up(b, 2));
+  L.rc = static_cast<int>(round_up(ceil_div(a, C), 4));
+  const int64_t base = 4 * (b * L.rc + round_up(a * L.bp, 4)), bs = 4 * round_up(b * L.bp, 4);
+  if (whole) return static_cast<size_t>(base + 4 * a * round_up(a, 4) + bs);
+  const int64_t max = static_cast<int64_t>(kMaxSmem), as = 4 * a * L.rc;
+  L.stage_a = base + as <= max;
+  L.stage_b = base + (L.stage_a ? as : 0) + bs <= max;
+  return static_cast<size_t>(base + (L.stage_a ? as : 0) + (L.stage_b ? bs : 0));
+}
 
-// The layer's split over C CTAs and its staging; returns its shared memory.
-size_t rot_layout(RotLayer& L, int C) {
-  L.ap = static_cast<int>(round_up(L.a, 4));
-  L.bp = static_cast<int>(round_up(L.b, 2));
-  L.bc = static_cast<int>(ceil_div(L.b, C));
-  L.vs = static_cast<int>(round_up(L.bc, 2));
-  L.rc = static_cast<int>(ceil_div(L.a, C));
-  L.rs = static_cast<int>(round_up(L.rc, 4));
-  const size_t base = 4 * (static_cast<size_t>(L.b) * L.rs + round_up(static_cast<int64_t>(L.a) * L.vs, 4));
-  const size_t as = 4 * static_cast<size_t>(L.a) * L.ap;
-  const size_t bs = 4 * static_cast<size_t>(round_up(static_cast<int64_t>(L.b) * L.bp, 4));
-  L.stage_a = base + as <= kMaxSmem;
-  L.stage_b = base + (L.stage_a ? as : 0) + bs <= kMaxSmem;
-  return base + (L.stage_a ? as : 0) + (L.stage_b ? bs : 0);
+// The CTAs per token of a launch over `tokens` tokens (of all layers), the layers' layouts, and their
+// shared memory.  More CTAs shorten a token's products but read it as often, so a token with little
+// work takes fewer, and C is halved while the launch is more than the CTAs that fit at once (4/3 of
+// them at C = 4), unless a factor would lose its place in shared memory.  Measured with C = 1, 2, 4, 8
+// (us per call): 512 x 512 at 16 tokens 18.4, 18.3, 18.1, 18.9; 1024 x 1024 at 8 tokens 20.2, 20.1, 19.8,
+// 19.9; 2048 x 2048 at one token 23.2, 21.9, 21.1, 21.4, at 16 tokens 28.8, 30.0, 25.6, 24.0; three
+// 4096 x 4096 at 64 tokens 102, 91, 81, 86; 4096 to 11008 at 32 tokens 91, 71, 61, 63, three at 64 tokens
+// 208, 196, 202, 227.  With C = 4, 8, 16: 4096 x 4096 at one token 26.9, 27.5, 27.4, at 16 tokens 37.2,
+// 31.1, 29.5; 11008 x 11008 at 4 tokens 81.4, 71.9, 70.6, at 16 tokens 82.1, 74.0, 86.0.  With C = 8, 16,
+// 32: 28672 to 4096 at one token 124.6, 104.0, 102.7.
+constexpr int kRotPerSm = 4;      // CTAs that an SM's registers hold
+
+struct RotPlan {
+  int C;
+  bool staged;              // both factors of every layer, whole
+  int kept;                 // factors in shared memory
+  size_t smem;
+};
+
+RotPlan rot_plan(RotLayer* L, int n, int64_t tokens, int sms) {
+  int64_t work = 0;         // multiply-adds per token: 43 k for 24 x 32, 66 k for 32 x 32, 524 k for 64 x 64
+  int a = 0;
+  for (int l = 0; l < n; ++l) {
+    const int64_t w = static_cast<int64_t>(L[l].a) * L[l].b * (L[l].a + L[l].b);
+    if (w > work) work = w, a = L[l].a;
+  }
+  auto with = [&](int C) {
+    RotPlan p{C, true, 2 * n, 0};
+    for (int l = 0; l < n; ++l) p.smem = std::max(p.smem, rot_layout(L[l], C, true));
+    if (p.smem <= kMaxSmem) return p;
+    p = RotPlan{C, false, 0, 0};
+    for (int l = 0; l < n; ++l) {
+      p.smem = std::max(p.smem, rot_layout(L[l], C, false));
+      p.kept += L[l].stage_a + L[l].stage_b;
+    }
+    return p;
+  };
+  int C = work <= 50000 ? 1 : (work <= 70000 ? 4 : (work <= 250000 ? (tokens <= 2 ? 4 : 8) : 16));
+  while (C > 1 && work / C > 600000 && 8 * C <= a) C *= 2;
+  RotPlan p = with(C);
+  while (p.C > 2) {
+    const int64_t resident = sms * std::min<int64_t>(kRotPerSm, 228 * 1024 / (p.smem + 1024));
+    const RotPlan half = with(p.C / 2);
+    const int64_t most = p.C == 4 ? resident * 4 / 3 : resident;
+    if (tokens * p.C <= most || half.smem > kMaxSmem || half.kept < p.kept) break;
+    p = half;
+  }
+  return with(p.C);
 }
 
 cudaError_t set_smem_attributes() {
@@ -458,10 +484,7 @@ template <bool kSynth>
 cudaError_t rotate_batch(int n, const fq_frame* const* f, const void* const* in,
                          void* const* out, int M, cudaStream_t s) {
   RotBatch rb{};
-  int nb = 0, C = 1;
-  size_t smem = 0;
-  for (int l = 0; l < n; ++l)
-    if (f[l]->a != 0 && in[l]) C = std::max(C, rot_cluster(f[l]->d));
+  int nb = 0;
   for (int l = 0; l < n; ++l) {
     if (f[l]->a == 0 || !in[l]) continue;
     const fq_frame& F = *f[l];
@@ -472,27 +495,28 @@ cudaError_t rotate_batch(int n, const fq_frame* const* f, const void* const* in,
     L.b = F.b;
     L.At = kSynth ? F.QaT : F.Qa;
     L.B = kSynth ? F.QbT : F.Qb;
+    L.perm = F.perm;
     L.iperm = F.iperm;
     L.signs = F.signs;
-    smem = std::max(smem, rot_layout(L, C));
   }
   if (nb == 0) return cudaSuccess;
-  if (smem > kMaxSmem) return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const RotPlan p = rot_plan(rb.L, nb, static_cast<int64_t>(M) * nb, sms);
+  if (p.smem > kMaxSmem) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(C), static_cast<unsigned>(M), static_cast<unsigned>(nb));
+  cfg.gridDim = dim3(static_cast<unsigned>(p.C), static_cast<unsigned>(M), static_cast<unsigned>(nb));
   cfg.blockDim = dim3(kRotThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = p.smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = static_cast<unsigned>(C);
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = C > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, C > 1 ? rotate_kernel<kSynth, true> : rotate_kernel<kSynth, false>,
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, p.staged ? rotate_kernel<kSynth, true> : rotate_kernel<kSynth, false>,
                             rb);
 }
 
