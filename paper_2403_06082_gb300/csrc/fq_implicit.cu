@@ -423,7 +423,7 @@ constexpr int kRotPerSm = 4;      // CTAs that an SM's registers hold
 struct RotPlan {
   int C;
   bool staged;              // both factors of every layer, whole
-  int kept;                 // factors in shared memory
+  int kept, kept_a;         // factors in shared memory, and first factors (their CTAs' columns)
   size_t smem;
 };
 
@@ -435,19 +435,22 @@ RotPlan rot_plan(RotLayer* L, int n, int64_t tokens, int sms) {
     if (w > work) work = w, a = L[l].a;
   }
   auto with = [&](int C) {
-    RotPlan p{C, true, 2 * n, 0};
+    RotPlan p{C, true, 2 * n, n, 0};
     for (int l = 0; l < n; ++l) p.smem = std::max(p.smem, rot_layout(L[l], C, true));
     if (p.smem <= kMaxSmem) return p;
-    p = RotPlan{C, false, 0, 0};
+    p = RotPlan{C, false, 0, 0, 0};
     for (int l = 0; l < n; ++l) {
       p.smem = std::max(p.smem, rot_layout(L[l], C, false));
       p.kept += L[l].stage_a + L[l].stage_b;
+      p.kept_a += L[l].stage_a;
     }
     return p;
   };
   int C = work <= 50000 ? 1 : (work <= 70000 ? 4 : (work <= 250000 ? (tokens <= 2 ? 4 : 8) : 16));
   while (C > 1 && work / C > 600000 && 8 * C <= a) C *= 2;
   RotPlan p = with(C);
+  // (a first factor many times as long as the second: until a CTA's columns of it fit)
+  while (p.kept_a < n && 8 * C <= a && tokens * 2 * C <= 4 * sms) p = with(C *= 2);
   while (p.C > 2) {
     const int64_t resident = sms * std::min<int64_t>(kRotPerSm, 228 * 1024 / (p.smem + 1024));
     const RotPlan half = with(p.C / 2);
