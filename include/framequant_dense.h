@@ -21,11 +21,10 @@
 extern "C" {
 #endif
 
-/* Workspace bytes of fq_reconstruct_weight; 0 for invalid sizes.  It holds the tensor-core
- * chain's workspace for M = d_in tokens (z and u of the d_in unit vectors) and room for a
- * d_in x d_out matrix that is not used now: about 108 MB for a 4096 x 4096 layer at r = 1.1, 227 MB for
- * 11008 x 4096, 460 MB for 4096 x 11008, 432 MB for 8192 x 8192, 1.14 GB for 28672 x 8192 and
- * 2.8 GB for 8192 x 28672. */
+/* Workspace bytes of fq_reconstruct_weight; 0 for invalid sizes.  It is that of the tensor-core
+ * chain for M = d_in tokens (fq_workspace_bytes above 64 tokens): about 75 MB for a
+ * 4096 x 4096 layer (d_out x d_in) at r = 1.1, 137 MB for 11008 x 4096, 370 MB for 4096 x 11008, 298 MB for
+ * 8192 x 8192, 0.67 GB for 28672 x 8192 and 2.4 GB for 8192 x 28672. */
 size_t fq_reconstruct_workspace_bytes(int d_in, int n_in, int n_out, int d_out);
 
 /* W_hat = T_out^T diag(gamma) C_hat T_in, bf16 d_out x d_in row-major: the FQ_BF16 forward of

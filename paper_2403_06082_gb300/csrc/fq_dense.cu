@@ -11,14 +11,6 @@
 namespace fq {
 namespace {
 
-// The tensor-core chain's workspace for M = d_in tokens, then room for a d_in x d_out matrix that
-// this version does not use: the size that callers allocate stays what it was.
-size_t rec_ws_bytes(int d_in, int n_in, int n_out, int d_out) {
-  return static_cast<size_t>(round_up(
-             static_cast<int64_t>(tc_workspace_bytes(d_in, d_in, n_in, n_out, d_out, 0)), 256)) +
-         static_cast<size_t>(round_up(static_cast<int64_t>(d_in) * d_out * 2, 256));
-}
-
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -30,7 +22,7 @@ extern "C" {
 
 size_t fq_reconstruct_workspace_bytes(int d_in, int n_in, int n_out, int d_out) {
   if (d_in <= 0 || n_in <= 0 || n_out <= 0 || d_out <= 0) return 0;
-  return rec_ws_bytes(d_in, n_in, n_out, d_out);
+  return tc_workspace_bytes(d_in, d_in, n_in, n_out, d_out, 0);
 }
 
 fq_status fq_reconstruct_weight(const void* T_in, const fq_packed* C, const void* T_out_t,

@@ -1578,17 +1578,13 @@ cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const Devi
 // reconstructed weight as its A operand.
 WsLayout dense_ws_layout(int M, int d_out) {
   WsLayout L{};
-  size_t off = kWsHeader;
-  L.zsum = off;
-  off += round_up(ceil_div(d_out, kBM) * M * 4, 256);
   const int BN = pick_bn(M);
   const int64_t tiles = ceil_div(d_out, kBM) * ceil_div(M, BN);
   int64_t slots = 0;
   if (tiles < kMaxSplitSms) slots = std::min<int64_t>(kMaxSplitSms, tiles * kMaxSplits);
-  L.part = off;
+  L.part = kWsHeader;
   L.part_floats = slots * BN * kBM;
-  off += static_cast<size_t>(slots) * BN * kBM * 4;
-  L.total = off;
+  L.total = L.part + static_cast<size_t>(slots) * BN * kBM * 4;
   return L;
 }
 
