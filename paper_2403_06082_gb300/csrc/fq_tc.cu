@@ -1169,7 +1169,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairLayout<PHASE, BN
 // a multiple of 16).  With one block per token, 4-byte loads and 2-byte stores it took 69 us for 12608
 // tokens of 848 coefficients (0.9 TB/s); the ViT fc1 layer went from 327 to 299 us with this.
 constexpr int kQuantThreads = 256;
-constexpr int kWarpTokenMaxN = 2048;
 
 template <int kPer>
 __global__ void __launch_bounds__(kQuantThreads) ff_round_kernel(
@@ -1563,9 +1562,12 @@ cudaError_t launch_phase(const PhasePlan& pl, const PhaseArgs& a, cudaStream_t s
 
 cudaError_t launch_round(const PhaseArgs& an, int n_in, int act_bits, const DeviceInfo& d,
                          float* delta, __nv_bfloat16* zq, float* zsum, cudaStream_t s) {
-  // one warp per token when a token has little work for a block and there are tokens for every
-  // SM's warps; one block per token otherwise
-  const bool warps = n_in <= kWarpTokenMaxN && an.M >= 8 * d.sms;
+  // A warp per token once there are tokens for most of the SMs' warps, sooner where a token has work
+  // for few of a block's threads; a block per token otherwise.  Whole layers, us with a block and
+  // with a warp per token: n_in = 288 at 608 tokens 19.5, 20.3, at 1216 22.5, 20.5; 848 at 2432 33.0, 34.9,
+  // at 4864 47.6, 46.7, at 12608 85.7, 79.4; 2256 at 2432 90.2, 92.2, at 4864 130.6, 125.3; 3392 at 4864
+  // 128.6, 134.7, at 12608 348, 335; 4512 at 4864 357, 361, at 12608 1071, 1054.
+  const bool warps = an.M >= (n_in <= 512 ? 8 : (n_in <= 2304 ? 32 : 64)) * d.sms;
   const int blocks = static_cast<int>(ceil_div(an.M, warps ? kQuantThreads / 32 : 1));
   const ChainedLaunch l(std::min(blocks, 8 * d.sms), kQuantThreads, 0, s);
   const float L = static_cast<float>((1 << (act_bits - 1)) - 1);
