@@ -350,8 +350,8 @@ size_t fq_gptq_workspace_bytes(int n_out, int n_in);
  *     optimal-brain-surgeon update of the method GPTQ, which Algorithm 1 cites).
  *   codes  device uint8 n_out x n_in;  scale, zero  device fp16 bits [n_out];  gamma fp32 or NULL
  *   ws     device workspace of fq_gptq_workspace_bytes(n_out, n_in) bytes, 256-byte aligned
- * Synchronizes `stream` before returning.  n_in up to 25600 (the triangular inverse keeps one
- * column in shared memory).
+ * Synchronizes `stream` before returning.  n_in up to 25600 (a limit of this call's contract; the
+ * workspace for it holds 10.5 GB of fp64 factors).
  * Errors: FQ_ERR_INVALID_ARG, FQ_ERR_ALIGNMENT, FQ_ERR_WORKSPACE, FQ_ERR_UNSUPPORTED (n_in above
  * 25600), FQ_ERR_DEVICE_CHECK (the damped H is not positive definite), FQ_ERR_CUDA. */
 fq_status fq_quantize_gptq(const double* C, int n_out, int n_in, const double* H, double damp,

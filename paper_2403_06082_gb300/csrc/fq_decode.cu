@@ -122,7 +122,7 @@ __host__ __device__ constexpr int issuer_of(int warp, int ni) {
 // blocks of its later tasks after issuing its first task's loads.  When the code blocks and
 // T_out^T fit together, it also prefetches the T_out^T tiles of its synthesis tasks, once it
 // reaches its first code-product task: by then its analysis loads are out, and the code
-// product, bounded by the decode, leaves HBM mostly idle (prefetching them earlier competes with
+// product, which streams little, leaves HBM mostly idle (prefetching them earlier competes with
 // the analysis stream; prefetching part of a larger layer's T_out^T measured no faster).
 constexpr int64_t kL2PrefetchBudget = 64ll << 20;
 
@@ -1291,7 +1291,11 @@ struct Plan {
 
 // Cluster size and task lists for a launch's blocks, cached.  Cluster size: the busiest
 // cluster's K blocks over the blocks, with a fixed cost per task (pipeline fill and drain,
-// reduction) and code blocks weighted by their smaller bytes.
+// reduction) and code blocks weighted by their smaller bytes.  The two weights, 4.0 and 0.35, date from
+// an earlier round loop.  Of S = 1, 2, 4, 8 forced at 16 tokens the choice is the fastest or within 4% for
+// most sizes (2048 x 2048 25.6, 20.4, 16.6, 22.4 us, 4096 x 4096 47.8, 31.6, 25.1, 35.6: S = 4 taken), but
+// not for 256 x 256 (10.1, 12.3, 11.7, 12.0: 8 taken), 1024 x 1024 (17.1, 16.1, 13.8, 14.7: 8), 5120 x 5120
+// (58.7, 37.8, 35.7, 42.3: 8) and 8192 x 8192 (97.6, 71.7, 64.9, 76.7: 2).
 template <int BN>
 const Plan* plan_for(int dev, int sms, int budget, const std::vector<Block>& blocks) {
   static std::mutex mu;
