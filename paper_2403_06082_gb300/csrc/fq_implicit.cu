@@ -61,6 +61,7 @@ struct RotLayer {
   int bp;                 // row stride of V and of the staged B: b rounded up to 2
   int rc;                 // rows of Y per CTA, a multiple of 4, and T1t's row stride
   int stage_a, stage_b;   // (where not both factors of every layer are staged whole)
+  int wide;               // At, B, perm and signs are 16-byte aligned (as fq_frame_implicit lays them)
   const float* At;        // A^T, a x a row-major: At[i][r] = A[r][i]
   const float* B;         // b x b row-major
   const int32_t* perm;
@@ -86,11 +87,11 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 // `cols` columns of an n x n factor (row-major) into shared memory with row stride np, asynchronously:
 // one copy when they are whole rows without padding, else a warp per row, in the widest pieces that
-// the alignment allows (n, cols and the first column are multiples of them).  Nothing is written past
-// the last column (such entries only reach results that are dropped).
+// the alignment allows (n, cols and the first column are multiples of them; `wide`: src's base is 16-byte
+// aligned).  Nothing is written past the last column (such entries only reach results that are dropped).
 __device__ __forceinline__ void stage_factor(float* dst, const float* __restrict__ src, int n,
-                                             int cols, int np, int tid) {
-  if (n % 4 == 0 && cols == n) {       // np == n
+                                             int cols, int np, bool wide, int tid) {
+  if (wide && n % 4 == 0 && cols == n) {       // np == n
     for (int i = tid; i < n * n / 4; i += kRotThreads) cp_async<16>(dst + 4 * i, src + 4 * i);
     return;
   }
@@ -98,7 +99,7 @@ __device__ __forceinline__ void stage_factor(float* dst, const float* __restrict
   for (int r = tid >> 5; r < n; r += kRotThreads / 32) {
     const float* from = src + static_cast<int64_t>(r) * n;
     float* to = dst + r * np;
-    if (n % 2 == 0)
+    if (wide && n % 2 == 0)
       for (int i = 2 * lane; i < cols; i += 64) cp_async<8>(to + i, from + i);
     else
       for (int i = lane; i < cols; i += 32) cp_async<4>(to + i, from + i);
@@ -123,14 +124,15 @@ __device__ __forceinline__ void rot_product(float (&acc)[4][2], int n, Rows rows
   }
 }
 
-// kStaged: both factors of every layer of the launch are in shared memory, all of A.  Otherwise each
-// may or may not be, and of A only the CTA's columns of A^T.
+// kStaged: both factors of every layer of the launch are in shared memory, all of A, and their arrays
+// are wide.  Otherwise each may or may not be, and of A only the CTA's columns of A^T.
 template <bool kSynth, bool kStaged>
 __global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_constant__ RotBatch rb) {
   const RotLayer& ly = rb.L[blockIdx.z];
   const int a = ly.a, b = ly.b, bp = ly.bp, rc = ly.rc;
   const int tid = threadIdx.x;
   const int r0 = min(a, static_cast<int>(blockIdx.x) * rc), nr = min(rc, a - r0);   // its rows
+  const bool wide = kStaged || ly.wide;
   const int al = kStaged ? (a + 3) & ~3 : rc, a0 = kStaged ? r0 : 0;   // As's row stride, and r0 in it
   extern __shared__ float4 rot_smem4[];
   float* T1t = reinterpret_cast<float*>(rot_smem4);   // [b][rc]: T1t[k][r] = T1[r0 + r][k]
@@ -139,21 +141,21 @@ __global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_consta
   float* Bs = V + a * bp + ((a * bp) & 2);            // [b][bp], 16-byte aligned
   pdl_launch_dependents();
   if (kStaged)
-    stage_factor(As, ly.At, a, a, al, tid);
+    stage_factor(As, ly.At, a, a, al, wide, tid);
   else if (ly.stage_a)
-    stage_factor(As, ly.At + r0, a, nr, al, tid);
-  if (kStaged || ly.stage_b) stage_factor(Bs, ly.B, b, b, bp, tid);
+    stage_factor(As, ly.At + r0, a, nr, al, wide, tid);
+  if (kStaged || ly.stage_b) stage_factor(Bs, ly.B, b, b, bp, wide, tid);
   cp_async_commit();
   pdl_wait();
   const int64_t tok = static_cast<int64_t>(blockIdx.y) * a * b;
   // four entries of the token at a time (a b is a multiple of 8)
   const uint2* in = reinterpret_cast<const uint2*>(ly.in + tok);
-  const float4* side = reinterpret_cast<const float4*>(kSynth ? ly.signs
-                                                              : reinterpret_cast<const float*>(ly.perm));
+  const float* side = kSynth ? ly.signs : reinterpret_cast<const float*>(ly.perm);
 #pragma unroll 4
   for (int i = tid; i < a * b / 4; i += kRotThreads) {
     const uint2 w = in[i];
-    const float4 h = side[i];
+    const float4 h = wide ? reinterpret_cast<const float4*>(side)[i]
+                          : make_float4(side[4 * i], side[4 * i + 1], side[4 * i + 2], side[4 * i + 3]);
     const float x[4] = {__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
                         __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u)};
     const float sv[4] = {h.x, h.y, h.z, h.w};
@@ -206,7 +208,7 @@ __global__ void __launch_bounds__(kRotThreads) rotate_kernel(const __grid_consta
     if (kStaged || ly.stage_b) {
       rot_product<4>(acc, b, rows,
                      [&](int k) { return *reinterpret_cast<const float2*>(Bs + k * bp + c); });
-    } else if (bp == b) {                        // (many loads in flight for their latency)
+    } else if (wide && bp == b) {                // (many loads in flight for their latency)
       rot_product<32>(acc, b, rows, [&](int k) {
         return __ldg(reinterpret_cast<const float2*>(ly.B + static_cast<int64_t>(k) * b + c));
       });
@@ -422,7 +424,7 @@ constexpr int kRotPerSm = 4;      // CTAs that an SM's registers hold
 
 struct RotPlan {
   int C;
-  bool staged;              // both factors of every layer, whole
+  bool staged;              // both factors of every layer, whole, of wide arrays
   int kept, kept_a;         // factors in shared memory, and first factors (their CTAs' columns)
   size_t smem;
 };
@@ -430,14 +432,16 @@ struct RotPlan {
 RotPlan rot_plan(RotLayer* L, int n, int64_t tokens, int sms) {
   int64_t work = 0;         // multiply-adds per token: 43 k for 24 x 32, 66 k for 32 x 32, 524 k for 64 x 64
   int a = 0;
+  bool wide = true;
   for (int l = 0; l < n; ++l) {
+    wide = wide && L[l].wide;
     const int64_t w = static_cast<int64_t>(L[l].a) * L[l].b * (L[l].a + L[l].b);
     if (w > work) work = w, a = L[l].a;
   }
   auto with = [&](int C) {
     RotPlan p{C, true, 2 * n, n, 0};
     for (int l = 0; l < n; ++l) p.smem = std::max(p.smem, rot_layout(L[l], C, true));
-    if (p.smem <= kMaxSmem) return p;
+    if (wide && p.smem <= kMaxSmem) return p;
     p = RotPlan{C, false, 0, 0, 0};
     for (int l = 0; l < n; ++l) {
       p.smem = std::max(p.smem, rot_layout(L[l], C, false));
@@ -501,6 +505,7 @@ cudaError_t rotate_batch(int n, const fq_frame* const* f, const void* const* in,
     L.perm = F.perm;
     L.iperm = F.iperm;
     L.signs = F.signs;
+    L.wide = aligned16(L.At) && aligned16(L.B) && aligned16(L.perm) && aligned16(L.signs);
   }
   if (nb == 0) return cudaSuccess;
   int dev = 0, sms = 0;

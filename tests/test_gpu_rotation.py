@@ -8,6 +8,8 @@ The products are chains of a and b fused multiply-adds in fp32, so what is round
 gamma_k = k u / (1 - k u) and u = 2^-24, within
     e = ((1 + gamma_a) (1 + gamma_b) (1 + u) - 1) |A| |V| |B|
 of the 64-bit value v, and rounding is monotonic: bf16(v - e) <= y <= bf16(v + e)."""
+import copy
+
 import numpy as np
 import pytest
 
@@ -124,3 +126,28 @@ def test_layers_that_share_tokens_and_frame(M):
     for shared, own in zip(run(False), run(True)):
         assert torch.isfinite(shared).all()
         assert torch.equal(shared, own)
+
+
+@pytest.mark.parametrize("M", [1, 17])
+@pytest.mark.parametrize("a,b", [(24, 32), (33, 80), (16, 43), (36, 36), (40, 34), (128, 224)])
+def test_arrays_off_16_byte_boundaries(a, b, M):
+    """A frame's factors, permutation and signs may lie at any 4-byte boundary: the same sums in the
+    same order, so bitwise the results of the frame as it was built."""
+    d = a * b
+    F, FN = fq.fq_frame_implicit(1, d, d, _rotation(a, b, 0)), fq.fq_frame_implicit(1, N, N, None)
+    moved, keep = copy.copy(F), []
+    moved.c = type(F.c).from_buffer_copy(F.c)
+    sizes = dict(Qa=a * a, QaT=a * a, Qb=b * b, QbT=b * b, perm=d, iperm=d, signs=d)
+    for name, n in sizes.items():
+        at = getattr(F.c, name) - F.buf.data_ptr()
+        other = torch.zeros(4 * n + 16, dtype=torch.uint8, device="cuda")
+        other[4:4 + 4 * n] = F.buf[at:at + 4 * n]
+        setattr(moved.c, name, other.data_ptr() + 4)
+        keep.append(other)
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn(M, d, generator=g, device="cuda").to(BF16)
+    C = _packed(N, d, g)
+    assert all(torch.equal(p, q) for p, q in zip(_run(x, F, C, FN)[:2], _run(x, moved, C, FN)[:2]))
+    x = torch.randn(M, N, generator=g, device="cuda").to(BF16)
+    C = _packed(d, N, g)
+    assert torch.equal(_run(x, FN, C, F)[0], _run(x, FN, C, moved)[0])
