@@ -56,8 +56,9 @@ extern "C" fq_status fq_linear_forward_static(const void* x, int M, int d_in, co
   void* scratch = nullptr;
   if (fq::scratch_for_current_device(&scratch) != cudaSuccess) return FQ_ERR_CUDA;
   // Nothing left behind by the previous call needs clearing here: the status word at the head
-  // of the scratch is zeroed by the forward itself before its kernels report into it, and z, u
-  // and the sums of z are written before they are read within one call.
+  // of the scratch is zeroed by the forward itself before its kernels report into it, a completed
+  // call leaves the header's flags and counters valid for one of any sizes, and z, u and the sums
+  // of z are written before they are read within one call.
   return fq_linear_forward(x, M, d_in, T_in, C, T_out_t, d_out, gamma, y, scratch,
                            fq::kStaticScratchBytes, mode, stream);
 }
